@@ -1,0 +1,155 @@
+// fr_fixed.cuh -- block fixed point for the linear operators of the FP64 form.
+//
+// GB300 issues 2 FP64 multiply-adds per clock and SM against 128 32-bit operations, so the FP64
+// pipe bounds the element kernel while the integer pipes idle.  The linear parts of the method (the
+// folded derivative, the correction terms, the traces) are contractions with a fixed small matrix;
+// they are computed here on integers, exactly up to one rounding of the operands at 2^-59 of the
+// element's largest value in the variable group and one of the sum at 2^-58 of the largest
+// possible sum, against 2^-53 per operation of a chain of FP64 multiply-adds.
+//
+// A value x of an element is the 60-bit integer v = trunc(x 2^(1081 - E)), E the biased exponent of
+// the largest magnitude of its group (density, momenta, energy) in the element, so |v| < 2^59.
+// An operator entry c is the integer C = round(c 2^k), k the largest exponent at which the sum of
+// |C| over the terms of one result stays below 2^61.  Both are held in two limbs,
+//   v = vh 2^31 + vl, vh, vl of v's sign, |vl| < 2^31;   C = ch 2^31 + cl, |cl| <= 2^30,
+// and a result is H = sum vh ch + (sum (vh cl + vl ch) + 2^30) >> 31: three 32x32+64 multiply-adds
+// a term (the product vl cl lies below 2^-58 of the result's range).  Bounds: |sum vh ch| < 2^28 2^30
+// and |sum (vh cl + vl ch)| < 2^28 2^30 n + 2^31 2^30 < 2^63 for the n <= 21 terms of any result here.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <cmath>
+#include <cstring>
+
+namespace frg {
+
+constexpr int FX_GROUPS = 3;      // density, momenta, energy: one exponent each
+constexpr int FX_E_MIN = 64;      // smallest group exponent: results never fall below the normal range
+constexpr int FX_E_BAD = 2040;    // groups with infinities, NaN or values above 2^1017: results are NaN
+constexpr int FX_SUM_BITS = 61;   // log2 of the bound on the sum of |C|
+
+struct FxAcc {
+  long long h, m;
+};
+__host__ __device__ __forceinline__ void fx_mac(FxAcc& a, int2 v, int2 c) {
+  a.h += (long long)v.x * c.x;
+  a.m += (long long)v.x * c.y;
+  a.m += (long long)v.y * c.x;
+}
+__host__ __device__ __forceinline__ long long fx_sum(const FxAcc& a) {
+  return a.h + ((a.m + (1ll << 30)) >> 31);
+}
+
+__host__ __device__ __forceinline__ uint64_t fx_bits(double x) {
+#ifdef __CUDA_ARCH__
+  return uint64_t(__double_as_longlong(x));
+#else
+  uint64_t b;
+  memcpy(&b, &x, 8);
+  return b;
+#endif
+}
+__host__ __device__ __forceinline__ double fx_from_bits(uint64_t b) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)b);
+#else
+  double x;
+  memcpy(&x, &b, 8);
+  return x;
+#endif
+}
+// the high word of |x|: these order as the magnitudes, and >> 20 is the biased exponent
+__host__ __device__ __forceinline__ uint32_t fx_mag(double x) { return uint32_t(fx_bits(x) >> 32) & 0x7FFFFFFFu; }
+
+// limbs of trunc(x 2^(1081 - E)); |x| < 2^(E - 1022), E >= FX_E_MIN.  The significand with its
+// leading one at bit 62 is shifted down by E - e + 4 (e: x's biased exponent); zeros and subnormals
+// (e = 0) come out as 0.
+__host__ __device__ __forceinline__ int2 fx_limbs(double x, int E) {
+  const uint64_t b = fx_bits(x);
+  const int e = int(b >> 52) & 0x7FF;
+  const uint64_t m = ((b << 10) & 0x3FFFFFFFFFFFFFFFull) | 0x4000000000000000ull;
+  int s = E - e + 4;
+  s = s < 63 ? s : 63;
+  const uint64_t a = m >> s;
+  const int sg = int(uint32_t(b >> 32)) < 0 ? -1 : 1;
+  return make_int2(int(a >> 31) * sg, int(uint32_t(a) & 0x7FFFFFFFu) * sg);
+}
+
+// v 2^(e - 1023), rounded to nearest (ties away from zero); e: biased exponent of one unit of v,
+// at least 1 (and e + 62 below 2047); bad: NaN
+__host__ __device__ __forceinline__ double fx_double(long long v, int e, bool bad) {
+  const uint64_t s = uint64_t(v >> 63);
+  uint64_t a = (uint64_t(v) ^ s) - s;
+#ifdef __CUDA_ARCH__
+  const int z = __clzll((long long)a);
+#else
+  const int z = a ? __builtin_clzll(a) : 63;
+#endif
+  a <<= (z & 63);
+  uint64_t r = (a >> 11) + ((a >> 10) & 1);        // the leading one at bit 52 (a carry moves up)
+  r += uint64_t(uint32_t(e + 62 - z)) << 52;       // ... counts one in the exponent field
+  r = v == 0 ? 0 : (r | (s << 63));
+  if (bad) r = 0x7FF8000000000000ull;
+  return fx_from_bits(r);
+}
+
+// biased exponent of one unit of a result: values of group exponent E, entries scaled by 2^k
+__host__ __device__ __forceinline__ int fx_unit(int E, int k) { return E + 4 - k; }
+
+// one operator entry at scale 2^k
+inline int2 fx_coef(double c, int k) {
+  const long long C = llrint(ldexp(c, k));
+  const long long h = (C + (1ll << 30)) >> 31;
+  return make_int2(int(h), int(C - (h << 31)));
+}
+// largest k with sum 2^k <= 2^FX_SUM_BITS; at most 67, so that the smallest group exponent leaves a
+// unit (fx_unit) in the normal range
+inline int fx_scale(double sum) {
+  int e = 0;
+  frexp(sum, &e);  // sum < 2^e
+  const int k = FX_SUM_BITS - e;
+  return k < 67 ? k : 67;
+}
+
+// Largest magnitude (high words) per group over the N threads of one element, thread i of it, into
+// s[3] of the element (biased exponents; zeroed before a barrier by the caller, read after one).
+// All threads of the block call it; those without a point bring zeros and act = false.
+template <int N>
+__device__ __forceinline__ void fx_group_max(uint32_t w0, uint32_t w1, uint32_t w2, int i, bool act, uint32_t* s) {
+  const int lane = threadIdx.x & 31;
+  if constexpr (N % 32 == 0) {
+    // whole warps belong to one element
+    w0 = __reduce_max_sync(~0u, w0);
+    w1 = __reduce_max_sync(~0u, w1);
+    w2 = __reduce_max_sync(~0u, w2);
+    if (act && lane == 0) {
+      atomicMax(&s[0], w0 >> 20);
+      atomicMax(&s[1], w1 >> 20);
+      atomicMax(&s[2], w2 >> 20);
+    }
+  } else {
+    // segments of N lanes that may cross warps: each segment's first lane in a warp collects it;
+    // two groups to a register, exponents only
+    uint32_t p = (w0 >> 20) | ((w1 >> 20) << 16), q = w2 >> 20;
+#pragma unroll
+    for (int o = 1; o < 32 && o < N; o <<= 1) {
+      const uint32_t po = __shfl_down_sync(~0u, p, o), qo = __shfl_down_sync(~0u, q, o);
+      if (i + o < N && lane + o < 32) {
+        p = __vmaxu2(p, po);
+        q = q > qo ? q : qo;
+      }
+    }
+    if (act && (i == 0 || lane == 0)) {
+      atomicMax(&s[0], p & 0xFFFFu);
+      atomicMax(&s[1], p >> 16);
+      atomicMax(&s[2], q);
+    }
+  }
+}
+// the group of variable v of nv: 0 density, 1 momenta, 2 energy
+__host__ __device__ constexpr int fx_group(int v, int nv) { return v == 0 ? 0 : (v == nv - 1 ? 2 : 1); }
+__device__ __forceinline__ int fx_exp(uint32_t e) { return int(e) < FX_E_MIN ? FX_E_MIN : int(e); }
+
+}  // namespace frg

@@ -17,7 +17,6 @@ namespace frg {
 template <class T>
 struct OpsT {
   T Dt[NPMAX][NPMAX];
-  T D[NPMAX][NPMAX];  // plain derivative l_j'(x_i) (density-gradient indicator)
   // gLh, gRh: half the correction slopes g'_L, g'_R at the solution points, because the
   // interface kernel stores twice the common flux (exact scalings by 2 and 1/2)
   T gLh[NPMAX], gRh[NPMAX], lm[NPMAX], lp[NPMAX];
@@ -55,7 +54,6 @@ OpsT<T> make_ops_t(const DevOps& o) {
     r.lp[i] = host_conv(o.lp[i], tag);
     for (int j = 0; j < NPMAX; ++j) {
       r.Dt[i][j] = host_conv(o.Dt[i][j], tag);
-      r.D[i][j] = host_conv(o.D[i][j], tag);
       for (int h = 0; h < 2; ++h) {
         r.I[h][i][j] = host_conv(o.I[h][i][j], tag);
         r.P[h][i][j] = host_conv(o.P[h][i][j], tag);
@@ -398,7 +396,6 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value) k_s
   __shared__ T sfl[EPB * DIM * EU];
   __shared__ T sfc[EPB * EF];
   __shared__ double sh2[EPB];  // per element: c * (-2/h)
-  __shared__ unsigned long long sg2[EPB];  // per element: the indicator's max |D rho|^2 (as bits)
   const T* fcomm = static_cast<const T*>(A.fcomm);
   T* trace_out = static_cast<T*>(A.trace_out);
   const int tid = threadIdx.x;
@@ -422,7 +419,6 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value) k_s
   // c * (-2/h): 2^depth * (2/L) is exact, so this equals the rounded -2^(depth+1)/L times c
   if (tid < ne) {
     sh2[tid] = -A.c * (double(1ull << A.g.depth(A.keys[e0 + tid])) * A.twoL);
-    sg2[tid] = 0ull;
   }
   __syncthreads();
   const T gm1 = ops.gm1, ngmh = ops.ngmh;
@@ -491,15 +487,13 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value) k_s
       for (int v = 0; v < NV; ++v) R[v] = fma_t(ops.gLh[ia], Fm[v * NF], fma_t(ops.gRh[ia], Fp[v * NF], R[v]));
     }
     const double cs = sh2[le];
-    // u_s in FP64: the staged copy where it is exact (FP64 form), else the state in memory (an
-    // L2 hit: this block read it at its start); kept out of registers to hold the occupancy
+    // u_s in FP64 from memory (an L2 hit: this block read it at its start); kept out of registers
+    // to hold the occupancy
     double usr[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
-      usr[v] = std::is_same<T, double>::value ? Ar<T>::to_d(su[le * EU + v * N + i])
-                                              : A.us[(e0 + le) * EU + v * N + i];
+    for (int v = 0; v < NV; ++v) usr[v] = A.us[(e0 + le) * EU + v * N + i];
     if constexpr (!std::is_same<T, ff>::value) {
-      // FP64 combination (native FP64 and the mixed FP32 form).  The first stage (a = 0, b = 1)
+      // FP64 combination (the mixed FP32 form).  The first stage (a = 0, b = 1)
       // is one FMA per value; the branch is uniform over the grid (kernel arguments), so the
       // other stages do not pay for it
       if (A.rk == RK_B1) {
@@ -536,31 +530,6 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value) k_s
     }
   }
   __syncthreads();
-  if constexpr (std::is_same<T, double>::value) {
-    // the density-gradient indicator of the new state (FP64 form; the same arithmetic as the
-    // indicator kernel): eta = 2 max_i |D_xi rho|, flags from the thresholds
-    if (A.flags) {
-      if (act) {
-        const double* rho = su + le * EU;
-        double g2 = 0.0;
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-          int qf, ia;
-          pt_split<DIM, NP>(i, a, &qf, &ia);
-          double d = 0.0;
-#pragma unroll
-          for (int j = 0; j < NP; ++j) d += ops.D[ia][j] * rho[line_pt<DIM, NP>(a, qf, j)];
-          g2 += d * d;
-        }
-        atomicMax(&sg2[le], static_cast<unsigned long long>(__double_as_longlong(g2)));  // g2 >= 0
-      }
-      __syncthreads();
-      if (act && i == 0) {
-        const double val = 2.0 * sqrt(__longlong_as_double(static_cast<long long>(sg2[le])));
-        A.flags[e0 + le] = int8_t(val > A.th_r ? 1 : (val < A.th_c ? -1 : 0));
-      }
-    }
-  }
   if (trace_out) {
     // one thread per (element, face, face point), all variables from one set of indices
     constexpr int FQ = S::NFC * NF;
@@ -652,21 +621,6 @@ int launch_faces_impl(int dim, int p, FaceArgs A, const DevOps& o, cudaStream_t 
   return 0;
 }
 
-// Resident warps per SM allowed to the FP64 element kernel.  Its blocks are scheduled while the
-// interface kernel they wait for still runs (dependent launch) and hold their slots while they
-// wait; with the whole SM open to them (2D p = 3: 13 blocks of 4 warps, bounded by shared
-// memory) they leave that kernel too few warps.  Measured on the 2D p = 3 workload: 8, 9, 10, 11
-// and 16 resident blocks give +0.5, +0.7, +0.3, +0.15 and -1.4% against 13.  The other
-// arithmetic forms keep the full residency.
-constexpr int STAGE_F64_MAX_WARPS = 36;
-template <int DIM, int NP, class T>
-size_t stage_smem_pad() {
-  static const size_t pad = std::is_same<T, double>::value
-                                ? residency_pad(k_stage_t<DIM, NP, T>, Sz<DIM, NP>::BT, STAGE_F64_MAX_WARPS)
-                                : 0;
-  return pad;
-}
-
 template <class T>
 int launch_stage_impl(int dim, int p, const StageArgs& A, const DevOps& o, cudaStream_t s, Err* err) {
   if (A.M <= 0) return 0;
@@ -675,8 +629,7 @@ int launch_stage_impl(int dim, int p, const StageArgs& A, const DevOps& o, cudaS
   FR_NP_DISPATCH(dim, p, ({
                    using SS = Sz<DD, NN>;
                    unsigned nb = unsigned((A.M + SS::EPB - 1) / SS::EPB);
-                   if (launch_dependent_smem(k_stage_t<DD, NN, T>, nb, SS::BT, stage_smem_pad<DD, NN, T>(), s, A,
-                                             ops) != cudaSuccess)
+                   if (launch_dependent(k_stage_t<DD, NN, T>, nb, SS::BT, s, A, ops) != cudaSuccess)
                      return set_error(err, FR_ECUDA, "element kernel launch");
                  }));
   FR_LAUNCH_CHECK(err);

@@ -10,6 +10,7 @@
 #include "fr_internal.cuh"
 #include "fr_kernels.cuh"
 #include "fr_solver.cuh"
+#include "fr_stage_fx.cuh"
 
 namespace frg {
 
@@ -273,7 +274,8 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_transfer(KG g, const uint64
                                                               int64_t Mn_ub, const int64_t* __restrict__ d_Mn,
                                                               const __grid_constant__ DevOps ops,
                                                               const double* __restrict__ uo,
-                                                              double* __restrict__ un, const TraceCopy tc) {
+                                                              double* __restrict__ un, const TraceCopy tc,
+                                                              const __grid_constant__ TraceFx tfx) {
   pdl_wait_then_release();
   using S = Sz<DIM, NP>;
   constexpr int N = S::N, NV = S::NV, EU = S::EU, EPB = S::EPB;
@@ -376,10 +378,36 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_transfer(KG g, const uint64
 #pragma unroll
     for (int v = 0; v < NV; ++v) un[(j * NV + v) * N + i] = acc[v];
   }
-  if (tc.dst && rounds > 0) {
-    // the traces of this block's refined and fused elements, from their new state staged in
-    // shared memory (the last round ended with a barrier): one thread per (element, face, face
-    // point), all variables, the same sums in the same order as the trace kernel in FP64
+  if (tc.dst && tc.kind == 0 && rounds > 0) {
+    // FP64 form: the traces of this block's refined and fused elements in fixed point, bitwise those
+    // of the element and trace kernels (the last round ended with a barrier, sb is free)
+    __shared__ uint32_t se[EPB * FX_GROUPS];
+    __shared__ int2 slm[NP], slp[NP];
+    for (int k = threadIdx.x; k < EPB * FX_GROUPS; k += blockDim.x) se[k] = 0u;
+    if (threadIdx.x < NP) {
+      slm[threadIdx.x] = tfx.lm[threadIdx.x];
+      slp[threadIdx.x] = tfx.lp[threadIdx.x];
+    }
+    __syncthreads();
+    uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
+    if (work) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) w[fx_group(v, NV)] = max(w[fx_group(v, NV)], fx_mag(acc[v]));
+    }
+    fx_group_max<N>(w[0], w[1], w[2], i, act, se + (act ? le : 0) * FX_GROUPS);
+    __syncthreads();
+    int2* sv = reinterpret_cast<int2*>(&sb[0][0]);
+    if (work) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+        sv[le * EU + v * N + i] = fx_limbs(acc[v], fx_exp(se[le * FX_GROUPS + fx_group(v, NV)]));
+    }
+    __syncthreads();
+    const int ne = int((Mn - j0) < EPB ? (Mn - j0) : EPB);
+    fx_traces<DIM, NP>(sv, se, slm, slp, tfx.kt, ne, s_tag, static_cast<double*>(tc.dst) + j0 * S::EF);
+  } else if (tc.dst && rounds > 0) {
+    // the same in the other forms' trace types: FP64 sums in the trace kernel's order, from the new
+    // state staged in shared memory, one thread per (element, face, face point), all variables
     constexpr int NF = S::NF, FQ = S::NFC * NF, EF = S::EF;
     if (work) {
 #pragma unroll
@@ -397,9 +425,7 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_transfer(KG g, const uint64
         double t = 0.0;
 #pragma unroll
         for (int m = 0; m < NP; ++m) t = fma(lf[m], sa[le2][v * N + line_pt<DIM, NP>(f >> 1, q, m)], t);
-        if (tc.kind == 0)
-          static_cast<double*>(tc.dst)[o + v * NF] = t;
-        else if (tc.kind == 1)
+        if (tc.kind == 1)
           static_cast<float*>(tc.dst)[o + v * NF] = __double2float_rn(t);
         else
           static_cast<ff*>(tc.dst)[o + v * NF] = ff_from_double(t);
@@ -584,7 +610,8 @@ int launch_transfer(int dim, int p, const KG& g, const uint64_t* old_keys, int64
   FR_DISPATCH(dim, p, ({
                 using SS = Sz<DD, NN>;
                 launch_dependent(k_transfer<DD, NN>, unsigned((M_new + SS::EPB - 1) / SS::EPB), SS::BT, s, g,
-                                 old_keys, n_old, new_keys, src, tag, bad, M_new, d_M_new, ops, u_old, u_new, tc);
+                                 old_keys, n_old, new_keys, src, tag, bad, M_new, d_M_new, ops, u_old, u_new, tc,
+                                 make_trace_fx(p, ops));
               }));
   FR_LAUNCH_CHECK(err);
   return 0;

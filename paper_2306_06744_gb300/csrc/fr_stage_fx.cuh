@@ -1,0 +1,391 @@
+// fr_stage_fx.cuh -- element and trace kernels of the FP64 form (arXiv 2306.06744, Sec. 2.1), with
+// their contractions in block fixed point (fr_fixed.cuh).
+#pragma once
+
+#include "fr_fixed.cuh"
+#include "fr_kernels.cuh"
+
+namespace frg {
+
+// Operator tables of the fixed-point contractions (passed by value: constant bank, copied to shared
+// memory by the kernels because threads of a warp read different rows)
+struct TraceFx {
+  int2 lm[NPMAX], lp[NPMAX];
+  int kt;  // scale of the entries
+};
+struct OpsFx {
+  int2 Dt[NPMAX][NPMAX], gLh[NPMAX], gRh[NPMAX];
+  int kd;                    // scale of the derivative and its correction
+  TraceFx tr;
+  double D[NPMAX][NPMAX];    // plain derivative (density-gradient indicator, FP64)
+  double gm1, ngmh;          // gamma - 1, -(gamma - 1)/2
+};
+inline TraceFx make_trace_fx(int p, const DevOps& o) {
+  TraceFx r{};
+  double st[2] = {0.0, 0.0};
+  for (int i = 0; i <= p; ++i) {
+    st[0] += fabs(o.lm[i]);
+    st[1] += fabs(o.lp[i]);
+  }
+  r.kt = fx_scale(st[0] > st[1] ? st[0] : st[1]);
+  for (int i = 0; i <= p; ++i) {
+    r.lm[i] = fx_coef(o.lm[i], r.kt);
+    r.lp[i] = fx_coef(o.lp[i], r.kt);
+  }
+  return r;
+}
+// gLh, gRh carry the factor 1/2 of the doubled common flux
+inline OpsFx make_ops_fx(int dim, int p, const DevOps& o, double gamma) {
+  OpsFx r{};
+  const int n = p + 1;
+  double sd = 0.0;
+  for (int i = 0; i < n; ++i) {
+    double s = 0.5 * (fabs(o.gL[i]) + fabs(o.gR[i]));
+    for (int j = 0; j < n; ++j) s += fabs(o.Dt[i][j]);
+    sd = s > sd ? s : sd;
+  }
+  r.kd = fx_scale(dim * sd);  // one accumulator sums the terms of all axes
+  r.tr = make_trace_fx(p, o);
+  for (int i = 0; i < n; ++i) {
+    r.gLh[i] = fx_coef(0.5 * o.gL[i], r.kd);
+    r.gRh[i] = fx_coef(0.5 * o.gR[i], r.kd);
+    for (int j = 0; j < n; ++j) {
+      r.Dt[i][j] = fx_coef(o.Dt[i][j], r.kd);
+      r.D[i][j] = o.D[i][j];
+    }
+  }
+  r.gm1 = gamma - 1.0;
+  r.ngmh = -0.5 * (gamma - 1.0);
+  return r;
+}
+
+// Traces of the block's elements from their fixed-point state sv[le][v][i] with group exponents
+// se[le][group]: one thread per (element, face, face point), all variables.  need (nullable): only
+// elements with a non-zero entry.
+template <int DIM, int NP>
+__device__ __forceinline__ void fx_traces(const int2* sv, const uint32_t* se, const int2* slm, const int2* slp, int kt,
+                                          int ne, const int8_t* need, double* to) {
+  using S = Sz<DIM, NP>;
+  constexpr int N = S::N, NV = S::NV, NF = S::NF, EU = S::EU, EF = S::EF, FQ = S::NFC * NF;
+  for (int k = threadIdx.x; k < ne * FQ; k += blockDim.x) {
+    const int le = k / FQ, r = k % FQ;
+    if (need && !need[le]) continue;
+    const int f = r / NF, q = r % NF;
+    const int2* lf = (f & 1) ? slp : slm;
+    int2 c[NP];
+    int pts[NP];
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      c[j] = lf[j];
+      pts[j] = le * EU + line_pt<DIM, NP>(f >> 1, q, j);
+    }
+    double* t = to + int64_t(le) * EF + f * NV * NF + q;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      FxAcc a{0, 0};
+#pragma unroll
+      for (int j = 0; j < NP; ++j) fx_mac(a, sv[pts[j] + v * N], c[j]);
+      const uint32_t e = se[le * FX_GROUPS + fx_group(v, NV)];
+      t[v * NF] = fx_double(fx_sum(a), fx_unit(fx_exp(e), kt), e >= FX_E_BAD);
+    }
+  }
+}
+
+// traces tr[e][f][v][q] = sum_j l_j(+-1) u[e][v][line point j] of a whole mesh, bitwise those that the
+// element kernel writes with a state (blocks of EPB elements, one thread per point)
+template <int DIM, int NP>
+__global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_traces_fx(const double* __restrict__ u, int64_t M,
+                                                               const __grid_constant__ TraceFx ops,
+                                                               double* __restrict__ tr,
+                                                               const int8_t* __restrict__ mask,
+                                                               const int64_t* __restrict__ d_M) {
+  pdl_wait_then_release();
+  using S = Sz<DIM, NP>;
+  constexpr int N = S::N, NV = S::NV, EU = S::EU, EPB = S::EPB;
+  __shared__ int2 sv[EPB * EU];
+  __shared__ int2 slm[NP], slp[NP];
+  __shared__ uint32_t se[EPB * FX_GROUPS];
+  __shared__ int8_t need[EPB];
+  const int tid = threadIdx.x;
+  if (d_M && *d_M < M) M = *d_M;  // the element count on the device (M is then a bound of it)
+  const int64_t e0 = int64_t(blockIdx.x) * EPB;
+  if (e0 >= M) return;
+  const int ne = int((M - e0) < EPB ? (M - e0) : EPB);
+  const int le = tid / N, i = tid % N;
+  if (tid < ne) need[tid] = mask ? mask[e0 + tid] : 1;
+  if (tid < NP) {
+    slm[tid] = ops.lm[tid];
+    slp[tid] = ops.lp[tid];
+  }
+  for (int k = tid; k < EPB * FX_GROUPS; k += blockDim.x) se[k] = 0u;
+  __syncthreads();
+  const bool act = le < ne && need[le < EPB ? le : 0];
+  double q[NV];
+  uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    q[v] = act ? u[(e0 + le) * EU + v * N + i] : 0.0;
+    w[fx_group(v, NV)] = max(w[fx_group(v, NV)], fx_mag(q[v]));
+  }
+  fx_group_max<N>(w[0], w[1], w[2], i, act, se + (act ? le : 0) * FX_GROUPS);
+  __syncthreads();
+  if (act) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+      sv[le * EU + v * N + i] = fx_limbs(q[v], fx_exp(se[le * FX_GROUPS + fx_group(v, NV)]));
+  }
+  __syncthreads();
+  fx_traces<DIM, NP>(sv, se, slm, slp, ops.kt, ne, need, tr + e0 * S::EF);
+}
+
+// planes of the element's fluxes: the axes' mass fluxes, the distinct entries of the symmetric
+// momentum flux tensor, the axes' energy fluxes
+template <int DIM>
+struct FluxPlanes {
+  static constexpr int NS = DIM * (DIM + 1) / 2;
+  static constexpr int NPL = 2 * DIM + NS;
+  // row a, column b of the symmetric tensor
+  static __host__ __device__ constexpr int sym(int a, int b) {
+    return a > b ? sym(b, a) : a * DIM - a * (a - 1) / 2 + (b - a);
+  }
+  // plane of variable v's flux along axis a
+  static __host__ __device__ constexpr int of(int a, int v) {
+    return v == 0 ? a : (v == DIM + 1 ? DIM + NS + a : DIM + sym(a, v - 1));
+  }
+};
+
+// Element stage of the FP64 form: R = -sum_a (2/h) [ sum_j Dt_ij f_j + gL_i F(-1) + gR_i F(+1) ]
+// along each axis (corrected-flux derivative of Sec. 2.1 with the correction folded into Dt; the
+// interface kernel stores 2F and the slopes carry the 1/2), then out = a*un + b*us + c*R (Eq. rk3)
+// and (optionally) the flags of out and its traces.
+//
+// The pointwise flux and the Runge-Kutta combination are FP64 (about 38 operations a point in 3D); the
+// contractions, 120 of the 158 multiply-adds a point at 3D p = 3, run in fixed point on the integer
+// pipes (fr_fixed.cuh), all axes of a variable in one accumulator.  The correction's accumulator is
+// the derivative's, moved to the larger of the two exponents, so that the volume part stays before the
+// wait on the interface kernel.
+template <int DIM, int NP>
+__global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_stage_fx(StageArgs A, const __grid_constant__ OpsFx ops) {
+  using S = Sz<DIM, NP>;
+  using FP = FluxPlanes<DIM>;
+  constexpr int N = S::N, NV = S::NV, NF = S::NF, EU = S::EU, EF = S::EF, EPB = S::EPB, NPL = FP::NPL;
+  constexpr int NIT = (EF + N - 1) / N;
+  __shared__ int2 sfl[EPB * NPL * N];  // fluxes; after the derivative the new state
+  __shared__ int2 sfc[EPB * EF];       // common fluxes
+  __shared__ int2 sD[NP * NP], sgL[NP], sgR[NP], slm[NP], slp[NP];
+  __shared__ uint32_t sef[EPB * FX_GROUPS], sec[EPB * FX_GROUPS], seo[EPB * FX_GROUPS];
+  __shared__ double sh2[EPB];              // per element: c * (-2/h)
+  __shared__ unsigned long long sg2[EPB];  // per element: the indicator's max |D rho|^2 (as bits)
+  const int tid = threadIdx.x;
+  const int64_t e0 = int64_t(blockIdx.x) * EPB;
+  const int ne = int((A.M - e0) < EPB ? (A.M - e0) : EPB);
+  const int le = tid / N, i = tid % N;
+  const bool act = le < ne;
+  const int les = act ? le : 0;
+  // the stage's input state, the state at the start of the step and the keys come from earlier
+  // launches than the interface kernel this one depends on: everything up to the volume sums is done
+  // while that kernel drains; its common fluxes are read after the wait
+  const int64_t b0 = (e0 + le) * EU + i;
+  double q[NV], unr[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    q[v] = act ? A.us[b0 + v * N] : 1.0;
+    unr[v] = (act && (A.rk & RK_A)) ? A.un[b0 + v * N] : 0.0;
+  }
+  // c * (-2/h): 2^depth * (2/L) is exact, so this equals the rounded -2^(depth+1)/L times c
+  if (tid < ne) {
+    sh2[tid] = -A.c * (double(1ull << A.g.depth(A.keys[e0 + tid])) * A.twoL);
+    sg2[tid] = 0ull;
+  }
+  for (int k = tid; k < EPB * FX_GROUPS; k += blockDim.x) sef[k] = sec[k] = seo[k] = 0u;
+  for (int k = tid; k < NP * NP; k += blockDim.x) sD[k] = ops.Dt[k / NP][k % NP];
+  if (tid < NP) {
+    sgL[tid] = ops.gLh[tid];
+    sgR[tid] = ops.gRh[tid];
+    slm[tid] = ops.tr.lm[tid];
+    slp[tid] = ops.tr.lp[tid];
+  }
+  __syncthreads();
+  // pointwise fluxes, FP64
+  double fl[NPL];
+  {
+    const double rinv = rcp_t(q[0]);
+    double vel[DIM];
+    double m2 = 0.0;
+#pragma unroll
+    for (int b = 0; b < DIM; ++b) {
+      vel[b] = q[1 + b] * rinv;
+      m2 = b == 0 ? q[1] * vel[0] : fma(q[1 + b], vel[b], m2);
+    }
+    const double p = fma(ops.ngmh, m2, ops.gm1 * q[NV - 1]);
+    const double Ep = q[NV - 1] + p;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+      fl[FP::of(a, 0)] = q[1 + a];
+#pragma unroll
+      for (int b = a; b < DIM; ++b) fl[FP::of(a, 1 + b)] = a == b ? fma(q[1 + b], vel[a], p) : q[1 + b] * vel[a];
+      fl[FP::of(a, NV - 1)] = Ep * vel[a];
+    }
+  }
+  {
+    uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      const int g = k < DIM ? 0 : (k < DIM + FP::NS ? 1 : 2);
+      w[g] = max(w[g], fx_mag(fl[k]));
+    }
+    if (!act) w[0] = w[1] = w[2] = 0u;
+    fx_group_max<N>(w[0], w[1], w[2], i, act, sef + les * FX_GROUPS);
+  }
+  __syncthreads();
+  int E[FX_GROUPS];
+#pragma unroll
+  for (int g = 0; g < FX_GROUPS; ++g) E[g] = fx_exp(sef[les * FX_GROUPS + g]);
+  if (act) {
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) {
+      const int g = k < DIM ? 0 : (k < DIM + FP::NS ? 1 : 2);
+      sfl[(le * NPL + k) * N + i] = fx_limbs(fl[k], E[g]);
+    }
+  }
+  __syncthreads();
+  // volume part of the folded derivative, sum_a sum_j Dt_ij f_j
+  FxAcc acc[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) acc[v] = FxAcc{0, 0};
+  if (act) {
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+      int qf, ia;
+      pt_split<DIM, NP>(i, a, &qf, &ia);
+#pragma unroll
+      for (int j = 0; j < NP; ++j) {
+        const int2 c = sD[ia * NP + j];
+        const int2* f = sfl + le * NPL * N + line_pt<DIM, NP>(a, qf, j);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) fx_mac(acc[v], f[FP::of(a, v) * N], c);
+      }
+    }
+  }
+  pdl_wait_then_release();
+  // common fluxes of the element, staged by its own threads
+  {
+    const double* fc = static_cast<const double*>(A.fcomm) + (e0 + le) * EF;
+    double F[NIT];
+    uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
+#pragma unroll
+    for (int t = 0; t < NIT; ++t) {
+      const int k = i + t * N;
+      F[t] = (act && k < EF) ? fc[k] : 0.0;
+    }
+#pragma unroll
+    for (int t = 0; t < NIT; ++t) {
+      const int v = ((i + t * N) / NF) % NV;
+      const uint32_t m = fx_mag(F[t]);
+      if (v == 0)
+        w[0] = max(w[0], m);
+      else if (v == NV - 1)
+        w[2] = max(w[2], m);
+      else
+        w[1] = max(w[1], m);
+    }
+    fx_group_max<N>(w[0], w[1], w[2], i, act, sec + les * FX_GROUPS);
+    __syncthreads();
+    // the sums move to the larger exponent of fluxes and common fluxes
+#pragma unroll
+    for (int g = 0; g < FX_GROUPS; ++g) {
+      const int Ec = fx_exp(sec[les * FX_GROUPS + g]);
+      if (Ec > E[g]) {
+        const int s = Ec - E[g] < 63 ? Ec - E[g] : 63;
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+          if (fx_group(v, NV) == g) {
+            acc[v].h = fx_sum(acc[v]) >> s;
+            acc[v].m = 0;
+          }
+        E[g] = Ec;
+      }
+    }
+    if (act) {
+#pragma unroll
+      for (int t = 0; t < NIT; ++t) {
+        const int k = i + t * N;
+        if (k < EF) {
+          const int v = (k / NF) % NV;
+          sfc[le * EF + k] = fx_limbs(F[t], v == 0 ? E[0] : (v == NV - 1 ? E[2] : E[1]));
+        }
+      }
+    }
+  }
+  __syncthreads();
+  double out[NV];
+  uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
+  if (act) {
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+      int qf, ia;
+      pt_split<DIM, NP>(i, a, &qf, &ia);
+      const int2 cl = sgL[ia], cr = sgR[ia];
+      const int2* Fm = sfc + le * EF + (2 * a) * NV * NF + qf;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        fx_mac(acc[v], Fm[v * NF], cl);
+        fx_mac(acc[v], Fm[(NV + v) * NF], cr);
+      }
+    }
+    const double cs = sh2[le];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const int Ev = E[fx_group(v, NV)];
+      const double R = fx_double(fx_sum(acc[v]), fx_unit(Ev, ops.kd), Ev >= FX_E_BAD);
+      // the first stage (a = 0, b = 1) is one FMA per value; the tests are uniform over the grid
+      double o = fma(cs, R, (A.rk & RK_B1) ? q[v] : A.b * q[v]);
+      if (A.rk & RK_A) o = fma(A.a, unr[v], o);
+      out[v] = o;
+      A.out[b0 + v * N] = o;
+      w[fx_group(v, NV)] = max(w[fx_group(v, NV)], fx_mag(o));
+    }
+  }
+  if (A.flags) {
+    // the density-gradient indicator of the new state (the same arithmetic as the indicator
+    // kernel): eta = 2 max_i |D_xi rho|, flags from the thresholds
+    double* rho = reinterpret_cast<double*>(sfl) + les * N;
+    if (act) rho[i] = out[0];
+    __syncthreads();
+    if (act) {
+      double g2 = 0.0;
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) {
+        int qf, ia;
+        pt_split<DIM, NP>(i, a, &qf, &ia);
+        double d = 0.0;
+#pragma unroll
+        for (int j = 0; j < NP; ++j) d += ops.D[ia][j] * rho[line_pt<DIM, NP>(a, qf, j)];
+        g2 += d * d;
+      }
+      atomicMax(&sg2[le], static_cast<unsigned long long>(__double_as_longlong(g2)));  // g2 >= 0
+    }
+    __syncthreads();
+    if (act && i == 0) {
+      const double val = 2.0 * sqrt(__longlong_as_double(static_cast<long long>(sg2[le])));
+      A.flags[e0 + le] = int8_t(val > A.th_r ? 1 : (val < A.th_c ? -1 : 0));
+    }
+  }
+  if (A.trace_out) {
+    fx_group_max<N>(w[0], w[1], w[2], i, act, seo + les * FX_GROUPS);
+    __syncthreads();
+    if (act) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+        sfl[le * EU + v * N + i] = fx_limbs(out[v], fx_exp(seo[le * FX_GROUPS + fx_group(v, NV)]));
+    }
+    __syncthreads();
+    fx_traces<DIM, NP>(sfl, seo, slm, slp, ops.tr.kt, ne, nullptr, static_cast<double*>(A.trace_out) + e0 * EF);
+  }
+}
+
+// Resident warps per SM allowed to the element kernel: its blocks are scheduled while the interface
+// kernel they wait for still runs and hold their slots while they wait.
+constexpr int STAGE_F64_MAX_WARPS = 64;
+
+}  // namespace frg
