@@ -170,26 +170,52 @@ struct Ar<ff> {
 };
 
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
-// reciprocals: FP64 by Newton-Raphson from the hardware approximation (two iterations square the
-// relative error twice, from ~2^-23 to below the FP64 rounding error); FP32 by the fast divide;
-// double-word by the corrected quotient above.
+// reciprocals: FP64 from the hardware approximation r (relative error e ~2^-23) by one third-order
+// step, r (1 + e + e^2), which leaves e^3 (three FP64 operations; two Newton steps take four); FP32 by
+// the fast divide; double-word by the corrected quotient above.
 __device__ __forceinline__ double rcp_t(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  double e = fma(-x, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-x, r, 1.0);
-  return fma(r, e, r);
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
 }
 __device__ __forceinline__ float rcp_t(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ ff rcp_t(ff x) { return ff{1.f, 0.f} / x; }
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double sqrt_t(double a) { return sqrt(a); }
+// FP64 square root from the hardware approximation y of 1/sqrt(a) (~2^-22): g = a y, one Newton step
+// for the root (error ~2^-44), then Markstein's correction with the exact residual a - g^2 and y/2
+// (Markstein 1990), which leaves half an ulp and 2^-66: five FP64 operations, the halving is done on
+// the exponent.  Zero, values below 2^-959 (whose residual could fall below the normal range),
+// infinities, NaN and negative values take the library's.
+__device__ __forceinline__ double sqrt_t(double a) {
+  const uint32_t ex = uint32_t(__double2hiint(a)) >> 20;  // sign and exponent
+  if (ex - 64u > 1982u) return sqrt(a);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double h = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));
+  double g = a * y;
+  g = fma(g, fma(-g, h, 0.5), g);
+  return fma(fma(-g, g, a), h, g);
+}
 __device__ __forceinline__ float sqrt_t(float a) { return sqrtf(a); }
 __device__ __forceinline__ double fabs_t(double a) { return fabs(a); }
 __device__ __forceinline__ float fabs_t(float a) { return fabsf(a); }
 __device__ __forceinline__ double fmax_t(double a, double b) { return fmax(a, b); }
+// the larger of two non-negative values: positive doubles order as their bit patterns, so the FP64
+// pipe is left out (a NaN wins)
+__device__ __forceinline__ double fmax_pos(double a, double b) {
+  return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+}
+__device__ __forceinline__ float fmax_pos(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ ff fmax_pos(ff a, ff b) { return fmax_t(a, b); }
 __device__ __forceinline__ float fmax_t(float a, float b) { return fmaxf(a, b); }
+
+// -x/2 without a multiplication where the exponent can be lowered (x normal, above 2^-1021)
+__device__ __forceinline__ double neg_half(double x) {
+  return __hiloint2double((__double2hiint(x) - (1 << 20)) ^ int(0x80000000u), __double2loint(x));
+}
+__device__ __forceinline__ float neg_half(float x) { return -0.5f * x; }
+__device__ __forceinline__ ff neg_half(ff x) { return {-0.5f * x.h, -0.5f * x.l}; }
 
 // zero / constant helpers
 template <class T>

@@ -5,6 +5,7 @@
 // instantiated in its own translation unit (fr_prec_*.cu).
 #pragma once
 
+#include <cmath>
 #include <type_traits>
 
 #include "fr_arith.cuh"
@@ -22,9 +23,9 @@ struct OpsT {
   T gLh[NPMAX], gRh[NPMAX], lm[NPMAX], lp[NPMAX];
   T I[2][NPMAX][NPMAX];
   T P[2][NPMAX][NPMAX];
-  // gas constants in the arithmetic type, formed on the host (set_gas): gamma, gamma - 1 and
+  // gas constants in the arithmetic type, formed on the host (set_gas): sqrt(gamma), gamma - 1 and
   // -(gamma - 1)/2, so that no thread spends FP64 operations on them
-  T gam, gm1, ngmh;
+  T sgam, gm1, ngmh;
 };
 
 inline double host_conv(double x, double*) { return x; }
@@ -38,7 +39,7 @@ inline ff host_conv(double x, ff*) {
 template <class T>
 void set_gas(OpsT<T>* r, double gamma) {
   T* tag = nullptr;
-  r->gam = host_conv(gamma, tag);
+  r->sgam = host_conv(std::sqrt(gamma), tag);
   r->gm1 = host_conv(gamma - 1.0, tag);
   r->ngmh = host_conv(-0.5 * (gamma - 1.0), tag);
 }
@@ -105,11 +106,10 @@ __device__ __forceinline__ void pt_split(int i, int axis, int* q, int* ia) {
 
 // Twice the Rusanov common flux along +axis between the minus-side state qL and the plus-side
 // qR, F2 = f(qL) + f(qR) - lambda (qR - qL) with lambda = max(|u_n| + c) of the two states
-// (Sec. 4.3); the factor 1/2 is carried by the correction slopes.  ngmh = -(gamma - 1)/2, so
-// that p = (gamma - 1) E + ngmh |m|^2 / rho.
+// (Sec. 4.3); the factor 1/2 is carried by the correction slopes.  sgam = sqrt(gamma), gm1 =
+// gamma - 1.
 template <int DIM, class T>
-__device__ __forceinline__ void rusanov2_t(const T* qL, const T* qR, int axis, T gam, T gm1, T ngmh,
-                                           T* F2) {
+__device__ __forceinline__ void rusanov2_t(const T* qL, const T* qR, int axis, T sgam, T gm1, T* F2) {
   constexpr int NV = DIM + 2;
   // both reciprocal densities from one reciprocal: 1/rho_L = rho_R / (rho_L rho_R), and so on
   const T rLR = rcp_t(qL[0] * qR[0]);
@@ -120,8 +120,8 @@ __device__ __forceinline__ void rusanov2_t(const T* qL, const T* qR, int axis, T
     m2L = fma_t(qL[1 + b], qL[1 + b], m2L);
     m2R = fma_t(qR[1 + b], qR[1 + b], m2R);
   }
-  T pL = fma_t(ngmh, m2L * rL, gm1 * qL[NV - 1]);
-  T pR = fma_t(ngmh, m2R * rR, gm1 * qR[NV - 1]);
+  const T pL = gm1 * fma_t(m2L, neg_half(rL), qL[NV - 1]);
+  const T pR = gm1 * fma_t(m2R, neg_half(rR), qR[NV - 1]);
   // normal momenta, selected with unrolled predicates so the state stays in registers
   T mnL = qL[1], mnR = qR[1];
 #pragma unroll
@@ -131,21 +131,18 @@ __device__ __forceinline__ void rusanov2_t(const T* qL, const T* qR, int axis, T
       mnR = qR[1 + b];
     }
   T vL = mnL * rL, vR = mnR * rR;
-  T cL = sqrt_t(gam * pL * rL), cR = sqrt_t(gam * pR * rR);
-  T lam = fmax_t(fabs_t(vL) + cL, fabs_t(vR) + cR);
-  T fL[NV], fR[NV];
-  fL[0] = mnL;
-  fR[0] = mnR;
+  // |v| + c with c = sqrt(gamma) sqrt(p / rho)
+  const T lam = fmax_pos(fma_t(sgam, sqrt_t(pL * rL), fabs_t(vL)), fma_t(sgam, sqrt_t(pR * rR), fabs_t(vR)));
+  // f(qL) + f(qR) - lambda (qR - qL), the sums as multiply-adds; the pressures enter the normal
+  // momentum through the chain's start (a select) instead of an addition per component
+  const T pp = pL + pR;
+  F2[0] = fma_t(lam, qL[0] - qR[0], mnL + mnR);
 #pragma unroll
   for (int b = 0; b < DIM; ++b) {
-    T a = qL[1 + b] * vL, c = qR[1 + b] * vR;
-    fL[1 + b] = (b == axis) ? a + pL : a;
-    fR[1 + b] = (b == axis) ? c + pR : c;
+    const T s = fma_t(qL[1 + b], vL, fma_t(qR[1 + b], vR, b == axis ? pp : zero_t<T>()));
+    F2[1 + b] = fma_t(lam, qL[1 + b] - qR[1 + b], s);
   }
-  fL[NV - 1] = (qL[NV - 1] + pL) * vL;
-  fR[NV - 1] = (qR[NV - 1] + pR) * vR;
-#pragma unroll
-  for (int v = 0; v < NV; ++v) F2[v] = fma_t(lam, qL[v] - qR[v], fL[v] + fR[v]);
+  F2[NV - 1] = fma_t(lam, qL[NV - 1] - qR[NV - 1], fma_t(qL[NV - 1] + pL, vL, (qR[NV - 1] + pR) * vR));
 }
 
 // traces tr[e][f][v][q] = sum_j l_j(+-1) u[e][v][line point j]  (mortar procedure step 1).
@@ -233,7 +230,7 @@ __global__ void __launch_bounds__(FaceCfg<DIM, NP>::T) k_faces_t(FaceArgs A, con
   __shared__ T sW[FPB][DIM == 3 ? (HA > HB ? HA : HB) : 1];
   const T* trace = static_cast<const T*>(A.trace);
   T* fcomm = static_cast<T*>(A.fcomm);
-  const T gam = ops.gam, gm1 = ops.gm1, ngmh = ops.ngmh;
+  const T sgam = ops.sgam, gm1 = ops.gm1;
   const int tid = threadIdx.x;
   // the face lists and neighbour tables are fixed during a time step: they are read while the
   // element kernel this one depends on drains; the traces it wrote are read after the wait
@@ -255,7 +252,7 @@ __global__ void __launch_bounds__(FaceCfg<DIM, NP>::T) k_faces_t(FaceArgs A, con
       qL[v] = tL[v * NF];
       qR[v] = tR[v * NF];
     }
-    rusanov2_t<DIM, T>(qL, qR, axis, gam, gm1, ngmh, F);
+    rusanov2_t<DIM, T>(qL, qR, axis, sgam, gm1, F);
     T* fL = fcomm + ((e * NFC + 2 * axis + 1) * NV) * NF + q;
     T* fR = fcomm + ((nb * NFC + 2 * axis) * NV) * NF + q;
 #pragma unroll
@@ -315,9 +312,9 @@ __global__ void __launch_bounds__(FaceCfg<DIM, NP>::T) k_faces_t(FaceArgs A, con
       uf[v] = trace[((ek * NFC + fk) * NV + v) * NF + q];
     }
     if (sidec)
-      rusanov2_t<DIM, T>(uc, uf, axis, gam, gm1, ngmh, F);
+      rusanov2_t<DIM, T>(uc, uf, axis, sgam, gm1, F);
     else
-      rusanov2_t<DIM, T>(uf, uc, axis, gam, gm1, ngmh, F);
+      rusanov2_t<DIM, T>(uf, uc, axis, sgam, gm1, F);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       fcomm[((ek * NFC + fk) * NV + v) * NF + q] = F[v];
