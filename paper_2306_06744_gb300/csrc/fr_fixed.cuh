@@ -65,7 +65,7 @@ __host__ __device__ __forceinline__ uint32_t fx_mag(double x) { return uint32_t(
 
 // limbs of trunc(x 2^(1081 - E)); |x| < 2^(E - 1022), E >= FX_E_MIN.  The significand with its
 // leading one at bit 62 is shifted down by E - e + 4 (e: x's biased exponent); zeros and subnormals
-// (e = 0) come out as 0.
+// (e = 0) come out as 0.  (The hardware's conversion to 64-bit integers runs on the FP64 pipe.)
 __host__ __device__ __forceinline__ int2 fx_limbs(double x, int E) {
   const uint64_t b = fx_bits(x);
   const int e = int(b >> 52) & 0x7FF;
@@ -73,7 +73,7 @@ __host__ __device__ __forceinline__ int2 fx_limbs(double x, int E) {
   int s = E - e + 4;
   s = s < 63 ? s : 63;
   const uint64_t a = m >> s;
-  const int sg = int(uint32_t(b >> 32)) < 0 ? -1 : 1;
+  const int sg = (int(uint32_t(b >> 32)) >> 31) | 1;
   return make_int2(int(a >> 31) * sg, int(uint32_t(a) & 0x7FFFFFFFu) * sg);
 }
 
@@ -81,18 +81,18 @@ __host__ __device__ __forceinline__ int2 fx_limbs(double x, int E) {
 // at least 1 (and e + 62 below 2047); bad: NaN
 __host__ __device__ __forceinline__ double fx_double(long long v, int e, bool bad) {
   const uint64_t s = uint64_t(v >> 63);
-  uint64_t a = (uint64_t(v) ^ s) - s;
+  uint64_t a = (uint64_t(v) ^ s) - s;  // below 2^62
 #ifdef __CUDA_ARCH__
   const int z = __clzll((long long)a);
 #else
-  const int z = a ? __builtin_clzll(a) : 63;
+  const int z = a ? __builtin_clzll(a) : 64;
 #endif
-  a <<= (z & 63);
-  uint64_t r = (a >> 11) + ((a >> 10) & 1);        // the leading one at bit 52 (a carry moves up)
-  r += uint64_t(uint32_t(e + 62 - z)) << 52;       // ... counts one in the exponent field
-  r = v == 0 ? 0 : (r | (s << 63));
-  if (bad) r = 0x7FF8000000000000ull;
-  return fx_from_bits(r);
+  a <<= (z - 1) & 63;                              // the leading one at bit 62
+  a = (a + 0x200) >> 10;                           // ... at bit 52 (a carry moves up)
+  uint32_t hi = uint32_t(a >> 32) + (uint32_t(e + 62 - z) << 20);  // it counts one in the exponent field
+  hi = v == 0 ? 0u : hi;
+  hi |= (uint32_t(s) & 0x80000000u) | (bad ? 0x7FF80000u : 0u);
+  return fx_from_bits((uint64_t(hi) << 32) | uint32_t(a));
 }
 
 // biased exponent of one unit of a result: values of group exponent E, entries scaled by 2^k

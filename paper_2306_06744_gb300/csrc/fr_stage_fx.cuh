@@ -146,12 +146,24 @@ struct FluxPlanes {
   static constexpr int NPL = 2 * DIM + NS;
   // row a, column b of the symmetric tensor
   static __host__ __device__ constexpr int sym(int a, int b) {
-    return a > b ? sym(b, a) : a * DIM - a * (a - 1) / 2 + (b - a);
+    return (a < b ? a : b) * DIM - (a < b ? a : b) * ((a < b ? a : b) - 1) / 2 + (a < b ? b - a : a - b);
   }
+  // exponent group of plane k
+  static __host__ __device__ constexpr int group(int k) { return k < DIM ? 0 : (k < DIM + NS ? 1 : 2); }
   // plane of variable v's flux along axis a
   static __host__ __device__ constexpr int of(int a, int v) {
     return v == 0 ? a : (v == DIM + 1 ? DIM + NS + a : DIM + sym(a, v - 1));
   }
+};
+
+// Resident blocks the element kernel is compiled for.  It waits on shared memory, barriers and fixed
+// latencies more than on any one pipe, so threads are worth more than registers: 1024 threads an SM (64
+// registers, a few spilled) against 768 and 512 give, per launch, 3D p = 2 (184k leaves) 587, 631 and 712
+// us, 3D p = 4 (15k) 230, 242 and 258 us; at 3D p = 3 (127k), 896 threads are best: 838 us against 853
+// (1024), 872 (768) and 903 (640).  Blocks of 64 threads instead of 128: 894 us.
+template <int DIM, int NP>
+struct StageOcc {
+  static constexpr int value = (Sz<DIM, NP>::N == 64 ? 896 : 1024) / Sz<DIM, NP>::BT;
 };
 
 // Element stage of the FP64 form: R = -sum_a (2/h) [ sum_j Dt_ij f_j + gL_i F(-1) + gR_i F(+1) ]
@@ -159,17 +171,21 @@ struct FluxPlanes {
 // interface kernel stores 2F and the slopes carry the 1/2), then out = a*un + b*us + c*R (Eq. rk3)
 // and (optionally) the flags of out and its traces.
 //
-// The pointwise flux and the Runge-Kutta combination are FP64 (about 38 operations a point in 3D); the
-// contractions, 120 of the 158 multiply-adds a point at 3D p = 3, run in fixed point on the integer
-// pipes (fr_fixed.cuh), all axes of a variable in one accumulator.  The correction's accumulator is
-// the derivative's, moved to the larger of the two exponents, so that the volume part stays before the
-// wait on the interface kernel.
+// The pointwise flux and the Runge-Kutta combination are FP64 (38 operations a point in 3D, of the 158
+// that bounded the kernel at 2 a clock and SM); the contractions run in fixed point on the integer pipes
+// (fr_fixed.cuh), all axes of a variable in one accumulator, the correction's terms in the derivative's
+// accumulator once that has moved to the larger of the two exponents, so that the volume part stays
+// before the wait on the interface kernel.  Per point about 2,400 instructions (a third of them the
+// conversions of 28 values to limbs and 13 back); FP64 pipe 55%, issue slots 54%, shared memory 59% busy,
+// DRAM 28% of peak.  Four 3D p = 3 tubes, 242k leaves: 3.95 ms per launch with the contractions in FP64,
+// 1.62 ms so.
 template <int DIM, int NP>
-__global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_stage_fx(StageArgs A, const __grid_constant__ OpsFx ops) {
+__global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageOcc<DIM, NP>::value)
+    k_stage_fx(StageArgs A, const __grid_constant__ OpsFx ops) {
   using S = Sz<DIM, NP>;
   using FP = FluxPlanes<DIM>;
-  constexpr int N = S::N, NV = S::NV, NF = S::NF, EU = S::EU, EF = S::EF, EPB = S::EPB, NPL = FP::NPL;
-  constexpr int NIT = (EF + N - 1) / N;
+  constexpr int N = S::N, NV = S::NV, NF = S::NF, EU = S::EU, EF = S::EF, EPB = S::EPB, BT = S::BT, NPL = FP::NPL;
+  constexpr int FQ = S::NFC * NF, NIT = (EPB * FQ + BT - 1) / BT;
   __shared__ int2 sfl[EPB * NPL * N];  // fluxes; after the derivative the new state
   __shared__ int2 sfc[EPB * EF];       // common fluxes
   __shared__ int2 sD[NP * NP], sgL[NP], sgR[NP], slm[NP], slp[NP];
@@ -179,26 +195,26 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_stage_fx(StageArgs A, const
   const int tid = threadIdx.x;
   const int64_t e0 = int64_t(blockIdx.x) * EPB;
   const int ne = int((A.M - e0) < EPB ? (A.M - e0) : EPB);
-  const int le = tid / N, i = tid % N;
-  const bool act = le < ne;
-  const int les = act ? le : 0;
+  // threads past the last element repeat its work without storing it, threads past the last point
+  // of the block (27, 9, 25 or 125 points an element) the first element's
+  const int i = tid % N;
+  const bool own = EPB * N == BT || tid < EPB * N;
+  const int le = own ? tid / N : 0;
+  const bool act = own && le < ne;
+  const int64_t b0 = (e0 + (le < ne ? le : ne - 1)) * EU + i;
   // the stage's input state, the state at the start of the step and the keys come from earlier
   // launches than the interface kernel this one depends on: everything up to the volume sums is done
   // while that kernel drains; its common fluxes are read after the wait
-  const int64_t b0 = (e0 + le) * EU + i;
-  double q[NV], unr[NV];
+  double q[NV];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    q[v] = act ? A.us[b0 + v * N] : 1.0;
-    unr[v] = (act && (A.rk & RK_A)) ? A.un[b0 + v * N] : 0.0;
-  }
+  for (int v = 0; v < NV; ++v) q[v] = A.us[b0 + v * N];
   // c * (-2/h): 2^depth * (2/L) is exact, so this equals the rounded -2^(depth+1)/L times c
   if (tid < ne) {
     sh2[tid] = -A.c * (double(1ull << A.g.depth(A.keys[e0 + tid])) * A.twoL);
     sg2[tid] = 0ull;
   }
-  for (int k = tid; k < EPB * FX_GROUPS; k += blockDim.x) sef[k] = sec[k] = seo[k] = 0u;
-  for (int k = tid; k < NP * NP; k += blockDim.x) sD[k] = ops.Dt[k / NP][k % NP];
+  for (int k = tid; k < EPB * FX_GROUPS; k += BT) sef[k] = sec[k] = seo[k] = 0u;
+  for (int k = tid; k < NP * NP; k += BT) sD[k] = ops.Dt[k / NP][k % NP];
   if (tid < NP) {
     sgL[tid] = ops.gLh[tid];
     sgR[tid] = ops.gRh[tid];
@@ -206,9 +222,11 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_stage_fx(StageArgs A, const
     slp[tid] = ops.tr.lp[tid];
   }
   __syncthreads();
-  // pointwise fluxes, FP64
-  double fl[NPL];
+  int E[FX_GROUPS];
+  FxAcc acc[NV];
   {
+    // pointwise fluxes, FP64
+    double fl[NPL];
     const double rinv = rcp_t(q[0]);
     double vel[DIM];
     double m2 = 0.0;
@@ -226,101 +244,98 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_stage_fx(StageArgs A, const
       for (int b = a; b < DIM; ++b) fl[FP::of(a, 1 + b)] = a == b ? fma(q[1 + b], vel[a], p) : q[1 + b] * vel[a];
       fl[FP::of(a, NV - 1)] = Ep * vel[a];
     }
-  }
-  {
     uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
 #pragma unroll
-    for (int k = 0; k < NPL; ++k) {
-      const int g = k < DIM ? 0 : (k < DIM + FP::NS ? 1 : 2);
-      w[g] = max(w[g], fx_mag(fl[k]));
-    }
-    if (!act) w[0] = w[1] = w[2] = 0u;
-    fx_group_max<N>(w[0], w[1], w[2], i, act, sef + les * FX_GROUPS);
-  }
-  __syncthreads();
-  int E[FX_GROUPS];
+    for (int k = 0; k < NPL; ++k) w[FP::group(k)] = max(w[FP::group(k)], fx_mag(fl[k]));
+    if (!own) w[0] = w[1] = w[2] = 0u;
+    fx_group_max<N>(w[0], w[1], w[2], i, own, sef + le * FX_GROUPS);
+    __syncthreads();
 #pragma unroll
-  for (int g = 0; g < FX_GROUPS; ++g) E[g] = fx_exp(sef[les * FX_GROUPS + g]);
-  if (act) {
+    for (int g = 0; g < FX_GROUPS; ++g) E[g] = fx_exp(sef[le * FX_GROUPS + g]);
+    if (own) {
 #pragma unroll
-    for (int k = 0; k < NPL; ++k) {
-      const int g = k < DIM ? 0 : (k < DIM + FP::NS ? 1 : 2);
-      sfl[(le * NPL + k) * N + i] = fx_limbs(fl[k], E[g]);
+      for (int k = 0; k < NPL; ++k) sfl[(le * NPL + k) * N + i] = fx_limbs(fl[k], E[FP::group(k)]);
     }
+    __syncthreads();
   }
-  __syncthreads();
   // volume part of the folded derivative, sum_a sum_j Dt_ij f_j
-  FxAcc acc[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) acc[v] = FxAcc{0, 0};
-  if (act) {
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      int qf, ia;
-      pt_split<DIM, NP>(i, a, &qf, &ia);
+  for (int a = 0; a < DIM; ++a) {
+    int qf, ia;
+    pt_split<DIM, NP>(i, a, &qf, &ia);
 #pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        const int2 c = sD[ia * NP + j];
-        const int2* f = sfl + le * NPL * N + line_pt<DIM, NP>(a, qf, j);
+    for (int j = 0; j < NP; ++j) {
+      const int2 c = sD[ia * NP + j];
+      const int2* f = sfl + le * NPL * N + line_pt<DIM, NP>(a, qf, j);
 #pragma unroll
-        for (int v = 0; v < NV; ++v) fx_mac(acc[v], f[FP::of(a, v) * N], c);
-      }
+      for (int v = 0; v < NV; ++v) fx_mac(acc[v], f[FP::of(a, v) * N], c);
     }
   }
   pdl_wait_then_release();
-  // common fluxes of the element, staged by its own threads
-  {
-    const double* fc = static_cast<const double*>(A.fcomm) + (e0 + le) * EF;
-    double F[NIT];
+  // common fluxes of the block's elements, one thread per face point: staged in FP64 while the group
+  // exponents are formed, then converted in place
+#pragma unroll
+  for (int t = 0; t < NIT; ++t) {
+    const int k = tid + t * BT;
+    const bool in = (t + 1) * BT <= EPB * FQ || k < EPB * FQ;
+    if ((EPB * FQ) % 32 == 0 && FQ % 32 == 0 && !in) break;  // whole warps
+    const int lf = in ? k / FQ : 0, r = k % FQ, o = (r / NF) * NV * NF + r % NF;
+    const double* fc = static_cast<const double*>(A.fcomm) + (e0 + (lf < ne ? lf : ne - 1)) * EF + o;
     uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
+    if (in) {
+      double F[NV];
 #pragma unroll
-    for (int t = 0; t < NIT; ++t) {
-      const int k = i + t * N;
-      F[t] = (act && k < EF) ? fc[k] : 0.0;
-    }
+      for (int v = 0; v < NV; ++v) F[v] = fc[v * NF];
 #pragma unroll
-    for (int t = 0; t < NIT; ++t) {
-      const int v = ((i + t * N) / NF) % NV;
-      const uint32_t m = fx_mag(F[t]);
-      if (v == 0)
-        w[0] = max(w[0], m);
-      else if (v == NV - 1)
-        w[2] = max(w[2], m);
-      else
-        w[1] = max(w[1], m);
+      for (int v = 0; v < NV; ++v) {
+        w[fx_group(v, NV)] = max(w[fx_group(v, NV)], fx_mag(F[v]));
+        reinterpret_cast<double*>(sfc)[lf * EF + o + v * NF] = F[v];
+      }
     }
-    fx_group_max<N>(w[0], w[1], w[2], i, act, sec + les * FX_GROUPS);
-    __syncthreads();
-    // the sums move to the larger exponent of fluxes and common fluxes
+    fx_group_max<FQ>(w[0], w[1], w[2], r, in, sec + lf * FX_GROUPS);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < NIT; ++t) {
+    const int k = tid + t * BT;
+    if ((t + 1) * BT <= EPB * FQ || k < EPB * FQ) {
+      const int lf = k / FQ, r = k % FQ, o = lf * EF + (r / NF) * NV * NF + r % NF;
+      int Ec[FX_GROUPS];
+#pragma unroll
+      for (int g = 0; g < FX_GROUPS; ++g)
+        Ec[g] = fx_exp(max(sef[lf * FX_GROUPS + g], sec[lf * FX_GROUPS + g]));
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+        sfc[o + v * NF] = fx_limbs(reinterpret_cast<const double*>(sfc)[o + v * NF], Ec[fx_group(v, NV)]);
+    }
+  }
+  // the sums move to the larger exponent of fluxes and common fluxes
+  {
+    int sh[FX_GROUPS];
 #pragma unroll
     for (int g = 0; g < FX_GROUPS; ++g) {
-      const int Ec = fx_exp(sec[les * FX_GROUPS + g]);
-      if (Ec > E[g]) {
-        const int s = Ec - E[g] < 63 ? Ec - E[g] : 63;
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-          if (fx_group(v, NV) == g) {
-            acc[v].h = fx_sum(acc[v]) >> s;
-            acc[v].m = 0;
-          }
-        E[g] = Ec;
-      }
+      const int Ec = max(E[g], fx_exp(sec[le * FX_GROUPS + g]));
+      sh[g] = min(Ec - E[g], 63);
+      E[g] = Ec;
     }
-    if (act) {
+    if (sh[0] | sh[1] | sh[2]) {
 #pragma unroll
-      for (int t = 0; t < NIT; ++t) {
-        const int k = i + t * N;
-        if (k < EF) {
-          const int v = (k / NF) % NV;
-          sfc[le * EF + k] = fx_limbs(F[t], v == 0 ? E[0] : (v == NV - 1 ? E[2] : E[1]));
-        }
-      }
+      for (int v = 0; v < NV; ++v)
+        if (sh[fx_group(v, NV)]) acc[v] = FxAcc{fx_sum(acc[v]) >> sh[fx_group(v, NV)], 0};
     }
   }
   __syncthreads();
   double out[NV];
-  uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
-  if (act) {
+  {
+    // u_s and u^n of the combination, read here (u_s from the caches) to keep the registers free
+    double unr[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      out[v] = A.us[b0 + v * N];
+      if (A.rk & RK_A) unr[v] = A.un[b0 + v * N];
+    }
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
       int qf, ia;
@@ -333,23 +348,25 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_stage_fx(StageArgs A, const
         fx_mac(acc[v], Fm[(NV + v) * NF], cr);
       }
     }
-    const double cs = sh2[le];
+    const double cs = sh2[le < ne ? le : 0];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const int Ev = E[fx_group(v, NV)];
       const double R = fx_double(fx_sum(acc[v]), fx_unit(Ev, ops.kd), Ev >= FX_E_BAD);
       // the first stage (a = 0, b = 1) is one FMA per value; the tests are uniform over the grid
-      double o = fma(cs, R, (A.rk & RK_B1) ? q[v] : A.b * q[v]);
+      double o = fma(cs, R, (A.rk & RK_B1) ? out[v] : A.b * out[v]);
       if (A.rk & RK_A) o = fma(A.a, unr[v], o);
       out[v] = o;
-      A.out[b0 + v * N] = o;
-      w[fx_group(v, NV)] = max(w[fx_group(v, NV)], fx_mag(o));
     }
+  }
+  if (act) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) A.out[b0 + v * N] = out[v];
   }
   if (A.flags) {
     // the density-gradient indicator of the new state (the same arithmetic as the indicator
     // kernel): eta = 2 max_i |D_xi rho|, flags from the thresholds
-    double* rho = reinterpret_cast<double*>(sfl) + les * N;
+    double* rho = reinterpret_cast<double*>(sfl) + le * N;
     if (act) rho[i] = out[0];
     __syncthreads();
     if (act) {
@@ -372,9 +389,13 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_stage_fx(StageArgs A, const
     }
   }
   if (A.trace_out) {
-    fx_group_max<N>(w[0], w[1], w[2], i, act, seo + les * FX_GROUPS);
+    uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
+#pragma unroll
+    for (int v = 0; v < NV; ++v) w[fx_group(v, NV)] = max(w[fx_group(v, NV)], fx_mag(out[v]));
+    if (!own) w[0] = w[1] = w[2] = 0u;
+    fx_group_max<N>(w[0], w[1], w[2], i, own, seo + le * FX_GROUPS);
     __syncthreads();
-    if (act) {
+    if (own) {
 #pragma unroll
       for (int v = 0; v < NV; ++v)
         sfl[le * EU + v * N + i] = fx_limbs(out[v], fx_exp(seo[le * FX_GROUPS + fx_group(v, NV)]));
@@ -383,9 +404,5 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_stage_fx(StageArgs A, const
     fx_traces<DIM, NP>(sfl, seo, slm, slp, ops.tr.kt, ne, nullptr, static_cast<double*>(A.trace_out) + e0 * EF);
   }
 }
-
-// Resident warps per SM allowed to the element kernel: its blocks are scheduled while the interface
-// kernel they wait for still runs and hold their slots while they wait.
-constexpr int STAGE_F64_MAX_WARPS = 64;
 
 }  // namespace frg
