@@ -20,6 +20,7 @@
 #include "fr_arith.cuh"
 #include "fr_internal.cuh"
 #include "fr_mlp.cuh"
+#include "fr_stage_fx.cuh"
 #include "fr_tc.cuh"
 
 namespace frg {
@@ -56,106 +57,182 @@ __host__ __device__ inline Lay lay(int in) {
   return L;
 }
 
-// features from the FP64 state: the conserved variables are interpolated from the element's own
-// points to the 3 Gauss-Legendre points per axis (I3 = 3 x n Lagrange matrix, as double-word
-// constants), where density and pressure are taken
-struct I3Mat {
-  ff m[3][NPMAX];
+// Lagrange matrix from the element's points to the 3 Gauss-Legendre points per axis, as fixed-point
+// entries (fr_fixed.cuh)
+struct I3Fx {
+  int2 c[3][NPMAX];
 };
+// one axis of the interpolation: three results from the n values at `in` (stride st), as limbs at the
+// scale of the input (entries summing to at most 2^61: results stay below 2^59) or, last, as integers
+// half as large
+template <int NP>
+__device__ __forceinline__ void interp3(const I3Fx& I3, const int2* in, int st, FxAcc (&a)[3]) {
+#pragma unroll
+  for (int s = 0; s < 3; ++s) a[s] = FxAcc{0, 0};
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    const int2 x = in[j * st];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) fx_mac(a[s], x, I3.c[s][j]);
+  }
+}
+__device__ __forceinline__ int2 interp_limbs(const FxAcc& a) {
+  const long long v = (a.h << 1) + ((a.m + (1ll << 29)) >> 30);
+  return make_int2(int(v >> 31), int(uint32_t(v) & 0x7FFFFFFFu));
+}
+// a 58-bit integer as a double-word value (the low 11 bits rounded away)
+__device__ __forceinline__ ff ff_from_fixed(long long v) {
+  v += 1ll << 10;
+  const float hi = __int2float_rn(int(v >> 35)) * 34359738368.f;
+  return ff_fast_two_sum(hi, __int2float_rn(int(uint32_t(v >> 11) & 0xFFFFFFu)) * 2048.f);
+}
 
-// One thread per element, in double-word arithmetic (pairs of floats, ~48-bit significand, on
-// the FP32 pipes; the state converts from FP64 by integer operations): the features are relative
-// deviations of nearly equal values, which FP32 alone would swamp with rounding noise, while FP64
-// on GB300 runs at 1/58 of the FP32 rate.  The interpolation to the 3^dim sample points is
-// sum-factorised (one axis at a time: n^dim -> 3 n^(dim-1) -> ... -> 3^dim values per variable);
-// density is kept per sample point, the squared momentum accumulated, and pressure formed when
-// the energy arrives.  In 3D the first two axes are done per z-slice, so only 3^2 n values stay
-// live.
+// quotient from one float reciprocal r: a.h r, then the exact residual's quotient, twice (each leaves the
+// 2^-23 of r), with relative error ~2^-47; a third of the instructions of the general quotient
+__device__ __forceinline__ ff ff_div(ff a, ff b) {
+  const float r = __fdividef(1.f, b.h);
+  const float q1 = a.h * r;
+  const float e1 = fmaf(-q1, b.h, a.h), t1 = fmaf(-q1, b.l, a.l);
+  const float q2 = (e1 + t1) * r;
+  const float q3 = (fmaf(-q2, b.h, e1) + fmaf(-q2, b.l, t1)) * r;
+  return ff_fast_two_sum(q1, q2 + q3);
+}
+
+// Features.  Blocks of 128 threads and EPB elements (a multiple of the four warps): the state is staged
+// in shared memory as fixed-point limbs and interpolated to the 3^dim sample points axis by axis
+// (n^dim -> 3 n^(dim-1) -> ... -> 3^dim values per variable), each item three results from one line; then
+// one warp per element takes a sample per lane.  The features are relative deviations of nearly equal
+// values: those of the density are differences of integers, rounded once; the pressure is formed in
+// double-word arithmetic (~48 bits; FP64 on GB300 runs at 1/58 of the FP32 rate).
+constexpr int FT_T = 128;
 template <int DIM, int NP>
-__global__ void __launch_bounds__(128) k_features(const double* __restrict__ u, const uint64_t* __restrict__ keys,
-                                                  int64_t M, KG g, int Dbase, double gamma,
-                                                  const __grid_constant__ I3Mat I3, __nv_bfloat16* __restrict__ X) {
-  constexpr int N = DIM == 2 ? NP * NP : NP * NP * NP;
-  constexpr int NZ = DIM == 2 ? 1 : NP;  // z-slices
-  constexpr int S = DIM == 2 ? 9 : 27;   // sample points, t = s0 + 3 s1 (+ 9 s2)
-  constexpr int NV = DIM + 2, IN = 2 * S + 1;
-  int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= M) return;
-  const double* q = u + e * NV * N;
-  const ff gm1 = ff_from_double(gamma - 1.0), half = {0.5f, 0.f}, zero = {0.f, 0.f};
-  ff rho[S], ke[S];
+struct FeatBlk {
+  static constexpr int N = Sz<DIM, NP>::N;
+  static constexpr int EPB = N == 8 ? 16 : (N <= 4 ? 32 : (N <= 9 ? 24 : (N <= 16 ? 16 : (N <= 27 ? 8 : 4))));
+  static constexpr int PT = (EPB * N + FT_T - 1) / FT_T;  // points per thread
+};
+template <int DIM, int NP>
+__global__ void __launch_bounds__(FT_T) k_features(const double* __restrict__ u, const uint64_t* __restrict__ keys,
+                                                   int64_t M, KG g, int Dbase, const __grid_constant__ I3Fx I3,
+                                                   __nv_bfloat16* __restrict__ X) {
+  using Z = Sz<DIM, NP>;
+  constexpr int N = Z::N, NV = Z::NV, EPB = FeatBlk<DIM, NP>::EPB, PT = FeatBlk<DIM, NP>::PT, BT = FT_T;
+  constexpr int NZ = DIM == 2 ? 1 : NP;        // z-slices
+  constexpr int S = DIM == 2 ? 9 : 27;         // sample points, t = s0 + 3 s1 (+ 9 s2)
+  constexpr int IN = 2 * S + 1, L = N / NP;    // lines along x
+  constexpr int AS = N > 9 * NZ ? N : 9 * NZ, BS = 3 * L > S ? 3 * L : S;
+  __shared__ int2 sa[EPB * NV * AS];
+  __shared__ long long sb[EPB * NV * BS];
+  __shared__ uint32_t se[EPB * FX_GROUPS];
+  const int tid = threadIdx.x;
+  const int64_t e0 = int64_t(blockIdx.x) * EPB;
+  const int ne = int((M - e0) < EPB ? (M - e0) : EPB);
+  for (int k = tid; k < EPB * FX_GROUPS; k += BT) se[k] = 0u;
+  __syncthreads();
+  {
+    double q[PT][NV];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    // b[i2][s1][s0] = sum_i1 I[s1][i1] sum_i0 I[s0][i0] q[i2][i1][i0]
-    ff b[NZ][3][3];
+    for (int p = 0; p < PT; ++p) {
+      const int k = tid + p * BT, le = k / N, i = k % N;
 #pragma unroll
-    for (int i2 = 0; i2 < NZ; ++i2) {
-      ff a[NP][3];
-#pragma unroll
-      for (int i1 = 0; i1 < NP; ++i1) {
-        ff x[NP];
-#pragma unroll
-        for (int i0 = 0; i0 < NP; ++i0) x[i0] = ff_from_double(q[v * N + (i2 * NP + i1) * NP + i0]);
-#pragma unroll
-        for (int s0 = 0; s0 < 3; ++s0) {
-          ff acc = zero;
-#pragma unroll
-          for (int i0 = 0; i0 < NP; ++i0) acc = fma_t(I3.m[s0][i0], x[i0], acc);
-          a[i1][s0] = acc;
-        }
-      }
-#pragma unroll
-      for (int s1 = 0; s1 < 3; ++s1)
-#pragma unroll
-        for (int s0 = 0; s0 < 3; ++s0) {
-          ff acc = zero;
-#pragma unroll
-          for (int i1 = 0; i1 < NP; ++i1) acc = fma_t(I3.m[s1][i1], a[i1][s0], acc);
-          b[i2][s1][s0] = acc;
-        }
+      for (int v = 0; v < NV; ++v) q[p][v] = le < ne ? u[((e0 + le) * NV + v) * N + i] : 0.0;
     }
 #pragma unroll
-    for (int t = 0; t < S; ++t) {
-      const int s0 = t % 3, s1 = (t / 3) % 3, s2 = t / 9;
-      ff c;
-      if (DIM == 2) {
-        c = b[0][s1][s0];
-      } else {
-        c = zero;
+    for (int p = 0; p < PT; ++p) {
+      const int k = tid + p * BT, le = k / N, i = k % N;
+      uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
 #pragma unroll
-        for (int i2 = 0; i2 < NZ; ++i2) c = fma_t(I3.m[s2][i2], b[i2][s1][s0], c);
-      }
-      if (v == 0) {
-        rho[t] = c;
-        ke[t] = zero;
-      } else if (v < NV - 1) {
-        ke[t] = fma_t(c, c, ke[t]);
-      } else {
-        ke[t] = gm1 * (c - half * ke[t] / rho[t]);  // pressure
+      for (int v = 0; v < NV; ++v) w[fx_group(v, NV)] = max(w[fx_group(v, NV)], fx_mag(q[p][v]));
+      fx_group_max<N>(w[0], w[1], w[2], i, le < ne, se + (le < ne ? le : 0) * FX_GROUPS);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < PT; ++p) {
+      const int k = tid + p * BT, le = k / N, i = k % N;
+      if (le >= ne) continue;
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+        sa[(le * NV + v) * AS + i] = fx_limbs(q[p][v], fx_exp(se[le * FX_GROUPS + fx_group(v, NV)]));
+    }
+  }
+  __syncthreads();
+  FxAcc a[3];
+  int2* sbl = reinterpret_cast<int2*>(sb);
+  // along x: b[line][s0]
+  for (int k = tid; k < ne * NV * L; k += BT) {
+    const int r = k / L, l = k % L;
+    interp3<NP>(I3, sa + r * AS + l * NP, 1, a);
+#pragma unroll
+    for (int s = 0; s < 3; ++s) sbl[r * BS + l * 3 + s] = interp_limbs(a[s]);
+  }
+  __syncthreads();
+  // along y: a[i2][s1][s0], in 2D the samples
+  for (int k = tid; k < ne * NV * NZ * 3; k += BT) {
+    const int r = k / (NZ * 3), i2 = (k / 3) % NZ, s0 = k % 3;
+    interp3<NP>(I3, sbl + r * BS + i2 * NP * 3 + s0, 3, a);
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+      if (DIM == 2)
+        reinterpret_cast<long long*>(sa)[r * AS + s * 3 + s0] = fx_sum(a[s]);
+      else
+        sa[r * AS + i2 * 9 + s * 3 + s0] = interp_limbs(a[s]);
+    }
+  }
+  __syncthreads();
+  const long long* sv = reinterpret_cast<const long long*>(sa);
+  int VS = AS;
+  if (DIM == 3) {
+    // along z: the samples
+    for (int k = tid; k < ne * NV * 9; k += BT) {
+      const int r = k / 9, s01 = k % 9;
+      interp3<NP>(I3, sa + r * AS + s01, 9, a);
+#pragma unroll
+      for (int s = 0; s < 3; ++s) sb[r * BS + s * 9 + s01] = fx_sum(a[s]);
+    }
+    __syncthreads();
+    sv = sb;
+    VS = BS;
+  }
+  const int lane = tid & 31, t = lane < S ? lane : S - 1;
+  for (int l = tid >> 5; l < ne; l += BT / 32) {
+    const uint32_t* ge = se + l * FX_GROUPS;
+    const bool badr = ge[0] >= FX_E_BAD, badp = badr || ge[1] >= FX_E_BAD || ge[2] >= FX_E_BAD;
+    const long long* H = sv + l * NV * VS + t;
+    // density: S q_t - sum over the sum, both exact integers (27 2^58 < 2^63)
+    const long long hr = H[0];
+    long long sr = lane < S ? hr : 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sr += __shfl_xor_sync(~0u, sr, o);
+    // pressure over (gamma - 1) in units of the energy: e - |m|^2 / (2 rho), the squared momentum's
+    // unit over those of density and energy being 2^(2 Em - Er - Ee)
+    ff m2 = {0.f, 0.f};
+#pragma unroll
+    for (int b = 0; b < DIM; ++b) {
+      const ff m = ff_from_fixed(H[(1 + b) * VS]);
+      m2 = fma_t(m, m, m2);
+    }
+    int k = 2 * fx_exp(ge[1]) - fx_exp(ge[0]) - fx_exp(ge[2]) - 1;
+    k = k < -126 ? -126 : (k > 127 ? 127 : k);
+    const float sc = __int_as_float((k + 127) << 23);
+    const ff ke = ff_div(m2, ff_from_fixed(hr));
+    const ff p = ff_from_fixed(H[(NV - 1) * VS]) - ff{ke.h * sc, ke.l * sc};
+    ff ps = lane < S ? p : ff{0.f, 0.f};
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      ps = ps + ff{__shfl_xor_sync(~0u, ps.h, o), __shfl_xor_sync(~0u, ps.l, o)};
+    // 100 (p_t - mean) / mean = (S p_t - sum) 100 / sum
+    const ff dp = ff{float(S), 0.f} * p - ps;
+    const float nan = __int_as_float(0x7FC00000);
+    if (lane < S) {
+      __nv_bfloat16* x = X + (e0 + l) * IN;
+      x[t] = __float2bfloat16_rn(badr ? nan : __ll2float_rn(S * hr - sr) * (100.f / __ll2float_rn(sr)));
+      x[S + t] = __float2bfloat16_rn(badp ? nan : (dp.h + dp.l) * (100.f / ps.h));
+      if (t == 0) {
+        const int span = g.Dmax - Dbase > 0 ? g.Dmax - Dbase : 1;
+        x[2 * S] = __float2bfloat16_rn(float(g.depth(keys[e0 + l]) - Dbase) / float(span));
       }
     }
   }
-  ff rm = zero, pm = zero;
-#pragma unroll
-  for (int t = 0; t < S; ++t) {
-    rm = rm + rho[t];
-    pm = pm + ke[t];
-  }
-  // 100 (q_t - mean) / mean = (q_t - mean) * (100 S / sum)
-  const ff hs = ff_from_double(100.0 * S);
-  const ff fr_ = hs / rm, fp_ = hs / pm;
-  const ff inv_s = ff_from_double(1.0 / S);
-  rm = rm * inv_s;
-  pm = pm * inv_s;
-  __nv_bfloat16* x = X + e * IN;
-#pragma unroll
-  for (int t = 0; t < S; ++t) {
-    const ff dr = (rho[t] - rm) * fr_, dp = (ke[t] - pm) * fp_;
-    x[t] = __float2bfloat16_rn(dr.h + dr.l);
-    x[S + t] = __float2bfloat16_rn(dp.h + dp.l);
-  }
-  int span = g.Dmax - Dbase > 0 ? g.Dmax - Dbase : 1;
-  x[2 * S] = __float2bfloat16_rn(float(g.depth(keys[e]) - Dbase) / float(span));
 }
 
 // Tensor-core forward.  Each block keeps the four weight matrices in shared memory as BF16 in the
@@ -713,21 +790,30 @@ int mlp_in_dim(int dim) { return 2 * (dim == 2 ? 9 : 27) + 1; }
 int mlp_features(int dim, int p, const double* u, const uint64_t* keys, int64_t M, const KG& g,
                  int Dbase, double gamma, const DevOps& ops, void* d_X, cudaStream_t s, Err* err) {
   if (M <= 0) return 0;
+  (void)gamma;  // the features are relative: gamma - 1 cancels
   // Lagrange basis of the element's points evaluated at the 3-point Gauss-Legendre nodes
-  I3Mat I3{};
+  I3Fx I3{};
   const double g3[3] = {-std::sqrt(0.6), 0.0, std::sqrt(0.6)};
-  int np = p + 1;
-  for (int t = 0; t < 3; ++t)
+  const int np = p + 1;
+  double c[3][NPMAX], sum = 0.0;
+  for (int t = 0; t < 3; ++t) {
+    double st = 0.0;
     for (int j = 0; j < np; ++j) {
       double pr = 1.0;
       for (int k = 0; k < np; ++k)
         if (k != j) pr *= (g3[t] - ops.x[k]) / (ops.x[j] - ops.x[k]);
-      const float h = float(pr);  // double-word constant: hi + lo
-      I3.m[t][j] = ff{h, float(pr - double(h))};
+      c[t][j] = pr;
+      st += std::fabs(pr);
     }
-  unsigned nb = unsigned((M + 127) / 128);
+    sum = st > sum ? st : sum;
+  }
+  const int kI = fx_scale(sum);
+  for (int t = 0; t < 3; ++t)
+    for (int j = 0; j < np; ++j) I3.c[t][j] = fx_coef(c[t][j], kI);
   __nv_bfloat16* X = static_cast<__nv_bfloat16*>(d_X);
-#define FEAT(D_, N_) k_features<D_, N_><<<nb, 128, 0, s>>>(u, keys, M, g, Dbase, gamma, I3, X)
+#define FEAT(D_, N_)                                                                                        \
+  k_features<D_, N_><<<unsigned((M + FeatBlk<D_, N_>::EPB - 1) / FeatBlk<D_, N_>::EPB), FT_T, 0, s>>>(u, keys, M, g, \
+                                                                                                       Dbase, I3, X)
   if (dim == 2) {
     if (np == 2) FEAT(2, 2); else if (np == 3) FEAT(2, 3); else if (np == 4) FEAT(2, 4); else FEAT(2, 5);
   } else {
