@@ -187,7 +187,9 @@ const char* fr_last_error(const fr_mesh* m);
    pressure give 100*(rho_i - mean rho)/mean rho and 100*(p_i - mean p)/mean p, then
    (D - Dbase)/max(1, Dmax - Dbase).
    Labels are classes -1/0/+1 (coarsen/keep/refine), int8.  class_w = {w_coarsen, w_keep, w_refine,
-   1/sum_batch w_label}: the loss is sum_b w_b CE_b * class_w[3] (weighted mean cross-entropy).
+   1/sum_batch w_label}: the loss is sum_b w_b CE_b * class_w[3] (weighted mean cross-entropy); with
+   class_w[3] = 0 the library forms that factor from the batch's labels (FR_EINVAL if it is infinite).
+   Labels outside -1..1 give FR_EINVAL and leave the parameters as they are.
    fr_mlp_train_step performs one Adam step (beta 0.9/0.999, eps 1e-8; d_m, d_v the moment arrays,
    step counts from 0) in place on d_params; d_loss (device, may be NULL) receives the batch loss.
    fr_mlp_grad returns the gradient of that loss instead.  Device pointers throughout; 1 <= IN <= 64

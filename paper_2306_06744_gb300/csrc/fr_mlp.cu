@@ -459,29 +459,32 @@ __global__ void __launch_bounds__(TC_ROWS) k_mlp_forward_tc(const float* __restr
 // end of the batch get dZ = 0.  At the end the block writes its partial gradient and loss; a
 // second kernel sums the blocks' partials in block order (deterministic).  Waits are bounded as
 // in inference (status word, drain, free).
-constexpr int TG_ROWS = 128, TG_TMEM_COLS = 512;
+constexpr int TG_ROWS = 128, TG_T = 512, TG_TMEM_COLS = 512;
 constexpr int TG_W1 = 0, TG_W2 = 8192, TG_W3 = 16384, TG_W4 = 24576, TG_W2T = 26624, TG_W3T = 34816,
               TG_W4T = 43008, TG_DZT = 45056, TG_A0 = 61440, TG_AT0 = 126976, TG_DZ = 192512,
               TG_BIAS = 208896, TG_MBAR = TG_BIAS + 208 * 4, TG_SMEM = TG_MBAR + 16 + 1024;
 // DZT is followed by A0, which the M = 128 weight-gradient products read as rows 64..127 of their
 // A operand: those rows only reach rows 64..127 of the accumulators, which are never read
 
-__global__ void __launch_bounds__(TG_ROWS) k_mlp_grad_tc(const float* __restrict__ P, int in,
-                                                         const __nv_bfloat16* __restrict__ X,
-                                                         const int8_t* __restrict__ y, int64_t B, float cw0,
-                                                         float cw1, float cw2, float inv_wsum,
-                                                         float* __restrict__ Gp, float* __restrict__ Lp,
-                                                         int* __restrict__ status) {
+__global__ void __launch_bounds__(TG_T) k_mlp_grad_tc(const float* __restrict__ P, int in,
+                                                      const __nv_bfloat16* __restrict__ X,
+                                                      const int8_t* __restrict__ y, int64_t B, float cw0,
+                                                      float cw1, float cw2, float* __restrict__ Gp,
+                                                      float* __restrict__ Lp, int* __restrict__ Cp,
+                                                      int* __restrict__ status) {
   extern __shared__ unsigned char sm_raw[];
   unsigned char* sm = sm_raw + ((1024 - (tc::smem_addr(sm_raw) & 1023)) & 1023);
-  const int t = threadIdx.x, warp = t >> 5;
+  __shared__ int s_cnt[4];
+  // thread t: row `row` of the tile (its warp's tensor-memory quarter), columns c0 .. c0 + 15
+  const int t = threadIdx.x, warp = t >> 5, row = (warp & 3) * 32 + (t & 31), c0 = (warp >> 2) * 16;
   const Lay L = lay(in);
   const int K1 = in <= 32 ? 32 : 64;
   auto put = [&](int off, uint32_t o, float v) {
     *reinterpret_cast<__nv_bfloat16*>(sm + off + o) = __float2bfloat16_rn(v);
   };
+  if (t < 4) s_cnt[t] = 0;
   // weights (BF16, zero padding) and their transposes for the backward products
-  for (int idx = t; idx < H * 64; idx += TG_ROWS) {
+  for (int idx = t; idx < H * 64; idx += TG_T) {
     const int o = idx >> 6, k = idx & 63;
     put(TG_W1, tc::canon_off(o, k), k < in ? P[L.oW1 + o * in + k] : 0.f);
     const float w2 = P[L.oW2 + o * H + k], w3 = P[L.oW3 + o * H + k];
@@ -496,10 +499,10 @@ __global__ void __launch_bounds__(TG_ROWS) k_mlp_grad_tc(const float* __restrict
     }
   }
   float* sb = reinterpret_cast<float*>(sm + TG_BIAS);
-  for (int i = t; i < H; i += TG_ROWS) {
-    sb[i] = bf16r(P[L.ob1 + i]);
-    sb[H + i] = bf16r(P[L.ob2 + i]);
-    sb[2 * H + i] = bf16r(P[L.ob3 + i]);
+  if (t < H) {
+    sb[t] = bf16r(P[L.ob1 + t]);
+    sb[H + t] = bf16r(P[L.ob2 + t]);
+    sb[2 * H + t] = bf16r(P[L.ob3 + t]);
   }
   if (t < 16) sb[3 * H + t] = t < NOUT ? bf16r(P[L.ob4 + t]) : 0.f;
   const uint32_t mb = tc::smem_addr(sm + TG_MBAR);
@@ -510,7 +513,7 @@ __global__ void __launch_bounds__(TG_ROWS) k_mlp_grad_tc(const float* __restrict
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm + TG_MBAR + 8);
-  const uint32_t tlane = tmem + (uint32_t(warp * 32) << 16);
+  const uint32_t tlane = tmem + (uint32_t((warp & 3) * 32) << 16);
   const uint32_t ACC1 = 0, ACC2 = 64, DW[4] = {128, 192, 256, 320};  // tensor-memory columns
   const uint32_t sa = tc::smem_addr(sm);
   auto aof = [](int l) { return TG_A0 + l * 16384; };
@@ -546,11 +549,21 @@ __global__ void __launch_bounds__(TG_ROWS) k_mlp_grad_tc(const float* __restrict
   const int64_t ntiles = (B + TG_ROWS - 1) / TG_ROWS;
   float loss = 0.f, db[4] = {0.f, 0.f, 0.f, 0.f};  // thread o: bias gradient o of each layer
   bool first = true;
-  // thread t's row of dZ (FP32) -> DZ (row t) and DZT (column t), BF16; ncol columns
-  auto put_dz = [&](int c, float v) {
-    put(TG_DZ, tc::canon_off(t, c), v);
-    put(TG_DZT, tc::canon_off_w(c, t, 128), v);
+  // 16 columns of this thread's row, BF16: two 16-byte stores into the row tile, and one column of the
+  // transposed tile
+  auto put_row = [&](int rows, int cols, const float (&v)[16]) {
+    uint32_t pk[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const __nv_bfloat162 h2 = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+      pk[j] = *reinterpret_cast<const uint32_t*>(&h2);
+      *reinterpret_cast<__nv_bfloat16*>(sm + cols + tc::canon_off_w(c0 + 2 * j, row, 128)) = h2.x;
+      *reinterpret_cast<__nv_bfloat16*>(sm + cols + tc::canon_off_w(c0 + 2 * j + 1, row, 128)) = h2.y;
+    }
+    *reinterpret_cast<uint4*>(sm + rows + tc::canon_off(row, c0)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    *reinterpret_cast<uint4*>(sm + rows + tc::canon_off(row, c0 + 8)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
   };
+  int cnt[4] = {0, 0, 0, 0};  // labels of each class, and labels outside -1..1
   auto sum_dzt_row = [&](int o) {  // fixed-order sum over the 128 samples of row o of DZT
     float acc = 0.f;
     for (int j = 0; j < TG_ROWS; j += 8) {
@@ -568,18 +581,19 @@ __global__ void __launch_bounds__(TG_ROWS) k_mlp_grad_tc(const float* __restrict
   for (int64_t tile = blockIdx.x; tile < ntiles && !failed; tile += gridDim.x) {
     const int64_t row0 = tile * TG_ROWS;
     const int nrow = int(B - row0 < TG_ROWS ? B - row0 : TG_ROWS);
-    const bool valid = t < nrow;
+    const bool valid = row < nrow;
     // features: coalesced reads of the tile's contiguous rows into A0 and AT0, zero padding
     const __nv_bfloat16* xs = X + row0 * in;
-    for (int idx = t; idx < TG_ROWS * in; idx += TG_ROWS) {
+    for (int idx = t; idx < TG_ROWS * in; idx += TG_T) {
       const int r = idx / in, k = idx - r * in;
       const __nv_bfloat16 v = r < nrow ? xs[idx] : __float2bfloat16_rn(0.f);
       *reinterpret_cast<__nv_bfloat16*>(sm + aof(0) + tc::canon_off(r, k)) = v;
       *reinterpret_cast<__nv_bfloat16*>(sm + atof(0) + tc::canon_off_w(k, r, 128)) = v;
     }
-    for (int k = in; k < 64; ++k) {
-      if (k < K1) put(aof(0), tc::canon_off(t, k), 0.f);
-      put(atof(0), tc::canon_off_w(k, t, 128), 0.f);
+    for (int idx = t; idx < TG_ROWS * (64 - in); idx += TG_T) {
+      const int r = idx & (TG_ROWS - 1), k = in + idx / TG_ROWS;
+      if (k < K1) put(aof(0), tc::canon_off(r, k), 0.f);
+      put(atof(0), tc::canon_off_w(k, r, 128), 0.f);
     }
     // forward: layers 1..3 into A_l / AT_l, layer 4 to logits
     for (int l = 0; l < 3 && !failed; ++l) {
@@ -588,46 +602,46 @@ __global__ void __launch_bounds__(TG_ROWS) k_mlp_grad_tc(const float* __restrict
         failed = true;
         break;
       }
-      const float* bl = sb + H * l;
+      const float* bl = sb + H * l + c0;
+      uint32_t r[16];
+      tc::tmem_ld16(tlane + ACC1 + uint32_t(c0), r);
+      tc::tmem_wait_ld();
+      float a[16];
 #pragma unroll
-      for (int c0 = 0; c0 < H; c0 += 16) {
-        uint32_t r[16];
-        tc::tmem_ld16(tlane + ACC1 + uint32_t(c0), r);
-        tc::tmem_wait_ld();
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float a = gelu(__uint_as_float(r[j]) + bl[c0 + j]);
-          put(aof(l + 1), tc::canon_off(t, c0 + j), a);
-          put(atof(l + 1), tc::canon_off_w(c0 + j, t, 128), a);
-        }
-      }
+      for (int j = 0; j < 16; ++j) a[j] = gelu(__uint_as_float(r[j]) + bl[j]);
+      put_row(aof(l + 1), atof(l + 1), a);
     }
     if (failed) break;
     if (!sync_issue_wait([&] { mma(ACC1, aof(3), tc::SBO, TG_W4, tc::SBO, H / 16, 16, false); })) {
       failed = true;
       break;
     }
-    {
+    if (warp < 4) {
       uint32_t r[16];
       tc::tmem_ld16(tlane + ACC1, r);
       tc::tmem_wait_ld();
       float dz[NOUT] = {0.f, 0.f, 0.f};
-      if (valid) {
+      const int cls = valid ? int(y[row0 + row]) + 1 : 0;
+      if (valid && (cls < 0 || cls >= NOUT)) ++cnt[3];
+      if (valid && cls >= 0 && cls < NOUT) {
         float o[NOUT];
 #pragma unroll
         for (int c = 0; c < NOUT; ++c) o[c] = __uint_as_float(r[c]) + sb[3 * H + c];
-        const int cls = int(y[row0 + t]) + 1;
         const float w = cls == 0 ? cw0 : (cls == 1 ? cw1 : cw2);
         const float mx = fmaxf(o[0], fmaxf(o[1], o[2]));
         const float e0 = expf(o[0] - mx), e1 = expf(o[1] - mx), e2 = expf(o[2] - mx);
         const float sum = e0 + e1 + e2;
         const float pz[NOUT] = {e0 / sum, e1 / sum, e2 / sum};
-        loss += -w * inv_wsum * logf(pz[cls]);
+        // unnormalised: the batch's total weight divides the sums in the reduction
+        loss += -w * logf(cls == 0 ? pz[0] : (cls == 1 ? pz[1] : pz[2]));
 #pragma unroll
-        for (int c = 0; c < NOUT; ++c) dz[c] = w * inv_wsum * (pz[c] - (c == cls ? 1.f : 0.f));
+        for (int c = 0; c < NOUT; ++c) {
+          dz[c] = w * (pz[c] - (c == cls ? 1.f : 0.f));
+          cnt[c] += c == cls;
+        }
       }
-      for (int c = 0; c < 16; ++c) put(TG_DZ, tc::canon_off(t, c), c < NOUT ? dz[c] : 0.f);
-      for (int c = 0; c < NOUT; ++c) put(TG_DZT, tc::canon_off_w(c, t, 128), dz[c]);
+      for (int c = 0; c < 16; ++c) put(TG_DZ, tc::canon_off(row, c), c < NOUT ? dz[c] : 0.f);
+      for (int c = 0; c < NOUT; ++c) put(TG_DZT, tc::canon_off_w(c, row, 128), dz[c]);
     }
     // backward: l = 3 (output layer's weights) down to 0
     for (int l = 3; l >= 0 && !failed; --l) {
@@ -651,19 +665,16 @@ __global__ void __launch_bounds__(TG_ROWS) k_mlp_grad_tc(const float* __restrict
       if (l == 0) break;
       __syncthreads();  // every row of DZT summed before it is overwritten
       // dZ of layer l-1: dA * GELU'(Z + b)
-      const float* bl = sb + H * (l - 1);
+      const float* bl = sb + H * (l - 1) + c0;
+      uint32_t ra[16], rz[16];
+      tc::tmem_ld16(tlane + ACC1 + uint32_t(c0), ra);
+      tc::tmem_ld16(tlane + ACC2 + uint32_t(c0), rz);
+      tc::tmem_wait_ld();
+      float d[16];
 #pragma unroll
-      for (int c0 = 0; c0 < H; c0 += 16) {
-        uint32_t ra[16], rz[16];
-        tc::tmem_ld16(tlane + ACC1 + uint32_t(c0), ra);
-        tc::tmem_ld16(tlane + ACC2 + uint32_t(c0), rz);
-        tc::tmem_wait_ld();
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float d = valid ? __uint_as_float(ra[j]) * gelu_d(__uint_as_float(rz[j]) + bl[c0 + j]) : 0.f;
-          put_dz(c0 + j, d);
-        }
-      }
+      for (int j = 0; j < 16; ++j)
+        d[j] = valid ? __uint_as_float(ra[j]) * gelu_d(__uint_as_float(rz[j]) + bl[j]) : 0.f;
+      put_row(TG_DZ, TG_DZT, d);
     }
     first = false;
   }
@@ -674,24 +685,22 @@ __global__ void __launch_bounds__(TG_ROWS) k_mlp_grad_tc(const float* __restrict
   __syncthreads();
   // the block's partial gradient in the parameter layout, and its loss
   float* g = Gp + int64_t(blockIdx.x) * L.total;
-  if (warp < 2) {  // rows 0..63 of the weight-gradient accumulators (tensor-memory lanes 0..63)
+  if ((warp & 3) < 2) {  // rows 0..63 of the weight-gradient accumulators (tensor-memory lanes 0..63)
     tc::fence_after_sync();
     for (int l = 0; l < 4; ++l) {
       const int nin = l == 0 ? in : H, ow = l == 0 ? L.oW1 : l == 1 ? L.oW2 : l == 2 ? L.oW3 : L.oW4;
       const int nout = l == 3 ? NOUT : H;
+      uint32_t r[16];
+      tc::tmem_ld16(tlane + DW[l] + uint32_t(c0), r);
+      tc::tmem_wait_ld();
+      if (row < nout && !first)
 #pragma unroll
-      for (int c0 = 0; c0 < H; c0 += 16) {
-        uint32_t r[16];
-        tc::tmem_ld16(tlane + DW[l] + uint32_t(c0), r);
-        tc::tmem_wait_ld();
-        if (t < nout && !first)
-          for (int j = 0; j < 16; ++j)
-            if (c0 + j < nin) g[ow + t * nin + c0 + j] = __uint_as_float(r[j]);
-      }
+        for (int j = 0; j < 16; ++j)
+          if (c0 + j < nin) g[ow + row * nin + c0 + j] = __uint_as_float(r[j]);
     }
   }
   if (first) {  // a block without tiles contributes zeros
-    for (int k = t; k < L.total; k += TG_ROWS) g[k] = 0.f;
+    for (int k = t; k < L.total; k += TG_T) g[k] = 0.f;
   } else {
     if (t < H) {
       g[L.ob1 + t] = db[0];
@@ -700,14 +709,20 @@ __global__ void __launch_bounds__(TG_ROWS) k_mlp_grad_tc(const float* __restrict
     }
     if (t < NOUT) g[L.ob4 + t] = db[3];
   }
-  // loss: warp sums, then the four warps in order
+  // loss: warp sums, then the four warps that hold it in order; label counts
   float* red = reinterpret_cast<float*>(sm + TG_BIAS);
   __syncthreads();
+  if (warp < 4) {
 #pragma unroll
-  for (int w = 16; w > 0; w >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, w);
-  if ((t & 31) == 0) red[warp] = loss;
+    for (int w = 16; w > 0; w >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, w);
+    if ((t & 31) == 0) red[warp] = loss;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (cnt[c]) atomicAdd(&s_cnt[c], cnt[c]);
+  }
   __syncthreads();
   if (t == 0) Lp[blockIdx.x] = red[0] + red[1] + red[2] + red[3];
+  if (t < 4) Cp[blockIdx.x * 4 + t] = s_cnt[t];
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) {
@@ -716,34 +731,63 @@ __global__ void __launch_bounds__(TG_ROWS) k_mlp_grad_tc(const float* __restrict
   }
 }
 
-// sums of the blocks' partial gradients and losses, in block order
-__global__ void k_grad_reduce(const float* __restrict__ Gp, const float* __restrict__ Lp, int nblk, int total,
-                              float* __restrict__ G, float* __restrict__ loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+// Sums of the blocks' partial gradients and losses (a fixed order), divided by the batch's total class
+// weight (from the exact label counts, unless the caller gives its inverse), then either stored (G) or
+// applied by Adam (Kingma & Ba): m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
+// p -= lr mhat / (sqrt(vhat) + eps).  A wait that gave up in the gradient kernel, a label outside
+// -1..1 (status 2) or a total weight of zero (status 4) leaves everything unchanged.
+struct AdamArgs {
+  float *P, *m, *v;
+  float lr, b1, b2, eps, c1, c2;
+};
+constexpr int RED_T = 64;
+__global__ void __launch_bounds__(RED_T) k_grad_reduce(const float* __restrict__ Gp, const float* __restrict__ Lp,
+                                                       const int* __restrict__ Cp, int nblk, int total, float cw0,
+                                                       float cw1, float cw2, float inv_given, float* __restrict__ G,
+                                                       float* __restrict__ loss, AdamArgs A, int* __restrict__ status) {
+  __shared__ int s_cnt[4];
+  const int t = threadIdx.x, p = blockIdx.x * RED_T + t;
+  if (t < 4) s_cnt[t] = 0;
+  __syncthreads();
+  for (int k = t; k < nblk * 4; k += RED_T) {
+    const int c = Cp[k];
+    if (c) atomicAdd(&s_cnt[k & 3], c);
+  }
+  __syncthreads();
+  const double ws = double(s_cnt[0]) * cw0 + double(s_cnt[1]) * cw1 + double(s_cnt[2]) * cw2;
+  const int bad = s_cnt[3] ? 2 : (inv_given == 0.f && ws == 0.0 ? 4 : 0);
+  if (bad) {
+    if (blockIdx.x == 0 && t == 0) atomicOr(status, bad);
+    return;
+  }
+  if (*status & 1) return;  // set before this kernel only
+  const float inv = inv_given != 0.f ? inv_given : float(1.0 / ws);
   if (p < total) {
-    float a = 0.f;
-    for (int c = 0; c < nblk; ++c) a += Gp[int64_t(c) * total + p];
-    G[p] = a;
+    float a[4] = {0.f, 0.f, 0.f, 0.f};
+    int c = 0;
+#pragma unroll 2
+    for (; c + 4 <= nblk; c += 4)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) a[j] += Gp[int64_t(c + j) * total + p];
+    for (; c < nblk; ++c) a[0] += Gp[int64_t(c) * total + p];
+    const float g = ((a[0] + a[1]) + (a[2] + a[3])) * inv;
+    if (G) {
+      G[p] = g;
+    } else {
+      const float mt = A.b1 * A.m[p] + (1.f - A.b1) * g;
+      const float vt = A.b2 * A.v[p] + (1.f - A.b2) * g * g;
+      A.m[p] = mt;
+      A.v[p] = vt;
+      A.P[p] -= A.lr * (mt / A.c1) / (sqrtf(vt / A.c2) + A.eps);
+    }
   }
-  if (p == 0 && loss) {
+  if (blockIdx.x == 0 && t < 32 && loss) {
     float a = 0.f;
-    for (int c = 0; c < nblk; ++c) a += Lp[c];
-    *loss = a;
+    for (int c = t; c < nblk; c += 32) a += Lp[c];
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) a += __shfl_xor_sync(0xffffffffu, a, w);
+    if (t == 0) *loss = a * inv;
   }
-}
-
-// Adam (Kingma & Ba): m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2, p -= lr mhat / (sqrt(vhat) + eps)
-__global__ void k_adam(float* __restrict__ P, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ G, int n, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  float g = G[t];
-  float mt = b1 * m[t] + (1.f - b1) * g;
-  float vt = b2 * v[t] + (1.f - b2) * g * g;
-  m[t] = mt;
-  v[t] = vt;
-  P[t] -= lr * (mt / c1) / (sqrtf(vt / c2) + eps);
 }
 
 }  // namespace
@@ -824,10 +868,11 @@ int mlp_features(int dim, int p, const double* u, const uint64_t* keys, int64_t 
   return 0;
 }
 
-// gradient (into G, total floats) and loss of one batch on the tensor cores; *d_st (scratch)
-// becomes nonzero if a completion wait gave up
-static int grad_tc(const float* d_params, int in, const void* d_X, const int8_t* d_y, int64_t B,
-                   const float* cw, float* G, float* d_loss, Scratch& S, int** d_st, cudaStream_t s, Err* err) {
+// Gradient and loss of one batch on the tensor cores, stored into G or (G null) applied by Adam.  The
+// label counts that normalise the sums come from the gradient kernel; cw[3] != 0 gives 1 / sum_b w_{y_b}
+// instead.  Synchronises: the status word is read at the end.
+static int grad_step(const float* d_params, int in, const void* d_X, const int8_t* d_y, int64_t B, const float* cw,
+                     float* G, float* d_loss, const AdamArgs& adam, Alloc& A, cudaStream_t s, Err* err) {
   if (B <= 0) return set_error(err, FR_EINVAL, "empty batch");
   if (in < 1 || in > 64) return set_error(err, FR_EINVAL, "the MLP takes 1..64 inputs");
   const Lay L = lay(in);
@@ -836,52 +881,41 @@ static int grad_tc(const float* d_params, int in, const void* d_X, const int8_t*
   FR_CUDA(err, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t ntiles = (B + TG_ROWS - 1) / TG_ROWS;
   const int grid = int(ntiles < sms ? ntiles : sms);  // one block per SM (shared memory, TMEM)
-  float* Gp = S.get<float>(size_t(grid) * L.total);
-  float* Lp = S.get<float>(size_t(grid));
-  int* st = S.get<int>(1);
-  if (!Gp || !Lp || !st) return set_error(err, FR_ENOMEM, "training scratch");
+  // one block of scratch: status word, label counts, losses, partial gradients
+  Scratch S(&A);
+  int* st = S.get<int>(64 + size_t(grid) * (5 + size_t(L.total)));
+  if (!st) return set_error(err, FR_ENOMEM, "training scratch");
+  int* Cp = st + 64;
+  float* Lp = reinterpret_cast<float*>(Cp + size_t(grid) * 4);
+  float* Gp = Lp + grid;
   FR_CUDA(err, cudaMemsetAsync(st, 0, 4, s));
   FR_CUDA(err, cudaFuncSetAttribute(k_mlp_grad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_SMEM));
-  // class weights normalised by the batch's total weight: cw[0..2], and cw[3] = 1 / sum_b w_{y_b}
-  k_mlp_grad_tc<<<unsigned(grid), TG_ROWS, TG_SMEM, s>>>(d_params, in, static_cast<const __nv_bfloat16*>(d_X),
-                                                         d_y, B, cw[0], cw[1], cw[2], cw[3], Gp, Lp, st);
+  k_mlp_grad_tc<<<unsigned(grid), TG_T, TG_SMEM, s>>>(d_params, in, static_cast<const __nv_bfloat16*>(d_X), d_y, B,
+                                                      cw[0], cw[1], cw[2], Gp, Lp, Cp, st);
   FR_LAUNCH_CHECK(err);
-  k_grad_reduce<<<unsigned((L.total + 255) / 256), 256, 0, s>>>(Gp, Lp, grid, L.total, G, d_loss);
+  k_grad_reduce<<<unsigned((L.total + RED_T - 1) / RED_T), RED_T, 0, s>>>(Gp, Lp, Cp, grid, L.total, cw[0], cw[1], cw[2],
+                                                                          cw[3], G, d_loss, adam, st);
   FR_LAUNCH_CHECK(err);
-  *d_st = st;
-  return 0;
-}
-
-static int check_status(const int* d_st, cudaStream_t s, Err* err) {
   int h = 0;
-  FR_CUDA(err, cudaMemcpyAsync(&h, d_st, 4, cudaMemcpyDeviceToHost, s));
+  FR_CUDA(err, cudaMemcpyAsync(&h, st, 4, cudaMemcpyDeviceToHost, s));
   FR_CUDA(err, cudaStreamSynchronize(s));
-  return h ? set_error(err, FR_ETIMEOUT, "a tensor-core completion wait gave up (training)") : 0;
+  if (h & 1) return set_error(err, FR_ETIMEOUT, "a tensor-core completion wait gave up (training)");
+  if (h & 2) return set_error(err, FR_EINVAL, "labels must be -1, 0 or 1");
+  return h ? set_error(err, FR_EINVAL, "the batch's class weights sum to zero") : 0;
 }
 
 int mlp_train_step(float* d_params, float* d_m, float* d_v, int64_t step, int in, const void* d_X,
                    const int8_t* d_y, int64_t B, const float* cw, float lr, float* d_loss,
                    Alloc& A, cudaStream_t s, Err* err) {
-  const Lay L = lay(in);
-  Scratch S(&A);
-  float* G = S.get<float>(L.total);
-  if (!G) return set_error(err, FR_ENOMEM, "training scratch");
-  int* st = nullptr;
-  FR_TRY(grad_tc(d_params, in, d_X, d_y, B, cw, G, d_loss, S, &st, s, err));
   const float b1 = 0.9f, b2 = 0.999f;
-  float c1 = 1.f - std::pow(b1, float(step + 1)), c2 = 1.f - std::pow(b2, float(step + 1));
-  k_adam<<<unsigned((L.total + 255) / 256), 256, 0, s>>>(d_params, d_m, d_v, G, L.total, lr, b1, b2,
-                                                         1e-8f, c1, c2);
-  FR_LAUNCH_CHECK(err);
-  return check_status(st, s, err);
+  const AdamArgs adam{d_params, d_m, d_v, lr, b1, b2, 1e-8f, 1.f - std::pow(b1, float(step + 1)),
+                      1.f - std::pow(b2, float(step + 1))};
+  return grad_step(d_params, in, d_X, d_y, B, cw, nullptr, d_loss, adam, A, s, err);
 }
 
 int mlp_grad(const float* d_params, int in, const void* d_X, const int8_t* d_y, int64_t B,
              const float* cw, float* d_grad, float* d_loss, Alloc& A, cudaStream_t s, Err* err) {
-  Scratch S(&A);
-  int* st = nullptr;
-  FR_TRY(grad_tc(d_params, in, d_X, d_y, B, cw, d_grad, d_loss, S, &st, s, err));
-  return check_status(st, s, err);
+  return grad_step(d_params, in, d_X, d_y, B, cw, d_grad, d_loss, AdamArgs{}, A, s, err);
 }
 
 }  // namespace frg

@@ -388,11 +388,10 @@ def mlp_param_count(in_dim: int) -> int:
     return n
 
 
-def _class_w(cw, y):
+def _class_w(cw):
+    """The C ABI's class_w: three weights, and 0 for the library to normalise by the batch's labels."""
     cw = np.asarray(cw, dtype=np.float64)
-    yy = np.asarray(y.cpu().numpy() if hasattr(y, "cpu") else y, dtype=np.int64) + 1
-    wsum = float(cw[yy].sum())
-    return np.array([cw[0], cw[1], cw[2], 1.0 / wsum], dtype=np.float32)
+    return np.array([cw[0], cw[1], cw[2], 0.0], dtype=np.float32)
 
 
 def mlp_forward(params, X, stream=None):
@@ -417,7 +416,7 @@ def mlp_grad(params, X, y, class_w, stream=None):
     n, n_in = X.shape
     g = torch.empty_like(params)
     loss = torch.empty(1, dtype=torch.float32, device="cuda")
-    cw = _class_w(class_w, y)
+    cw = _class_w(class_w)
     _check(load().fr_mlp_grad(n_in, C.c_void_p(params.data_ptr()), C.c_void_p(X.data_ptr()),
                               C.c_void_p(y.data_ptr()), n, _np_ptr(cw), C.c_void_p(g.data_ptr()),
                               C.c_void_p(loss.data_ptr()), _stream_handle(stream)))
@@ -427,7 +426,7 @@ def mlp_grad(params, X, y, class_w, stream=None):
 def mlp_train_step(params, m, v, step, X, y, class_w, lr, loss=None, stream=None):
     """One Adam step in place on `params` (CUDA FP32); X BF16 [B][in], y int8 in {-1,0,1}."""
     B, n_in = X.shape
-    cw = _class_w(class_w, y)
+    cw = _class_w(class_w)
     _check(load().fr_mlp_train_step(n_in, C.c_void_p(params.data_ptr()), C.c_void_p(m.data_ptr()),
                                     C.c_void_p(v.data_ptr()), step, C.c_void_p(X.data_ptr()),
                                     C.c_void_p(y.data_ptr()), B, _np_ptr(cw), C.c_float(lr),
