@@ -3,6 +3,8 @@
 // mapping and face connectivity.  Every generating step is count -> exclusive scan -> write at
 // the scanned position, so outputs are deterministic and already in Morton order (no atomic
 // counters, no retry on shared-memory overflow).
+#include <algorithm>
+
 #include "fr_internal.cuh"
 
 namespace frg {
@@ -208,12 +210,16 @@ __global__ void k_edit_write(const uint64_t* __restrict__ k, const int8_t* __res
 }
 
 // 2:1 balance pass at depth D (Sec. 3.2, balance algorithm): every depth-D leaf looks up the
-// leaf containing the anchor of each of its 3^dim-1 same-size neighbour boxes (periodic).  A
-// containing leaf A coarser than D-1 is split along the path towards that box down to depth D-1;
-// all 2^dim children of every level on the path are emitted.
+// leaf containing the anchor of its same-size neighbour boxes (periodic).  A containing leaf A
+// coarser than D-1 is split along the path towards that box down to depth D-1; all 2^dim children of
+// every level on the path are emitted.
+// Of the 3^dim-1 neighbour boxes only the 2^dim-1 that lie outside the leaf's parent in a set of axes,
+// each away from the parent's centre, are looked up: the others lie in the parent (whose cells are never
+// coarser than D) or share their depth-(D-1) cell with one of these, so that the leaf containing them
+// and the path to it are the same.  (600k points of a 3D torus, 829k leaves: see k_bal_gen_fast.)
 template <int DIM>
 struct Nofs {
-  static constexpr int value = DIM == 2 ? 8 : 26;
+  static constexpr int value = (1 << DIM) - 1;
 };
 
 template <int DIM>
@@ -222,13 +228,12 @@ __device__ __forceinline__ bool bal_query(const uint64_t* __restrict__ k, int64_
                                           const uint64_t* s_tab = nullptr, int m = 0, int sh = 0) {
   uint64_t key = k[i];
   if (g.depth(key) != D) return false;
-  int oo = o < (DIM == 2 ? 4 : 13) ? o : o + 1;  // skip the centre of the 3^dim stencil
   uint32_t x[3];
   deinterleave<DIM>(g.raw(key), x);
   uint32_t w = g.width(D), mask = (g.Dmax >= 32) ? 0xFFFFFFFFu : ((1u << g.Dmax) - 1u);
   for (int a = 0; a < DIM; ++a) {
-    int off = (oo / (a == 0 ? 1 : (a == 1 ? 3 : 9))) % 3 - 1;
-    N[a] = (x[a] + uint32_t(off) * w) & mask;  // periodic wrap on the 2^Dmax grid
+    const uint32_t step = (x[a] & w) ? w : 0u - w;  // away from the parent's centre
+    N[a] = (x[a] + (((o + 1) >> a) & 1 ? step : 0u)) & mask;  // periodic wrap on the 2^Dmax grid
   }
   int64_t j = bound_indexed<true>(k, n, cell_key<DIM>(g, N), s_tab, m, sh) - 1;
   if (j < 0) j = 0;  // only on an incomplete tree, which callers reject beforehand
@@ -248,13 +253,12 @@ __device__ __forceinline__ int64_t bal_nS(const int64_t* ctl, int64_t cap) {
   return (ctl[CTL_OVER] != 0 || G > cap) ? 0 : G;
 }
 
-// A group of lanes per leaf (8 in 2D, a warp in 3D), one lane per neighbour box of the leaf's
-// 3^dim-1 stencil: the lanes search in parallel and combine by warp shuffles, so the scan that
+// A group of lanes per leaf (4 in 2D, 8 in 3D), one lane per neighbour box looked up: the lanes search in parallel and combine by warp shuffles, so the scan that
 // places the generated octants runs over leaves, not over (leaf, neighbour) pairs.  Lanes past
 // the leaf count (an upper bound of it sizes the grid) contribute zeros.
 template <int DIM>
 struct BalLanes {
-  static constexpr int value = DIM == 2 ? 8 : 32;
+  static constexpr int value = 1 << DIM;
 };
 
 // number of octants lane (i, o) generates, with the containing leaf's depth and the box
@@ -1088,18 +1092,31 @@ __global__ void k_pts_encode(const double* __restrict__ pts, int64_t n, double L
   keys[i] = cell_key<DIM>(g, x);
 }
 
-// greedy decomposition of the raw-ID interval [lo, hi]; emits (raw, depth) when out != null
+// Greedy decomposition of the raw-ID interval [lo, hi): the largest aligned block that fits, again and
+// again, none coarser than Dmin.  Blocks below Dmin's size come at its two ends (at most
+// (2^dim - 1) (Dmax - Dmin) each); between them lies a run of Dmin cells, which may be thousands long
+// and is therefore only reported: its first ID, its length and its place among the blocks.  With out,
+// the other blocks are written.  Returns the count of all.
 template <int DIM>
 __device__ __forceinline__ int64_t gap_blocks(uint64_t lo, uint64_t hi_excl, const KG& g, int Dmin,
-                                              uint64_t* out) {
+                                              uint64_t* out, uint64_t* run_lo, int64_t* run_n, int64_t* run_at) {
   int64_t cnt = 0;
   const int kmax = g.Dmax - Dmin;
+  *run_n = 0;
+  *run_lo = 0;
+  *run_at = 0;
   while (lo < hi_excl) {
-    int k = 0;
-    while (k < kmax) {
-      uint64_t span = 1ull << (DIM * (k + 1));
-      if ((lo & (span - 1)) != 0 || lo + span > hi_excl) break;
-      ++k;
+    const int ka = lo ? (__ffsll((long long)lo) - 1) / DIM : 64;      // alignment
+    const int kf = (63 - __clzll((long long)(hi_excl - lo))) / DIM;  // room
+    const int k = min(min(ka, kf), kmax);
+    if (k == kmax) {
+      const int64_t r = int64_t((hi_excl - lo) >> (DIM * kmax));  // aligned here, so to the end of the run
+      *run_lo = lo;
+      *run_n = r;
+      *run_at = cnt;
+      cnt += r;
+      lo += uint64_t(r) << (DIM * kmax);
+      continue;
     }
     if (out) out[cnt] = g.make(lo, g.Dmax - k);
     ++cnt;
@@ -1125,9 +1142,10 @@ __global__ void k_gap_count(const uint64_t* __restrict__ S, const int64_t* __res
     cnt[t] = 0;
     return;
   }
-  uint64_t lo, hi;
+  uint64_t lo, hi, rl;
+  int64_t rn, ra;
   gap_bounds<DIM>(S, nS, t, g, &lo, &hi);
-  cnt[t] = int32_t(gap_blocks<DIM>(lo, hi, g, Dmin, nullptr) + (t < nS ? 1 : 0));
+  cnt[t] = int32_t(gap_blocks<DIM>(lo, hi, g, Dmin, nullptr, &rl, &rn, &ra) + (t < nS ? 1 : 0));
 }
 
 template <int DIM>
@@ -1135,14 +1153,26 @@ __global__ void k_gap_write(const uint64_t* __restrict__ S, const int64_t* __res
                             int64_t ncap, KG g, int Dmin, const int64_t* __restrict__ offs,
                             uint64_t* __restrict__ out) {
   int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t > ncap) return;
   const int64_t nS = *d_nS;
-  if (t > nS) return;
-  uint64_t lo, hi;
-  gap_bounds<DIM>(S, nS, t, g, &lo, &hi);
-  int64_t o = offs[t];
-  int64_t c = gap_blocks<DIM>(lo, hi, g, Dmin, out + o);
-  if (t < nS) out[o + c] = S[t];
+  uint64_t rl = 0;
+  int64_t rn = 0, ra = 0;
+  if (t <= ncap && t <= nS) {
+    uint64_t lo, hi;
+    gap_bounds<DIM>(S, nS, t, g, &lo, &hi);
+    const int64_t o = offs[t];
+    const int64_t c = gap_blocks<DIM>(lo, hi, g, Dmin, out + o, &rl, &rn, &ra);
+    if (t < nS) out[o + c] = S[t];
+    ra += o;
+  }
+  // the runs of Dmin cells, each by the whole warp (one thread alone would write thousands of cells
+  // while the grid waits for it)
+  const int lane = int(threadIdx.x & 31), kmax = g.Dmax - Dmin;
+  for (unsigned m = __ballot_sync(0xffffffffu, rn > 0); m; m &= m - 1) {
+    const int l = __ffs(m) - 1;
+    const uint64_t lo = __shfl_sync(0xffffffffu, (unsigned long long)rl, l);
+    const int64_t n = __shfl_sync(0xffffffffu, (long long)rn, l), at = __shfl_sync(0xffffffffu, (long long)ra, l);
+    for (int64_t j = lane; j < n; j += 32) out[at + j] = g.make(lo + (uint64_t(j) << (DIM * kmax)), Dmin);
+  }
 }
 
 int read_bad(const int32_t* d_bad, bool* bad, cudaStream_t s, Err* err) {
@@ -1369,9 +1399,11 @@ int tree_balance(int dim, const KG& g, int Dhigh, int Dlow, Buf<uint64_t>& keys,
     }
     Scratch S(&A);
     // one search pass: the octants are placed by an atomic counter (sorted next, so their order
-    // does not matter) into room for max(2^16, 2n) of them; a pass that generates more is counted,
-    // scanned and generated again at exact positions
-    const int64_t capG = 2 * n_ub > (int64_t(1) << 16) ? 2 * n_ub : (int64_t(1) << 16);
+    // does not matter) into room for max(2^16, 2n) of them, up to 8n while that stays below 2^24 (128
+    // MB: the first pass of a tree completed from points asks for about 3n); a pass that generates
+    // more is counted, scanned and generated again at exact positions, which costs two more searches
+    int64_t capG = 2 * n_ub > (int64_t(1) << 16) ? 2 * n_ub : (int64_t(1) << 16);
+    if (capG < (int64_t(1) << 24)) capG = 8 * n_ub < (int64_t(1) << 24) ? std::max(capG, 8 * n_ub) : (int64_t(1) << 24);
     if (gen.ensure(A, size_t(capG)) || cudaMemsetAsync(d_ctl + CTL_G, 0, 8, s) != cudaSuccess) {
       rc = set_error(err, FR_ENOMEM, "balance scratch");
       break;
