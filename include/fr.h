@@ -217,6 +217,13 @@ int fr_mlp_grad(int in_dim, const float* d_params, const void* d_X_bf16, const i
 int fr_mlp_train_step(int in_dim, float* d_params, float* d_m, float* d_v, int64_t step,
                       const void* d_X_bf16, const int8_t* d_y, int64_t B, const float* class_w,
                       float lr, float* d_loss, void* stream);
+/* The same with the call's scratch memory from the caller's allocator (NULL: the stream-ordered pool,
+   which gives its memory back at every synchronisation, so that the next call pays for it again). */
+int fr_mlp_forward_alloc(int in_dim, const float* d_params, const void* d_X_bf16, int64_t n,
+                         float* d_logits, int8_t* d_flags, void* stream, const fr_allocator* alloc);
+int fr_mlp_train_step_alloc(int in_dim, float* d_params, float* d_m, float* d_v, int64_t step,
+                            const void* d_X_bf16, const int8_t* d_y, int64_t B, const float* class_w,
+                            float lr, float* d_loss, void* stream, const fr_allocator* alloc);
 
 /* Measurement.  With profiling on, every interface and element kernel launched by fr_step,
    fr_run and fr_rhs is bracketed by CUDA events on the mesh's stream; fr_profile_read
@@ -283,6 +290,11 @@ int fr_tree_complete(int dim, int Dmin, int Dmax, double L, const double* d_pts,
    coarsest balanced refinement.  Depth passes from Dmax down to 2. */
 int fr_tree_balance(int dim, int Dmax, const uint64_t* d_keys, int64_t n, uint64_t* d_out,
                     int64_t cap, int64_t* n_out, void* stream);
+/* Tree completion and balance with the call's scratch memory from the caller's allocator (may be NULL). */
+int fr_tree_complete_alloc(int dim, int Dmin, int Dmax, double L, const double* d_pts, int64_t n,
+                           uint64_t* d_out, int64_t cap, int64_t* n_out, void* stream, const fr_allocator* alloc);
+int fr_tree_balance_alloc(int dim, int Dmax, const uint64_t* d_keys, int64_t n, uint64_t* d_out,
+                          int64_t cap, int64_t* n_out, void* stream, const fr_allocator* alloc);
 /* Adaptation procedure (Sec. 4.1) with flags int8[n], then 2:1 balance down to depth Dbase+2. */
 int fr_tree_adapt(int dim, int Dbase, int Dmax, const uint64_t* d_keys, const int8_t* d_flags,
                   int64_t n, uint64_t* d_out, int64_t cap, int64_t* n_out, void* stream);

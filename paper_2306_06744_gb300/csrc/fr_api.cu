@@ -759,6 +759,20 @@ KG geo_or_err(int dim, int Dmax, int* rc) {
   return KG{Dmax, depth_bits(Dmax)};
 }
 
+// Device memory of one call of a primitive: blocks released inside the call serve its later requests
+// (a depth pass of the balance asks for the sizes of the one before), and all of them go back to the
+// caller's allocator, or to the stream-ordered pool, when the call ends.
+struct CallAlloc {
+  BlockCache cache;
+  Alloc A;
+  CallAlloc(const fr_allocator* user, cudaStream_t s, Err* err) : A{user, s, err, &cache} {}
+  ~CallAlloc() {
+    auto live = cache.live;  // none but after an error
+    for (auto& b : live) A.put(b.first);
+    A.release_cache();
+  }
+};
+
 }  // namespace
 
 // =============================================================================================
@@ -1062,12 +1076,12 @@ int fr_set_learned_indicator(fr_mesh* m, const float* host_params, int64_t n) {
   return 0;
 }
 
-int fr_mlp_forward(int in_dim, const float* d_params, const void* d_X, int64_t n, float* d_logits,
-                   int8_t* d_flags, void* stream) {
+int fr_mlp_forward_alloc(int in_dim, const float* d_params, const void* d_X, int64_t n, float* d_logits,
+                         int8_t* d_flags, void* stream, const fr_allocator* alloc) {
   if (in_dim < 1 || in_dim > 64 || n < 0) return set_error(global_err(), FR_EINVAL, "bad arguments");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  Alloc A{nullptr, s, global_err()};
-  Scratch S(&A);
+  CallAlloc CA(alloc, s, global_err());
+  Scratch S(&CA.A);
   int* st = S.get<int>(1);
   if (!st) return set_error(global_err(), FR_ENOMEM, "scratch");
   FR_CUDA(global_err(), cudaMemsetAsync(st, 0, 4, s));
@@ -1077,6 +1091,11 @@ int fr_mlp_forward(int in_dim, const float* d_params, const void* d_X, int64_t n
   FR_CUDA(global_err(), cudaStreamSynchronize(s));
   if (hs) return set_error(global_err(), FR_ETIMEOUT, "a tensor-core completion wait gave up");
   return 0;
+}
+
+int fr_mlp_forward(int in_dim, const float* d_params, const void* d_X, int64_t n, float* d_logits,
+                   int8_t* d_flags, void* stream) {
+  return fr_mlp_forward_alloc(in_dim, d_params, d_X, n, d_logits, d_flags, stream, nullptr);
 }
 
 void fr_tc_set_wait_limit(long long cycles) { mlp_set_wait_cycles(cycles); }
@@ -1092,16 +1111,20 @@ int fr_mlp_grad(int in_dim, const float* d_params, const void* d_X, const int8_t
   return 0;
 }
 
-int fr_mlp_train_step(int in_dim, float* d_params, float* d_m, float* d_v, int64_t step,
-                      const void* d_X, const int8_t* d_y, int64_t B, const float* class_w, float lr,
-                      float* d_loss, void* stream) {
+int fr_mlp_train_step_alloc(int in_dim, float* d_params, float* d_m, float* d_v, int64_t step, const void* d_X,
+                            const int8_t* d_y, int64_t B, const float* class_w, float lr, float* d_loss,
+                            void* stream, const fr_allocator* alloc) {
   if (in_dim < 1 || in_dim > 64 || B <= 0 || !class_w || step < 0)
     return set_error(global_err(), FR_EINVAL, "bad arguments");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  Alloc A{nullptr, s, global_err()};
-  FR_TRY(mlp_train_step(d_params, d_m, d_v, step, in_dim, d_X, d_y, B, class_w, lr, d_loss, A, s,
-                        global_err()));
-  return 0;
+  CallAlloc CA(alloc, s, global_err());
+  return mlp_train_step(d_params, d_m, d_v, step, in_dim, d_X, d_y, B, class_w, lr, d_loss, CA.A, s, global_err());
+}
+
+int fr_mlp_train_step(int in_dim, float* d_params, float* d_m, float* d_v, int64_t step,
+                      const void* d_X, const int8_t* d_y, int64_t B, const float* class_w, float lr,
+                      float* d_loss, void* stream) {
+  return fr_mlp_train_step_alloc(in_dim, d_params, d_m, d_v, step, d_X, d_y, B, class_w, lr, d_loss, stream, nullptr);
 }
 
 // ---- tree primitives on caller-owned device arrays ----
@@ -1157,14 +1180,16 @@ int fr_keys_linearise(int dim, int Dmax, const uint64_t* d_keys, int64_t n, uint
 }
 
 static int balance_or_adapt(int dim, int Dbase, int Dmax, const uint64_t* d_keys, const int8_t* d_flags,
-                            int64_t n, uint64_t* d_out, int64_t cap, int64_t* n_out, void* stream) {
+                            int64_t n, uint64_t* d_out, int64_t cap, int64_t* n_out, void* stream,
+                            const fr_allocator* alloc) {
   int rc;
   KG g = geo_or_err(dim, Dmax, &rc);
   if (rc) return rc;
   if (n <= 0 || !n_out) return set_error(global_err(), FR_EINVAL, "bad arguments");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   Err* err = global_err();
-  Alloc A{nullptr, s, err};
+  CallAlloc CA(alloc, s, err);
+  Alloc& A = CA.A;
   bool ok = false;
   FR_TRY(tree_validate(dim, g, d_keys, n, 0, Dmax, &ok, A, s, err));
   if (!ok) return set_error(err, FR_EINVAL, "input is not a complete sorted linear tree");
@@ -1192,20 +1217,24 @@ static int balance_or_adapt(int dim, int Dbase, int Dmax, const uint64_t* d_keys
   return rc;
 }
 
+int fr_tree_balance_alloc(int dim, int Dmax, const uint64_t* d_keys, int64_t n, uint64_t* d_out,
+                          int64_t cap, int64_t* n_out, void* stream, const fr_allocator* alloc) {
+  return balance_or_adapt(dim, 0, Dmax, d_keys, nullptr, n, d_out, cap, n_out, stream, alloc);
+}
 int fr_tree_balance(int dim, int Dmax, const uint64_t* d_keys, int64_t n, uint64_t* d_out,
                     int64_t cap, int64_t* n_out, void* stream) {
-  return balance_or_adapt(dim, 0, Dmax, d_keys, nullptr, n, d_out, cap, n_out, stream);
+  return fr_tree_balance_alloc(dim, Dmax, d_keys, n, d_out, cap, n_out, stream, nullptr);
 }
 
 int fr_tree_adapt(int dim, int Dbase, int Dmax, const uint64_t* d_keys, const int8_t* d_flags,
                   int64_t n, uint64_t* d_out, int64_t cap, int64_t* n_out, void* stream) {
   if (!d_flags) return set_error(global_err(), FR_EINVAL, "null flags");
   if (Dbase < 0 || Dbase > Dmax) return set_error(global_err(), FR_EINVAL, "Dbase out of range");
-  return balance_or_adapt(dim, Dbase, Dmax, d_keys, d_flags, n, d_out, cap, n_out, stream);
+  return balance_or_adapt(dim, Dbase, Dmax, d_keys, d_flags, n, d_out, cap, n_out, stream, nullptr);
 }
 
-int fr_tree_complete(int dim, int Dmin, int Dmax, double L, const double* d_pts, int64_t n,
-                     uint64_t* d_out, int64_t cap, int64_t* n_out, void* stream) {
+int fr_tree_complete_alloc(int dim, int Dmin, int Dmax, double L, const double* d_pts, int64_t n,
+                           uint64_t* d_out, int64_t cap, int64_t* n_out, void* stream, const fr_allocator* alloc) {
   int rc;
   KG g = geo_or_err(dim, Dmax, &rc);
   if (rc) return rc;
@@ -1214,7 +1243,8 @@ int fr_tree_complete(int dim, int Dmin, int Dmax, double L, const double* d_pts,
   if (n > (int64_t(1) << 30)) return set_error(global_err(), FR_EINVAL, "too many points");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   Err* err = global_err();
-  Alloc A{nullptr, s, err};
+  CallAlloc CA(alloc, s, err);
+  Alloc& A = CA.A;
   Buf<uint64_t> out;
   int64_t m = 0;
   rc = tree_complete(dim, g, Dmin, L, d_pts, n, out, &m, A, s, err);
@@ -1226,6 +1256,11 @@ int fr_tree_complete(int dim, int Dmin, int Dmax, double L, const double* d_pts,
   out.release(A);
   if (!rc) FR_CUDA(err, cudaStreamSynchronize(s));
   return rc;
+}
+
+int fr_tree_complete(int dim, int Dmin, int Dmax, double L, const double* d_pts, int64_t n,
+                     uint64_t* d_out, int64_t cap, int64_t* n_out, void* stream) {
+  return fr_tree_complete_alloc(dim, Dmin, Dmax, L, d_pts, n, d_out, cap, n_out, stream, nullptr);
 }
 
 int fr_tree_map(int dim, int Dmax, const uint64_t* d_old, int64_t n_old, const uint64_t* d_new,

@@ -77,6 +77,7 @@ EXPORTS = ["fr_mesh_init", "fr_mesh_free", "fr_step", "fr_run", "fr_adapt", "fr_
            "fr_tree_conn", "fr_profile_enable", "fr_profile_read", "fr_kernel_launches",
            "fr_keys_sort_noalloc", "fr_tree_complete", "fr_mlp_param_count", "fr_features",
            "fr_set_learned_indicator", "fr_mlp_forward", "fr_mlp_grad", "fr_mlp_train_step",
+           "fr_mlp_forward_alloc", "fr_mlp_train_step_alloc", "fr_tree_complete_alloc", "fr_tree_balance_alloc",
            "fr_tc_set_wait_limit"]
 NOALLOC_SORT_MAX_KEYS = 1 << 18
 
@@ -131,6 +132,9 @@ def load(build_if_missing: bool = True):
     lib.fr_mlp_forward.argtypes = [C.c_int, vp, vp, i64, vp, vp, vp]
     lib.fr_mlp_grad.argtypes = [C.c_int, vp, vp, vp, i64, vp, vp, vp, vp]
     lib.fr_mlp_train_step.argtypes = [C.c_int, vp, vp, vp, i64, vp, vp, i64, vp, C.c_float, vp, vp]
+    al = C.POINTER(FRAllocator)
+    for name in ("fr_mlp_forward", "fr_mlp_train_step", "fr_tree_complete", "fr_tree_balance"):
+        getattr(lib, name + "_alloc").argtypes = getattr(lib, name).argtypes + [al]
     lib.fr_profile_enable.argtypes = [vp, C.c_int]
     lib.fr_profile_read.argtypes = [vp, C.POINTER(FRProfile)]
     lib.fr_tc_set_wait_limit.argtypes = [C.c_longlong]
@@ -217,6 +221,18 @@ class _TorchAllocator:
         self._a = ALLOC_FN(_alloc)
         self._f = FREE_FN(_free)
         self.struct = FRAllocator(self._a, self._f, None)
+
+
+_call_allocs = {}
+
+
+def _call_alloc():
+    """torch's caching allocator on the current device, for the scratch memory of one call (stateless,
+    so shared by all calls)."""
+    d = _torch().cuda.current_device()
+    if d not in _call_allocs:
+        _call_allocs[d] = _TorchAllocator(d)
+    return C.byref(_call_allocs[d].struct)
 
 
 class Mesh:
@@ -400,9 +416,9 @@ def mlp_forward(params, X, stream=None):
     n, n_in = X.shape
     logits = torch.empty((n, 3), dtype=torch.float32, device="cuda")
     flags = torch.empty(n, dtype=torch.int8, device="cuda")
-    _check(load().fr_mlp_forward(n_in, C.c_void_p(params.data_ptr()), C.c_void_p(X.data_ptr()), n,
+    _check(load().fr_mlp_forward_alloc(n_in, C.c_void_p(params.data_ptr()), C.c_void_p(X.data_ptr()), n,
                                  C.c_void_p(logits.data_ptr()), C.c_void_p(flags.data_ptr()),
-                                 _stream_handle(stream)))
+                                 _stream_handle(stream), _call_alloc()))
     return logits, flags
 
 
@@ -427,11 +443,11 @@ def mlp_train_step(params, m, v, step, X, y, class_w, lr, loss=None, stream=None
     """One Adam step in place on `params` (CUDA FP32); X BF16 [B][in], y int8 in {-1,0,1}."""
     B, n_in = X.shape
     cw = _class_w(class_w)
-    _check(load().fr_mlp_train_step(n_in, C.c_void_p(params.data_ptr()), C.c_void_p(m.data_ptr()),
+    _check(load().fr_mlp_train_step_alloc(n_in, C.c_void_p(params.data_ptr()), C.c_void_p(m.data_ptr()),
                                     C.c_void_p(v.data_ptr()), step, C.c_void_p(X.data_ptr()),
                                     C.c_void_p(y.data_ptr()), B, _np_ptr(cw), C.c_float(lr),
                                     C.c_void_p(loss.data_ptr()) if loss is not None else None,
-                                    _stream_handle(stream)))
+                                    _stream_handle(stream), _call_alloc()))
 
 
 def kernel_launches() -> int:
@@ -507,8 +523,8 @@ def _grow_call(fn, cap, *head, tail=()):
 def tree_balance(dim, Dmax, keys, stream=None):
     torch = _torch()
     k = _dev(np.asarray(keys, dtype=np.uint64).view(np.int64), torch.int64)
-    return _grow_call(load().fr_tree_balance, max(16, 2 * k.numel()), dim, Dmax,
-                      C.c_void_p(k.data_ptr()), k.numel(), tail=(_stream_handle(stream),))
+    return _grow_call(load().fr_tree_balance_alloc, max(16, 2 * k.numel()), dim, Dmax,
+                      C.c_void_p(k.data_ptr()), k.numel(), tail=(_stream_handle(stream), _call_alloc()))
 
 
 def tree_adapt(dim, Dbase, Dmax, keys, flags, stream=None):
@@ -525,9 +541,9 @@ def tree_complete(dim, Dmin, Dmax, L, pts, stream=None):
     torch = _torch()
     pt = _dev(np.asarray(pts, dtype=np.float64).reshape(-1, dim) if not isinstance(pts, torch.Tensor)
               else pts, torch.float64)
-    return _grow_call(load().fr_tree_complete, max(16, 4 * pt.shape[0] + (1 << (dim * Dmin))),
+    return _grow_call(load().fr_tree_complete_alloc, max(16, 4 * pt.shape[0] + (1 << (dim * Dmin))),
                       dim, Dmin, Dmax, C.c_double(L), C.c_void_p(pt.data_ptr()), pt.shape[0],
-                      tail=(_stream_handle(stream),))
+                      tail=(_stream_handle(stream), _call_alloc()))
 
 
 def tree_map(dim, Dmax, old_keys, new_keys, stream=None):
