@@ -95,6 +95,45 @@ __host__ __device__ __forceinline__ double fx_double(long long v, int e, bool ba
   return fx_from_bits((uint64_t(hi) << 32) | uint32_t(a));
 }
 
+// ---- sums of products of values (flux terms), each operand with its own exponent E ----
+// x = v 2^(E - 1082) with 60-bit v (one bit more than the operands of the operator contractions, whose
+// sums are longer).  All partial products are kept: the sums below are in units of
+// 2^(Ev + Ew - 2102 - FX_PK), below 2^62 and wrong by less than 5 units (one for each operand cut at its
+// last bit, and the rounding), that is 2^-55 of the product of the operands' powers of two.
+constexpr int FX_PK = 2;
+constexpr int FX_P_MIN = 600;  // smallest exponent of an operand: units of products stay normal
+__host__ __device__ __forceinline__ int2 fx_plimbs(double x, int E) { return fx_limbs(x, E - 1); }
+__host__ __device__ __forceinline__ int fx_pexp(uint32_t mag) {
+  const int e = int(mag >> 20);
+  return e < FX_P_MIN ? FX_P_MIN : e;
+}
+__host__ __device__ __forceinline__ int fx_punit(int Ev, int Ew) { return Ev + Ew - 1079 - FX_PK; }
+// no finite result for certain: an operand that is not finite, or a unit too large for the sum's range
+__host__ __device__ __forceinline__ bool fx_pbad(int Ev, int Ew) {
+  return Ev >= FX_E_BAD || Ew >= FX_E_BAD || fx_punit(Ev, Ew) > 2046 - 62;
+}
+// a b + c d: |h| <= 2 2^58, |m| <= 4 2^60 + 2 2^31
+__host__ __device__ __forceinline__ long long fx_dot2(int2 a, int2 b, int2 c, int2 d) {
+  const long long h = (long long)a.x * b.x + (long long)c.x * d.x;
+  long long m = (long long)a.x * b.y + (long long)a.y * b.x + (long long)c.x * d.y + (long long)c.y * d.x;
+  m += (((long long)a.y * b.y) >> 31) + (((long long)c.y * d.y) >> 31);
+  return (h << FX_PK) + ((m + (1ll << (30 - FX_PK))) >> (31 - FX_PK));
+}
+// sum of n <= 3 squares: h <= 3 2^58, |m| <= 3 2^60 (half of the cross products)
+template <int n>
+__host__ __device__ __forceinline__ long long fx_sum_sq(const int2* v) {
+  long long h = 0, m = 0;
+  unsigned long long l = 0;  // below 3 2^62
+#pragma unroll
+  for (int k = 0; k < n; ++k) {
+    h += (long long)v[k].x * v[k].x;
+    m += (long long)v[k].x * v[k].y;
+    l += (unsigned long long)((long long)v[k].y * v[k].y);
+  }
+  m += (long long)(l >> 32);
+  return (h << FX_PK) + ((m + (1ll << (29 - FX_PK))) >> (30 - FX_PK));
+}
+
 // biased exponent of one unit of a result: values of group exponent E, entries scaled by 2^k
 __host__ __device__ __forceinline__ int fx_unit(int E, int k) { return E + 4 - k; }
 

@@ -9,6 +9,7 @@
 #include <type_traits>
 
 #include "fr_arith.cuh"
+#include "fr_fixed.cuh"
 #include "fr_internal.cuh"
 #include "fr_solver.cuh"
 
@@ -145,6 +146,71 @@ __device__ __forceinline__ void rusanov2_t(const T* qL, const T* qR, int axis, T
   F2[NV - 1] = fma_t(lam, qL[NV - 1] - qR[NV - 1], fma_t(qL[NV - 1] + pL, vL, (qR[NV - 1] + pR) * vR));
 }
 
+// The same in FP64 with its products on the integer pipes (fr_fixed.cuh), which idle in this kernel
+// while the FP64 pipe (2 operations a clock and SM) bounds it: |m|^2 and, for every variable, the sum
+// F2 = qL (vL + lambda) + qR (vR - lambda) + pressure terms, whose products are kept to 2^-55 of
+// |q| lambda.  34 FP64 operations a point in 3D instead of 54.
+template <int DIM>
+__device__ __forceinline__ void rusanov2_fx(const double* qL, const double* qR, int axis, double sgam, double gm1,
+                                            double* F2) {
+  constexpr int NV = DIM + 2;
+  const double rLR = rcp_t(qL[0] * qR[0]);
+  const double rL = qR[0] * rLR, rR = qL[0] * rLR;
+  int E[FX_GROUPS];
+  {
+    uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
+#pragma unroll
+    for (int v = 0; v < NV; ++v) w[fx_group(v, NV)] = max(w[fx_group(v, NV)], max(fx_mag(qL[v]), fx_mag(qR[v])));
+#pragma unroll
+    for (int g = 0; g < FX_GROUPS; ++g) E[g] = fx_pexp(w[g]);
+  }
+  int2 lL[NV], lR[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    lL[v] = fx_plimbs(qL[v], E[fx_group(v, NV)]);
+    lR[v] = fx_plimbs(qR[v], E[fx_group(v, NV)]);
+  }
+  const bool badm = fx_pbad(E[1], E[1]);
+  const double m2L = fx_double(fx_sum_sq<DIM>(lL + 1), fx_punit(E[1], E[1]), badm);
+  const double m2R = fx_double(fx_sum_sq<DIM>(lR + 1), fx_punit(E[1], E[1]), badm);
+  const double pL = gm1 * fma(m2L, neg_half(rL), qL[NV - 1]);
+  const double pR = gm1 * fma(m2R, neg_half(rR), qR[NV - 1]);
+  double mnL = qL[1], mnR = qR[1];
+#pragma unroll
+  for (int b = 1; b < DIM; ++b)
+    if (b == axis) {
+      mnL = qL[1 + b];
+      mnR = qR[1 + b];
+    }
+  const double vL = mnL * rL, vR = mnR * rR;
+  const double lam = fmax_pos(fma(sgam, sqrt_t(pL * rL), fabs(vL)), fma(sgam, sqrt_t(pR * rR), fabs(vR)));
+  const double aL = vL + lam, aR = vR - lam;
+  const int Ea = fx_pexp(max(fx_mag(aL), fx_mag(aR)));
+  const int2 caL = fx_plimbs(aL, Ea), caR = fx_plimbs(aR, Ea);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const int Ev = E[fx_group(v, NV)];
+    F2[v] = fx_double(fx_dot2(lL[v], caL, lR[v], caR), fx_punit(Ev, Ea), fx_pbad(Ev, Ea));
+  }
+  const double pp = pL + pR;
+  double fn = F2[1];
+#pragma unroll
+  for (int b = 1; b < DIM; ++b)
+    if (b == axis) fn = F2[1 + b];
+  fn += pp;
+#pragma unroll
+  for (int b = 0; b < DIM; ++b)
+    if (b == axis) F2[1 + b] = fn;
+  F2[NV - 1] += fma(pL, vL, pR * vR);
+}
+template <int DIM, class T>
+__device__ __forceinline__ void rusanov2(const T* qL, const T* qR, int axis, T sgam, T gm1, T* F2) {
+  if constexpr (std::is_same<T, double>::value)
+    rusanov2_fx<DIM>(qL, qR, axis, sgam, gm1, F2);
+  else
+    rusanov2_t<DIM, T>(qL, qR, axis, sgam, gm1, F2);
+}
+
 // traces tr[e][f][v][q] = sum_j l_j(+-1) u[e][v][line point j]  (mortar procedure step 1).
 // Blocks of EPB elements as in the element kernel: the elements' state is staged in shared memory
 // with coalesced loads, then one thread per (element, face, face point) forms all variables.
@@ -252,7 +318,7 @@ __global__ void __launch_bounds__(FaceCfg<DIM, NP>::T) k_faces_t(FaceArgs A, con
       qL[v] = tL[v * NF];
       qR[v] = tR[v * NF];
     }
-    rusanov2_t<DIM, T>(qL, qR, axis, sgam, gm1, F);
+    rusanov2<DIM, T>(qL, qR, axis, sgam, gm1, F);
     T* fL = fcomm + ((e * NFC + 2 * axis + 1) * NV) * NF + q;
     T* fR = fcomm + ((nb * NFC + 2 * axis) * NV) * NF + q;
 #pragma unroll
@@ -312,9 +378,9 @@ __global__ void __launch_bounds__(FaceCfg<DIM, NP>::T) k_faces_t(FaceArgs A, con
       uf[v] = trace[((ek * NFC + fk) * NV + v) * NF + q];
     }
     if (sidec)
-      rusanov2_t<DIM, T>(uc, uf, axis, sgam, gm1, F);
+      rusanov2<DIM, T>(uc, uf, axis, sgam, gm1, F);
     else
-      rusanov2_t<DIM, T>(uf, uc, axis, sgam, gm1, F);
+      rusanov2<DIM, T>(uf, uc, axis, sgam, gm1, F);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       fcomm[((ek * NFC + fk) * NV + v) * NF + q] = F[v];

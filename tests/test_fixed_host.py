@@ -1,6 +1,7 @@
 """The block fixed point of the FP64 form's contractions (fr_fixed.cuh), run on the host: every result
 within the bound that its operand splitting implies, for the term counts of all degrees and dimensions
-(2 to 5 for traces, 8 to 21 for the derivative with its corrections), over group exponents from 2^-900
+(2 to 5 for traces, 8 to 21 for the derivative with its corrections) and the interface kernel's sums of
+products, over group exponents from 2^-900
 to 2^900 and spreads to 2^80 within a group (tests/cuda/fixed_check.cu)."""
 import os
 import subprocess
@@ -20,4 +21,5 @@ def test_fixed_point_contraction_bounds():
     vals = dict(line.split() for line in out.strip().splitlines())
     for n in TERMS:
         assert 0.0 < float(vals["n%d" % n]) <= 1.0, vals
+    assert 0.0 < float(vals["dot"]) <= 1.0 and 0.0 < float(vals["squares"]) <= 1.0, vals
     assert float(vals["double"]) <= 1.0 and float(vals["zero"]) == 0.0 and vals["nan"] == "1", vals
