@@ -154,7 +154,8 @@ inline int fx_scale(double sum) {
 
 // Largest magnitude (high words) per group over the N threads of one element, thread i of it, into
 // s[3] of the element (biased exponents; zeroed before a barrier by the caller, read after one).
-// All threads of the block call it; those without a point bring zeros and act = false.
+// All threads of the block call it; those without a point bring zeros and act = false.  With N a power
+// of two up to 16 an element lies in one warp and the values are stored, not accumulated.
 template <int N>
 __device__ __forceinline__ void fx_group_max(uint32_t w0, uint32_t w1, uint32_t w2, int i, bool act, uint32_t* s) {
   const int lane = threadIdx.x & 31;
@@ -167,6 +168,19 @@ __device__ __forceinline__ void fx_group_max(uint32_t w0, uint32_t w1, uint32_t 
       atomicMax(&s[0], w0 >> 20);
       atomicMax(&s[1], w1 >> 20);
       atomicMax(&s[2], w2 >> 20);
+    }
+  } else if constexpr (32 % N == 0) {
+    // whole elements in a warp: one value per element, no atomics
+    uint32_t p = (w0 >> 20) | ((w1 >> 20) << 16), q = w2 >> 20;
+#pragma unroll
+    for (int o = 1; o < N; o <<= 1) {
+      p = __vmaxu2(p, __shfl_xor_sync(~0u, p, o));
+      q = max(q, __shfl_xor_sync(~0u, q, o));
+    }
+    if (act && i == 0) {
+      s[0] = p & 0xFFFFu;
+      s[1] = p >> 16;
+      s[2] = q;
     }
   } else {
     // segments of N lanes that may cross warps: each segment's first lane in a warp collects it;

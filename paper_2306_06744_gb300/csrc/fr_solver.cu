@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_transfer(KG g, const uint64
     if (work) {
 #pragma unroll
       for (int v = 0; v < NV; ++v)
-        sv[le * EU + v * N + i] = fx_limbs(acc[v], fx_exp(se[le * FX_GROUPS + fx_group(v, NV)]));
+        sv[le * EU + v * N + fx_place<DIM, NP>(i)] = fx_limbs(acc[v], fx_exp(se[le * FX_GROUPS + fx_group(v, NV)]));
     }
     __syncthreads();
     const int ne = int((Mn - j0) < EPB ? (Mn - j0) : EPB);

@@ -59,7 +59,15 @@ inline OpsFx make_ops_fx(int dim, int p, const DevOps& o, double gamma) {
   return r;
 }
 
-// Traces of the block's elements from their fixed-point state sv[le][v][i] with group exponents
+// Place of point i in an element's staged state.  At 3D p = 3 the lines along x of 16 lanes start 32
+// bytes apart, four to a bank, and so do those along y in different planes: x and y are exclusive-ored
+// with the plane's index, which spreads both over all banks.
+template <int DIM, int NP>
+__device__ __forceinline__ constexpr int fx_place(int i) {
+  return DIM == 3 && NP == 4 ? i ^ ((i >> 4) * 5) : i;
+}
+
+// Traces of the block's elements from their fixed-point state sv[le][v][place of i] with group exponents
 // se[le][group]: one thread per (element, face, face point), all variables.  need (nullable): only
 // elements with a non-zero entry.
 template <int DIM, int NP>
@@ -77,7 +85,7 @@ __device__ __forceinline__ void fx_traces(const int2* sv, const uint32_t* se, co
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
       c[j] = lf[j];
-      pts[j] = le * EU + line_pt<DIM, NP>(f >> 1, q, j);
+      pts[j] = le * EU + fx_place<DIM, NP>(line_pt<DIM, NP>(f >> 1, q, j));
     }
     double* t = to + int64_t(le) * EF + f * NV * NF + q;
 #pragma unroll
@@ -132,7 +140,7 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_traces_fx(const double* __r
   if (act) {
 #pragma unroll
     for (int v = 0; v < NV; ++v)
-      sv[le * EU + v * N + i] = fx_limbs(q[v], fx_exp(se[le * FX_GROUPS + fx_group(v, NV)]));
+      sv[le * EU + v * N + fx_place<DIM, NP>(i)] = fx_limbs(q[v], fx_exp(se[le * FX_GROUPS + fx_group(v, NV)]));
   }
   __syncthreads();
   fx_traces<DIM, NP>(sv, se, slm, slp, ops.kt, ne, need, tr + e0 * S::EF);
@@ -177,8 +185,8 @@ struct StageOcc {
 // accumulator once that has moved to the larger of the two exponents, so that the volume part stays
 // before the wait on the interface kernel.  Per point about 2,400 instructions (a third of them the
 // conversions of 28 values to limbs and 13 back); FP64 pipe 55%, issue slots 54%, shared memory 59% busy,
-// DRAM 28% of peak.  Four 3D p = 3 tubes, 242k leaves: 3.95 ms per launch with the contractions in FP64,
-// 1.62 ms so.
+// DRAM 28% of peak.  Four 3D p = 3 tubes, 127k leaves: 2166 us per launch with the contractions in FP64,
+// 825 us so (838 without the spread places of fx_place and u^n's prefetch).
 template <int DIM, int NP>
 __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageOcc<DIM, NP>::value)
     k_stage_fx(StageArgs A, const __grid_constant__ OpsFx ops) {
@@ -208,6 +216,10 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageOcc<DIM, NP>::value)
   double q[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) q[v] = A.us[b0 + v * N];
+  // u^n is read at the end: into the second-level cache meanwhile
+  if (A.rk & RK_A)
+    for (int k = tid * 16; k < ne * EU; k += BT * 16)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(A.un + e0 * EU + k));
   // c * (-2/h): 2^depth * (2/L) is exact, so this equals the rounded -2^(depth+1)/L times c
   if (tid < ne) {
     sh2[tid] = -A.c * (double(1ull << A.g.depth(A.keys[e0 + tid])) * A.twoL);
@@ -398,7 +410,7 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageOcc<DIM, NP>::value)
     if (own) {
 #pragma unroll
       for (int v = 0; v < NV; ++v)
-        sfl[le * EU + v * N + i] = fx_limbs(out[v], fx_exp(seo[le * FX_GROUPS + fx_group(v, NV)]));
+        sfl[le * EU + v * N + fx_place<DIM, NP>(i)] = fx_limbs(out[v], fx_exp(seo[le * FX_GROUPS + fx_group(v, NV)]));
     }
     __syncthreads();
     fx_traces<DIM, NP>(sfl, seo, slm, slp, ops.tr.kt, ne, nullptr, static_cast<double*>(A.trace_out) + e0 * EF);
