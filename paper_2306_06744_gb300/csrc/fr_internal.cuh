@@ -60,6 +60,21 @@ __device__ __forceinline__ void pdl_wait_then_release() {
 // after its own wait, so when a kernel starts early, everything but its immediate predecessor has
 // completed.  Writes always come after the wait.
 
+// asynchronous copy of W bytes (4, 8 or 16, both addresses aligned to W) from global to shared memory;
+// visible to the issuing thread after cp_async_wait, to the block after a barrier behind that
+template <int W>
+__device__ __forceinline__ void cp_async(void* dst, const void* src) {
+  static_assert(W == 4 || W == 8 || W == 16, "cp.async size");
+  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+  if constexpr (W == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(W) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// bytes per copy of rows of B bytes one after another from a 16-byte aligned start
+constexpr int cp_width(int B) { return B % 16 == 0 ? 16 : (B % 8 == 0 ? 8 : 4); }
+
 template <class Kern, class... Args>
 cudaError_t launch_dependent(Kern kernel, unsigned grid, unsigned block, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};

@@ -424,17 +424,6 @@ __global__ void __launch_bounds__(FaceCfg<DIM, NP>::T) k_faces_t(FaceArgs A, con
   }
 }
 
-// Runge-Kutta combination type: FP64 for double and float (the mixed form keeps FP64 RK
-// accumulation), double-word for ff.
-template <class T>
-struct RkT {
-  using type = double;
-};
-template <>
-struct RkT<ff> {
-  using type = ff;
-};
-
 // Resident blocks the element kernel is compiled for: the FP32 form is bound by memory latency
 // and wants every block shared memory allows (the register budget is set to fit them); the others
 // keep the compiler's choice.
@@ -448,16 +437,18 @@ struct StageMinBlocks {
 // stores 2F and the slopes carry the 1/2), then out = a*un + b*us + c*R (Eq. rk3), and
 // (optionally) the traces of out.  Phases: stage state -> pointwise fluxes -> volume sums
 // sum_j Dt_ij f_j, all before the wait on the interface kernel; then its common fluxes ->
-// correction terms, Runge-Kutta combination, traces.
+// correction terms, Runge-Kutta combination, traces.  FP32 and double-word forms.
+// FP32: bound by the memory system (79% of the measured copy rate in large grids); double-word: by
+// instruction issue.  Three block barriers, no staging of the input state, the Runge-Kutta combination in
+// FP64 and the asynchronous fetch give, per launch at 3D p = 3 with 127k leaves, FP32 374 -> 274 us and
+// double-word 959 -> 806 us (2D p = 3, 11k leaves: 12.6 -> 11.9 and 20.5 -> 18.6 us).
 template <int DIM, int NP, class T>
 __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value) k_stage_t(StageArgs A, const __grid_constant__ OpsT<T> ops) {
   using S = Sz<DIM, NP>;
-  using RT = typename RkT<T>::type;
   constexpr int N = S::N, NV = S::NV, NF = S::NF, EU = S::EU, EF = S::EF;
   constexpr int EPB = S::EPB;
-  __shared__ T su[EPB * EU];
-  __shared__ T sfl[EPB * DIM * EU];
-  __shared__ T sfc[EPB * EF];
+  __shared__ T sfl[EPB * DIM * EU];  // fluxes; after the derivative the new state
+  __shared__ __align__(16) T sfc[EPB * EF];
   __shared__ double sh2[EPB];  // per element: c * (-2/h)
   const T* fcomm = static_cast<const T*>(A.fcomm);
   T* trace_out = static_cast<T*>(A.trace_out);
@@ -470,52 +461,60 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value) k_s
   // thread loads its own point; its u^n stays in registers for the Runge-Kutta combination.
   const int le = tid / N, i = tid % N;
   const bool act = le < ne;
-  double unr[NV];
+  const int64_t b0 = (e0 + le) * EU + i;
+  // the block's common fluxes, one contiguous piece of memory
+  auto fetch = [&]() {
+    constexpr int W = cp_width(EF * int(sizeof(T)));
+    const char* src = reinterpret_cast<const char*>(fcomm + e0 * EF);
+    if (A.fetch & FETCH_WIDE) {
+      for (int k = tid; k < ne * EF * int(sizeof(T)) / W; k += blockDim.x)
+        cp_async<W>(reinterpret_cast<char*>(sfc) + k * W, src + k * W);
+    } else {
+      for (int k = tid; k < ne * EF; k += blockDim.x) cp_async<sizeof(T)>(sfc + k, fcomm + e0 * EF + k);
+    }
+  };
+  if (A.fetch & FETCH_EARLY) {
+    pdl_wait_then_release();
+    fetch();
+  }
+  double unr[NV], outv[NV];
   if (act) {
-    const int64_t b0 = (e0 + le) * EU + i;
+    T q[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       unr[v] = (A.rk & RK_A) ? A.un[b0 + v * N] : 0.0;
-      su[le * EU + v * N + i] = Ar<T>::from_d(A.us[b0 + v * N]);
+      q[v] = Ar<T>::from_d(A.us[b0 + v * N]);
     }
-  }
-  // c * (-2/h): 2^depth * (2/L) is exact, so this equals the rounded -2^(depth+1)/L times c
-  if (tid < ne) {
-    sh2[tid] = -A.c * (double(1ull << A.g.depth(A.keys[e0 + tid])) * A.twoL);
-  }
-  __syncthreads();
-  const T gm1 = ops.gm1, ngmh = ops.ngmh;
-  RT outv[NV];
-  if (act) {
-    const T* q = su + le * EU;
-    T rho = q[i], rinv = rcp_t(rho), E = q[(NV - 1) * N + i];
+    const T gm1 = ops.gm1, ngmh = ops.ngmh;
+    const T rinv = rcp_t(q[0]), E = q[NV - 1];
     T vel[DIM];
     T m2 = zero_t<T>();
 #pragma unroll
     for (int b = 0; b < DIM; ++b) {
-      vel[b] = q[(1 + b) * N + i] * rinv;
-      m2 = fma_t(q[(1 + b) * N + i], vel[b], m2);
+      vel[b] = q[1 + b] * rinv;
+      m2 = fma_t(q[1 + b], vel[b], m2);
     }
-    T p = fma_t(ngmh, m2, gm1 * E);
-    T Ep = E + p;
+    const T p = fma_t(ngmh, m2, gm1 * E), Ep = E + p;
     // momentum flux m_b v_a, symmetric in (a, b): each off-diagonal product is formed once
     T mv[DIM][DIM];
 #pragma unroll
     for (int a = 0; a < DIM; ++a)
 #pragma unroll
       for (int b = a; b < DIM; ++b) {
-        mv[a][b] = q[(1 + b) * N + i] * vel[a];
+        mv[a][b] = q[1 + b] * vel[a];
         mv[b][a] = mv[a][b];
       }
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
       T* fa = sfl + (le * DIM + a) * EU;
-      fa[i] = q[(1 + a) * N + i];
+      fa[i] = q[1 + a];
 #pragma unroll
       for (int b = 0; b < DIM; ++b) fa[(1 + b) * N + i] = (a == b) ? mv[a][b] + p : mv[a][b];
       fa[(NV - 1) * N + i] = Ep * vel[a];
     }
   }
+  // c * (-2/h): 2^depth * (2/L) is exact, so this equals the rounded -2^(depth+1)/L times c
+  if (tid < ne) sh2[tid] = -A.c * (double(1ull << A.g.depth(A.keys[e0 + tid])) * A.twoL);
   __syncthreads();
   // volume part of the folded derivative, sum_a sum_j Dt_ij f_j, also before the wait: one FMA
   // chain per variable, the correction terms are added once the common fluxes are in
@@ -536,8 +535,11 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value) k_s
       }
     }
   }
-  pdl_wait_then_release();
-  for (int k = tid; k < ne * EF; k += blockDim.x) sfc[k] = fcomm[e0 * EF + k];
+  if (!(A.fetch & FETCH_EARLY)) {
+    pdl_wait_then_release();
+    fetch();
+  }
+  cp_async_wait();
   __syncthreads();
   if (act) {
 #pragma unroll
@@ -554,42 +556,28 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value) k_s
     // to hold the occupancy
     double usr[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) usr[v] = A.us[(e0 + le) * EU + v * N + i];
-    if constexpr (!std::is_same<T, ff>::value) {
-      // FP64 combination (the mixed FP32 form).  The first stage (a = 0, b = 1)
-      // is one FMA per value; the branch is uniform over the grid (kernel arguments), so the
-      // other stages do not pay for it
-      if (A.rk == RK_B1) {
+    for (int v = 0; v < NV; ++v) usr[v] = A.us[b0 + v * N];
+    // FP64 combination in both forms: the FP64 pipe is otherwise idle, and in the double-word form its
+    // 15 operations a point replace about 240 instructions.  The first stage (a = 0, b = 1) is one FMA
+    // per value; the branch is uniform over the grid (kernel arguments), so the other stages do not pay
+    // for it
+    if (A.rk == RK_B1) {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) outv[v] = fma(cs, Ar<T>::to_d(R[v]), usr[v]);
-      } else {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          double o = fma(cs, Ar<T>::to_d(R[v]), (A.rk & RK_B1) ? usr[v] : A.b * usr[v]);
-          if (A.rk & RK_A) o = fma(A.a, unr[v], o);
-          outv[v] = o;
-        }
-      }
+      for (int v = 0; v < NV; ++v) outv[v] = fma(cs, Ar<T>::to_d(R[v]), usr[v]);
     } else {
-      // double-word combination
-      const ff bb = ff_from_double(A.b), cc = ff_from_double(cs), aa = ff_from_double(A.a);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        ff o = fma_t(bb, su[le * EU + v * N + i], cc * R[v]);
-        if (A.rk & RK_A) o = fma_t(aa, ff_from_double(unr[v]), o);
+        double o = fma(cs, Ar<T>::to_d(R[v]), (A.rk & RK_B1) ? usr[v] : A.b * usr[v]);
+        if (A.rk & RK_A) o = fma(A.a, unr[v], o);
         outv[v] = o;
       }
     }
   }
-  __syncthreads();
   if (act) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      if constexpr (std::is_same<T, ff>::value)
-        su[le * EU + v * N + i] = outv[v];
-      else
-        su[le * EU + v * N + i] = Ar<T>::from_d(outv[v]);
-      A.out[(e0 + le) * EU + v * N + i] = Ar<RT>::to_d(outv[v]);
+      sfl[le * EU + v * N + i] = Ar<T>::from_d(outv[v]);
+      A.out[b0 + v * N] = outv[v];
     }
   }
   __syncthreads();
@@ -606,7 +594,7 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value) k_s
       T* to = trace_out + (e0 + le2) * EF + f * NV * NF + qq;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        const T* ue = su + le2 * EU + v * N;
+        const T* ue = sfl + le2 * EU + v * N;
         if constexpr (std::is_same<T, ff>::value) {
           ffacc A{0.f, 0.f};
 #pragma unroll
@@ -685,13 +673,15 @@ int launch_faces_impl(int dim, int p, FaceArgs A, const DevOps& o, cudaStream_t 
 }
 
 template <class T>
-int launch_stage_impl(int dim, int p, const StageArgs& A, const DevOps& o, cudaStream_t s, Err* err) {
+int launch_stage_impl(int dim, int p, const StageArgs& args, const DevOps& o, cudaStream_t s, Err* err) {
+  StageArgs A = args;
   if (A.M <= 0) return 0;
   OpsT<T> ops = make_ops_t<T>(o);
   set_gas(&ops, A.gamma);
   FR_NP_DISPATCH(dim, p, ({
                    using SS = Sz<DD, NN>;
                    unsigned nb = unsigned((A.M + SS::EPB - 1) / SS::EPB);
+                   A.fetch = fetch_mode(nb, A.fcomm);
                    if (launch_dependent(k_stage_t<DD, NN, T>, nb, SS::BT, s, A, ops) != cudaSuccess)
                      return set_error(err, FR_ECUDA, "element kernel launch");
                  }));

@@ -26,11 +26,22 @@ struct StageArgs {
   KG g;
   double twoL, gamma, a, b, c;  // twoL = 2 / L
   int rk;                       // RK_A: a != 0; RK_B1: b == 1 (integer tests, no FP64 compares per thread)
+  int fetch;                    // FETCH_EARLY, FETCH_WIDE
   int* status;                  // device word set by a tensor-core kernel whose completion wait gave up
   int8_t* flags;                // FP64 form: density-gradient flags of out (nullable)
   double th_r, th_c;            // their refine / coarsen thresholds
 };
 
+// The element kernel of the FP32 and double-word forms fetches its common fluxes asynchronously.  Its
+// volume part needs none and overlaps the interface kernel's drain, which matters while the grid is about
+// one wave (up to 4 waves here); in a grid of many waves the blocks instead wait for the interface kernel
+// at their start and let the fetch run behind the volume part.
+constexpr int64_t STAGE_EARLY_BLOCKS = 152 * 8 * 4;
+enum { FETCH_EARLY = 1, FETCH_WIDE = 2 };  // wide: the common fluxes start on a 16-byte boundary
+inline int fetch_mode(int64_t blocks, const void* fcomm) {
+  return (blocks >= STAGE_EARLY_BLOCKS ? FETCH_EARLY : 0) |
+         ((reinterpret_cast<uintptr_t>(fcomm) & 15) == 0 ? FETCH_WIDE : 0);
+}
 enum { RK_A = 1, RK_B1 = 2 };
 inline int rk_mode(double a, double b) { return (a != 0.0 ? RK_A : 0) | (b == 1.0 ? RK_B1 : 0); }
 
