@@ -20,7 +20,7 @@
 
 namespace frg {
 
-struct ff {
+struct __align__(8) ff {  // one 8-byte access
   float h, l;
 };
 
@@ -206,7 +206,6 @@ __device__ __forceinline__ double fmax_t(double a, double b) { return fmax(a, b)
 __device__ __forceinline__ double fmax_pos(double a, double b) {
   return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
 }
-__device__ __forceinline__ float fmax_pos(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ ff fmax_pos(ff a, ff b) { return fmax_t(a, b); }
 __device__ __forceinline__ float fmax_t(float a, float b) { return fmaxf(a, b); }
 
@@ -214,7 +213,6 @@ __device__ __forceinline__ float fmax_t(float a, float b) { return fmaxf(a, b); 
 __device__ __forceinline__ double neg_half(double x) {
   return __hiloint2double((__double2hiint(x) - (1 << 20)) ^ int(0x80000000u), __double2loint(x));
 }
-__device__ __forceinline__ float neg_half(float x) { return -0.5f * x; }
 __device__ __forceinline__ ff neg_half(ff x) { return {-0.5f * x.h, -0.5f * x.l}; }
 
 // zero / constant helpers

@@ -24,9 +24,9 @@ struct OpsT {
   T gLh[NPMAX], gRh[NPMAX], lm[NPMAX], lp[NPMAX];
   T I[2][NPMAX][NPMAX];
   T P[2][NPMAX][NPMAX];
-  // gas constants in the arithmetic type, formed on the host (set_gas): sqrt(gamma), gamma - 1 and
-  // -(gamma - 1)/2, so that no thread spends FP64 operations on them
-  T sgam, gm1, ngmh;
+  // gas constants in the arithmetic type, formed on the host (set_gas): gamma, its root, gamma - 1
+  // and -(gamma - 1)/2, so that no thread spends FP64 operations on them
+  T gam, sgam, gm1, ngmh;
 };
 
 inline double host_conv(double x, double*) { return x; }
@@ -40,6 +40,7 @@ inline ff host_conv(double x, ff*) {
 template <class T>
 void set_gas(OpsT<T>* r, double gamma) {
   T* tag = nullptr;
+  r->gam = host_conv(gamma, tag);
   r->sgam = host_conv(std::sqrt(gamma), tag);
   r->gm1 = host_conv(gamma - 1.0, tag);
   r->ngmh = host_conv(-0.5 * (gamma - 1.0), tag);
@@ -107,40 +108,84 @@ __device__ __forceinline__ void pt_split(int i, int axis, int* q, int* ia) {
 
 // Twice the Rusanov common flux along +axis between the minus-side state qL and the plus-side
 // qR, F2 = f(qL) + f(qR) - lambda (qR - qL) with lambda = max(|u_n| + c) of the two states
-// (Sec. 4.3); the factor 1/2 is carried by the correction slopes.  sgam = sqrt(gamma), gm1 =
-// gamma - 1.
-template <int DIM, class T>
-__device__ __forceinline__ void rusanov2_t(const T* qL, const T* qR, int axis, T sgam, T gm1, T* F2) {
+// (Sec. 4.3); the factor 1/2 is carried by the correction slopes.  ngmh = -(gamma - 1)/2, so
+// that p = (gamma - 1) E + ngmh |m|^2 / rho.
+// FP32 form.
+template <int DIM>
+__device__ __forceinline__ void rusanov2_f32(const float* qL, const float* qR, int axis, float gam, float gm1, float ngmh,
+                                             float* F2) {
   constexpr int NV = DIM + 2;
   // both reciprocal densities from one reciprocal: 1/rho_L = rho_R / (rho_L rho_R), and so on
-  const T rLR = rcp_t(qL[0] * qR[0]);
-  T rL = qR[0] * rLR, rR = qL[0] * rLR;
-  T m2L = qL[1] * qL[1], m2R = qR[1] * qR[1];
+  const float rLR = rcp_t(qL[0] * qR[0]);
+  float rL = qR[0] * rLR, rR = qL[0] * rLR;
+  float m2L = qL[1] * qL[1], m2R = qR[1] * qR[1];
 #pragma unroll
   for (int b = 1; b < DIM; ++b) {
     m2L = fma_t(qL[1 + b], qL[1 + b], m2L);
     m2R = fma_t(qR[1 + b], qR[1 + b], m2R);
   }
-  const T pL = gm1 * fma_t(m2L, neg_half(rL), qL[NV - 1]);
-  const T pR = gm1 * fma_t(m2R, neg_half(rR), qR[NV - 1]);
+  float pL = fma_t(ngmh, m2L * rL, gm1 * qL[NV - 1]);
+  float pR = fma_t(ngmh, m2R * rR, gm1 * qR[NV - 1]);
   // normal momenta, selected with unrolled predicates so the state stays in registers
-  T mnL = qL[1], mnR = qR[1];
+  float mnL = qL[1], mnR = qR[1];
 #pragma unroll
   for (int b = 1; b < DIM; ++b)
     if (b == axis) {
       mnL = qL[1 + b];
       mnR = qR[1 + b];
     }
-  T vL = mnL * rL, vR = mnR * rR;
+  float vL = mnL * rL, vR = mnR * rR;
+  float cL = sqrt_t(gam * pL * rL), cR = sqrt_t(gam * pR * rR);
+  float lam = fmax_t(fabs_t(vL) + cL, fabs_t(vR) + cR);
+  float fL[NV], fR[NV];
+  fL[0] = mnL;
+  fR[0] = mnR;
+#pragma unroll
+  for (int b = 0; b < DIM; ++b) {
+    float a = qL[1 + b] * vL, c = qR[1 + b] * vR;
+    fL[1 + b] = (b == axis) ? a + pL : a;
+    fR[1 + b] = (b == axis) ? c + pR : c;
+  }
+  fL[NV - 1] = (qL[NV - 1] + pL) * vL;
+  fR[NV - 1] = (qR[NV - 1] + pR) * vR;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) F2[v] = fma_t(lam, qL[v] - qR[v], fL[v] + fR[v]);
+}
+
+// The same in double-word arithmetic, with fewer operations: the flux sums are multiply-add chains, the
+// pressures enter by a select, c = sqrt(gamma) sqrt(p / rho) joins |v| in a multiply-add.
+template <int DIM>
+__device__ __forceinline__ void rusanov2_ff(const ff* qL, const ff* qR, int axis, ff sgam, ff gm1, ff* F2) {
+  constexpr int NV = DIM + 2;
+  // both reciprocal densities from one reciprocal: 1/rho_L = rho_R / (rho_L rho_R), and so on
+  const ff rLR = rcp_t(qL[0] * qR[0]);
+  ff rL = qR[0] * rLR, rR = qL[0] * rLR;
+  ff m2L = qL[1] * qL[1], m2R = qR[1] * qR[1];
+#pragma unroll
+  for (int b = 1; b < DIM; ++b) {
+    m2L = fma_t(qL[1 + b], qL[1 + b], m2L);
+    m2R = fma_t(qR[1 + b], qR[1 + b], m2R);
+  }
+  const ff pL = gm1 * fma_t(m2L, neg_half(rL), qL[NV - 1]);
+  const ff pR = gm1 * fma_t(m2R, neg_half(rR), qR[NV - 1]);
+  // normal momenta, selected with unrolled predicates so the state stays in registers
+  ff mnL = qL[1], mnR = qR[1];
+#pragma unroll
+  for (int b = 1; b < DIM; ++b)
+    if (b == axis) {
+      mnL = qL[1 + b];
+      mnR = qR[1 + b];
+    }
+  ff vL = mnL * rL, vR = mnR * rR;
   // |v| + c with c = sqrt(gamma) sqrt(p / rho)
-  const T lam = fmax_pos(fma_t(sgam, sqrt_t(pL * rL), fabs_t(vL)), fma_t(sgam, sqrt_t(pR * rR), fabs_t(vR)));
+  const ff lam = fmax_pos(fma_t(sgam, sqrt_t(pL * rL), fabs_t(vL)), fma_t(sgam, sqrt_t(pR * rR), fabs_t(vR)));
   // f(qL) + f(qR) - lambda (qR - qL), the sums as multiply-adds; the pressures enter the normal
   // momentum through the chain's start (a select) instead of an addition per component
-  const T pp = pL + pR;
+  const ff pp = pL + pR;
   F2[0] = fma_t(lam, qL[0] - qR[0], mnL + mnR);
 #pragma unroll
   for (int b = 0; b < DIM; ++b) {
-    const T s = fma_t(qL[1 + b], vL, fma_t(qR[1 + b], vR, b == axis ? pp : zero_t<T>()));
+    const ff s = fma_t(qL[1 + b], vL, fma_t(qR[1 + b], vR, b == axis ? pp : zero_t<ff>()));
     F2[1 + b] = fma_t(lam, qL[1 + b] - qR[1 + b], s);
   }
   F2[NV - 1] = fma_t(lam, qL[NV - 1] - qR[NV - 1], fma_t(qL[NV - 1] + pL, vL, (qR[NV - 1] + pR) * vR));
@@ -204,11 +249,13 @@ __device__ __forceinline__ void rusanov2_fx(const double* qL, const double* qR, 
   F2[NV - 1] += fma(pL, vL, pR * vR);
 }
 template <int DIM, class T>
-__device__ __forceinline__ void rusanov2(const T* qL, const T* qR, int axis, T sgam, T gm1, T* F2) {
+__device__ __forceinline__ void rusanov2(const T* qL, const T* qR, int axis, const OpsT<T>& o, T* F2) {
   if constexpr (std::is_same<T, double>::value)
-    rusanov2_fx<DIM>(qL, qR, axis, sgam, gm1, F2);
+    rusanov2_fx<DIM>(qL, qR, axis, o.sgam, o.gm1, F2);
+  else if constexpr (std::is_same<T, ff>::value)
+    rusanov2_ff<DIM>(qL, qR, axis, o.sgam, o.gm1, F2);
   else
-    rusanov2_t<DIM, T>(qL, qR, axis, sgam, gm1, F2);
+    rusanov2_f32<DIM>(qL, qR, axis, o.gam, o.gm1, o.ngmh, F2);
 }
 
 // traces tr[e][f][v][q] = sum_j l_j(+-1) u[e][v][line point j]  (mortar procedure step 1).
@@ -296,7 +343,6 @@ __global__ void __launch_bounds__(FaceCfg<DIM, NP>::T) k_faces_t(FaceArgs A, con
   __shared__ T sW[FPB][DIM == 3 ? (HA > HB ? HA : HB) : 1];
   const T* trace = static_cast<const T*>(A.trace);
   T* fcomm = static_cast<T*>(A.fcomm);
-  const T sgam = ops.sgam, gm1 = ops.gm1;
   const int tid = threadIdx.x;
   // the face lists and neighbour tables are fixed during a time step: they are read while the
   // element kernel this one depends on drains; the traces it wrote are read after the wait
@@ -318,7 +364,7 @@ __global__ void __launch_bounds__(FaceCfg<DIM, NP>::T) k_faces_t(FaceArgs A, con
       qL[v] = tL[v * NF];
       qR[v] = tR[v * NF];
     }
-    rusanov2<DIM, T>(qL, qR, axis, sgam, gm1, F);
+    rusanov2<DIM, T>(qL, qR, axis, ops, F);
     T* fL = fcomm + ((e * NFC + 2 * axis + 1) * NV) * NF + q;
     T* fR = fcomm + ((nb * NFC + 2 * axis) * NV) * NF + q;
 #pragma unroll
@@ -378,9 +424,9 @@ __global__ void __launch_bounds__(FaceCfg<DIM, NP>::T) k_faces_t(FaceArgs A, con
       uf[v] = trace[((ek * NFC + fk) * NV + v) * NF + q];
     }
     if (sidec)
-      rusanov2<DIM, T>(uc, uf, axis, sgam, gm1, F);
+      rusanov2<DIM, T>(uc, uf, axis, ops, F);
     else
-      rusanov2<DIM, T>(uf, uc, axis, sgam, gm1, F);
+      rusanov2<DIM, T>(uf, uc, axis, ops, F);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       fcomm[((ek * NFC + fk) * NV + v) * NF + q] = F[v];
