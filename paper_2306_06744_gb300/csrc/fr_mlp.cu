@@ -57,180 +57,121 @@ __host__ __device__ inline Lay lay(int in) {
   return L;
 }
 
-// Lagrange matrix from the element's points to the 3 Gauss-Legendre points per axis, as fixed-point
-// entries (fr_fixed.cuh)
-struct I3Fx {
-  int2 c[3][NPMAX];
+// Lagrange matrix from the element's points to the 3 Gauss-Legendre points per axis, as double-word
+// constants
+struct I3Mat {
+  ff m[3][NPMAX];
 };
-// one axis of the interpolation: three results from the n values at `in` (stride st), as limbs at the
-// scale of the input (entries summing to at most 2^61: results stay below 2^59) or, last, as integers
-// half as large
+// one axis of the interpolation: three results from the n values at `in` (stride st)
 template <int NP>
-__device__ __forceinline__ void interp3(const I3Fx& I3, const int2* in, int st, FxAcc (&a)[3]) {
+__device__ __forceinline__ void interp3(const I3Mat& I3, const ff* in, int st, ff (&a)[3]) {
 #pragma unroll
-  for (int s = 0; s < 3; ++s) a[s] = FxAcc{0, 0};
+  for (int s = 0; s < 3; ++s) a[s] = ff{0.f, 0.f};
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
-    const int2 x = in[j * st];
+    const ff x = in[j * st];
 #pragma unroll
-    for (int s = 0; s < 3; ++s) fx_mac(a[s], x, I3.c[s][j]);
+    for (int s = 0; s < 3; ++s) a[s] = fma_t(I3.m[s][j], x, a[s]);
   }
 }
-__device__ __forceinline__ int2 interp_limbs(const FxAcc& a) {
-  const long long v = (a.h << 1) + ((a.m + (1ll << 29)) >> 30);
-  return make_int2(int(v >> 31), int(uint32_t(v) & 0x7FFFFFFFu));
-}
-// a 58-bit integer as a double-word value (the low 11 bits rounded away)
-__device__ __forceinline__ ff ff_from_fixed(long long v) {
-  v += 1ll << 10;
-  const float hi = __int2float_rn(int(v >> 35)) * 34359738368.f;
-  return ff_fast_two_sum(hi, __int2float_rn(int(uint32_t(v >> 11) & 0xFFFFFFu)) * 2048.f);
-}
 
-// quotient from one float reciprocal r: a.h r, then the exact residual's quotient, twice (each leaves the
-// 2^-23 of r), with relative error ~2^-47; a third of the instructions of the general quotient
-__device__ __forceinline__ ff ff_div(ff a, ff b) {
-  const float r = __fdividef(1.f, b.h);
-  const float q1 = a.h * r;
-  const float e1 = fmaf(-q1, b.h, a.h), t1 = fmaf(-q1, b.l, a.l);
-  const float q2 = (e1 + t1) * r;
-  const float q3 = (fmaf(-q2, b.h, e1) + fmaf(-q2, b.l, t1)) * r;
-  return ff_fast_two_sum(q1, q2 + q3);
-}
-
-// Features.  Blocks of 128 threads and EPB elements (a multiple of the four warps): the state is staged
-// in shared memory as fixed-point limbs and interpolated to the 3^dim sample points axis by axis
-// (n^dim -> 3 n^(dim-1) -> ... -> 3^dim values per variable), each item three results from one line; then
-// one warp per element takes a sample per lane.  The features are relative deviations of nearly equal
-// values: those of the density are differences of integers, rounded once; the pressure is formed in
-// double-word arithmetic (~48 bits; FP64 on GB300 runs at 1/58 of the FP32 rate).
+// Features, in double-word arithmetic (pairs of floats, ~48-bit significand, on the FP32 pipes): they are
+// relative deviations of nearly equal values, which FP32 alone would swamp with rounding noise, while
+// FP64 on GB300 runs at 1/58 of the FP32 rate.  Blocks of 128 threads and EPB elements: the state is
+// staged in shared memory and interpolated to the 3^dim sample points axis by axis (n^dim ->
+// 3 n^(dim-1) -> ... -> 3^dim values per variable), each item three results from one line; then a thread
+// takes a sample, a thread each the sums of an element's densities and pressures (in sample order), and
+// again a thread a sample.  Bound by instruction issue (a double-word multiply-add is 15 instructions,
+// an element of 3D p = 3 has 2,200).  One thread per element, which kept all samples in registers and
+// read the state with the stride of an element: 2417 us for the 3D p = 3 mesh of 500k leaves; so: 939 us.
 constexpr int FT_T = 128;
 template <int DIM, int NP>
 struct FeatBlk {
   static constexpr int N = Sz<DIM, NP>::N;
   static constexpr int EPB = N == 8 ? 16 : (N <= 4 ? 32 : (N <= 9 ? 24 : (N <= 16 ? 16 : (N <= 27 ? 8 : 4))));
-  static constexpr int PT = (EPB * N + FT_T - 1) / FT_T;  // points per thread
 };
 template <int DIM, int NP>
 __global__ void __launch_bounds__(FT_T) k_features(const double* __restrict__ u, const uint64_t* __restrict__ keys,
-                                                   int64_t M, KG g, int Dbase, const __grid_constant__ I3Fx I3,
-                                                   __nv_bfloat16* __restrict__ X) {
+                                                   int64_t M, KG g, int Dbase, double gamma,
+                                                   const __grid_constant__ I3Mat I3, __nv_bfloat16* __restrict__ X) {
   using Z = Sz<DIM, NP>;
-  constexpr int N = Z::N, NV = Z::NV, EPB = FeatBlk<DIM, NP>::EPB, PT = FeatBlk<DIM, NP>::PT, BT = FT_T;
+  constexpr int N = Z::N, NV = Z::NV, EPB = FeatBlk<DIM, NP>::EPB, BT = FT_T;
   constexpr int NZ = DIM == 2 ? 1 : NP;        // z-slices
   constexpr int S = DIM == 2 ? 9 : 27;         // sample points, t = s0 + 3 s1 (+ 9 s2)
   constexpr int IN = 2 * S + 1, L = N / NP;    // lines along x
   constexpr int AS = N > 9 * NZ ? N : 9 * NZ, BS = 3 * L > S ? 3 * L : S;
-  __shared__ int2 sa[EPB * NV * AS];
-  __shared__ long long sb[EPB * NV * BS];
-  __shared__ uint32_t se[EPB * FX_GROUPS];
+  __shared__ ff sa[EPB * NV * AS], sb[EPB * NV * BS];
+  __shared__ ff smean[EPB][2], sfac[EPB][2];
   const int tid = threadIdx.x;
   const int64_t e0 = int64_t(blockIdx.x) * EPB;
   const int ne = int((M - e0) < EPB ? (M - e0) : EPB);
-  for (int k = tid; k < EPB * FX_GROUPS; k += BT) se[k] = 0u;
+  // the block's state is one contiguous piece of memory
+  for (int k = tid; k < ne * NV * N; k += BT) sa[k / N * AS + k % N] = ff_from_double(u[e0 * NV * N + k]);
   __syncthreads();
-  {
-    double q[PT][NV];
-#pragma unroll
-    for (int p = 0; p < PT; ++p) {
-      const int k = tid + p * BT, le = k / N, i = k % N;
-#pragma unroll
-      for (int v = 0; v < NV; ++v) q[p][v] = le < ne ? u[((e0 + le) * NV + v) * N + i] : 0.0;
-    }
-#pragma unroll
-    for (int p = 0; p < PT; ++p) {
-      const int k = tid + p * BT, le = k / N, i = k % N;
-      uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
-#pragma unroll
-      for (int v = 0; v < NV; ++v) w[fx_group(v, NV)] = max(w[fx_group(v, NV)], fx_mag(q[p][v]));
-      fx_group_max<N>(w[0], w[1], w[2], i, le < ne, se + (le < ne ? le : 0) * FX_GROUPS);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int p = 0; p < PT; ++p) {
-      const int k = tid + p * BT, le = k / N, i = k % N;
-      if (le >= ne) continue;
-#pragma unroll
-      for (int v = 0; v < NV; ++v)
-        sa[(le * NV + v) * AS + i] = fx_limbs(q[p][v], fx_exp(se[le * FX_GROUPS + fx_group(v, NV)]));
-    }
-  }
-  __syncthreads();
-  FxAcc a[3];
-  int2* sbl = reinterpret_cast<int2*>(sb);
+  ff a[3];
   // along x: b[line][s0]
   for (int k = tid; k < ne * NV * L; k += BT) {
     const int r = k / L, l = k % L;
     interp3<NP>(I3, sa + r * AS + l * NP, 1, a);
 #pragma unroll
-    for (int s = 0; s < 3; ++s) sbl[r * BS + l * 3 + s] = interp_limbs(a[s]);
+    for (int s = 0; s < 3; ++s) sb[r * BS + l * 3 + s] = a[s];
   }
   __syncthreads();
   // along y: a[i2][s1][s0], in 2D the samples
   for (int k = tid; k < ne * NV * NZ * 3; k += BT) {
     const int r = k / (NZ * 3), i2 = (k / 3) % NZ, s0 = k % 3;
-    interp3<NP>(I3, sbl + r * BS + i2 * NP * 3 + s0, 3, a);
+    interp3<NP>(I3, sb + r * BS + i2 * NP * 3 + s0, 3, a);
 #pragma unroll
-    for (int s = 0; s < 3; ++s) {
-      if (DIM == 2)
-        reinterpret_cast<long long*>(sa)[r * AS + s * 3 + s0] = fx_sum(a[s]);
-      else
-        sa[r * AS + i2 * 9 + s * 3 + s0] = interp_limbs(a[s]);
-    }
+    for (int s = 0; s < 3; ++s) sa[r * AS + i2 * 9 + s * 3 + s0] = a[s];
   }
   __syncthreads();
-  const long long* sv = reinterpret_cast<const long long*>(sa);
+  ff* sv = sa;  // the samples
   int VS = AS;
   if (DIM == 3) {
-    // along z: the samples
     for (int k = tid; k < ne * NV * 9; k += BT) {
       const int r = k / 9, s01 = k % 9;
       interp3<NP>(I3, sa + r * AS + s01, 9, a);
 #pragma unroll
-      for (int s = 0; s < 3; ++s) sb[r * BS + s * 9 + s01] = fx_sum(a[s]);
+      for (int s = 0; s < 3; ++s) sb[r * BS + s * 9 + s01] = a[s];
     }
     __syncthreads();
     sv = sb;
     VS = BS;
   }
-  const int lane = tid & 31, t = lane < S ? lane : S - 1;
-  for (int l = tid >> 5; l < ne; l += BT / 32) {
-    const uint32_t* ge = se + l * FX_GROUPS;
-    const bool badr = ge[0] >= FX_E_BAD, badp = badr || ge[1] >= FX_E_BAD || ge[2] >= FX_E_BAD;
-    const long long* H = sv + l * NV * VS + t;
-    // density: S q_t - sum over the sum, both exact integers (27 2^58 < 2^63)
-    const long long hr = H[0];
-    long long sr = lane < S ? hr : 0;
+  // pressure of every sample, in the place of its energy
+  const ff gm1 = ff_from_double(gamma - 1.0), half = {0.5f, 0.f}, zero = {0.f, 0.f};
+  for (int k = tid; k < ne * S; k += BT) {
+    const int l = k / S, t = k % S;
+    ff* q = sv + l * NV * VS + t;
+    ff ke = zero;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sr += __shfl_xor_sync(~0u, sr, o);
-    // pressure over (gamma - 1) in units of the energy: e - |m|^2 / (2 rho), the squared momentum's
-    // unit over those of density and energy being 2^(2 Em - Er - Ee)
-    ff m2 = {0.f, 0.f};
-#pragma unroll
-    for (int b = 0; b < DIM; ++b) {
-      const ff m = ff_from_fixed(H[(1 + b) * VS]);
-      m2 = fma_t(m, m, m2);
+    for (int v = 1; v < NV - 1; ++v) {
+      const ff c = q[v * VS];
+      ke = fma_t(c, c, ke);
     }
-    int k = 2 * fx_exp(ge[1]) - fx_exp(ge[0]) - fx_exp(ge[2]) - 1;
-    k = k < -126 ? -126 : (k > 127 ? 127 : k);
-    const float sc = __int_as_float((k + 127) << 23);
-    const ff ke = ff_div(m2, ff_from_fixed(hr));
-    const ff p = ff_from_fixed(H[(NV - 1) * VS]) - ff{ke.h * sc, ke.l * sc};
-    ff ps = lane < S ? p : ff{0.f, 0.f};
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      ps = ps + ff{__shfl_xor_sync(~0u, ps.h, o), __shfl_xor_sync(~0u, ps.l, o)};
-    // 100 (p_t - mean) / mean = (S p_t - sum) 100 / sum
-    const ff dp = ff{float(S), 0.f} * p - ps;
-    const float nan = __int_as_float(0x7FC00000);
-    if (lane < S) {
-      __nv_bfloat16* x = X + (e0 + l) * IN;
-      x[t] = __float2bfloat16_rn(badr ? nan : __ll2float_rn(S * hr - sr) * (100.f / __ll2float_rn(sr)));
-      x[S + t] = __float2bfloat16_rn(badp ? nan : (dp.h + dp.l) * (100.f / ps.h));
-      if (t == 0) {
-        const int span = g.Dmax - Dbase > 0 ? g.Dmax - Dbase : 1;
-        x[2 * S] = __float2bfloat16_rn(float(g.depth(keys[e0 + l]) - Dbase) / float(span));
-      }
+    q[(NV - 1) * VS] = gm1 * (q[(NV - 1) * VS] - half * ke / q[0]);
+  }
+  __syncthreads();
+  // means of density and pressure; 100 (q_t - mean) / mean = (q_t - mean) * (100 S / sum)
+  for (int k = tid; k < ne * 2; k += BT) {
+    const int l = k >> 1, w = k & 1;
+    const ff* q = sv + (l * NV + (w ? NV - 1 : 0)) * VS;
+    ff sum = zero;
+    for (int t = 0; t < S; ++t) sum = sum + q[t];
+    sfac[l][w] = ff_from_double(100.0 * S) / sum;
+    smean[l][w] = sum * ff_from_double(1.0 / S);
+  }
+  __syncthreads();
+  for (int k = tid; k < ne * S; k += BT) {
+    const int l = k / S, t = k % S;
+    const ff* q = sv + l * NV * VS + t;
+    const ff dr = (q[0] - smean[l][0]) * sfac[l][0], dp = (q[(NV - 1) * VS] - smean[l][1]) * sfac[l][1];
+    __nv_bfloat16* x = X + (e0 + l) * IN;
+    x[t] = __float2bfloat16_rn(dr.h + dr.l);
+    x[S + t] = __float2bfloat16_rn(dp.h + dp.l);
+    if (t == 0) {
+      const int span = g.Dmax - Dbase > 0 ? g.Dmax - Dbase : 1;
+      x[2 * S] = __float2bfloat16_rn(float(g.depth(keys[e0 + l]) - Dbase) / float(span));
     }
   }
 }
@@ -444,6 +385,32 @@ __global__ void __launch_bounds__(TC_ROWS) k_mlp_forward_tc(const float* __restr
   }
 }
 
+// Labels of each class, and those outside -1..1, of a batch: cnt[0..3]
+__global__ void __launch_bounds__(256) k_label_count(const int8_t* __restrict__ y, int64_t B,
+                                                     unsigned long long* __restrict__ cnt) {
+  int c[4] = {0, 0, 0, 0};
+  for (int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x; i < B; i += int64_t(gridDim.x) * 256) {
+    const int k = int(y[i]) + 1;
+    c[0] += k == 0;
+    c[1] += k == 1;
+    c[2] += k == 2;
+    c[3] += k < 0 || k > 2;
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int n = __reduce_add_sync(0xffffffffu, c[k]);
+    if (n && (threadIdx.x & 31) == 0) atomicAdd(&cnt[k], (unsigned long long)n);
+  }
+}
+// total class weight of the batch, and its inverse (or the caller's)
+__device__ __forceinline__ double class_weight(const unsigned long long* cnt, float cw0, float cw1, float cw2) {
+  return double(cnt[0]) * cw0 + double(cnt[1]) * cw1 + double(cnt[2]) * cw2;
+}
+__device__ __forceinline__ float inverse_weight(const unsigned long long* cnt, float cw0, float cw1, float cw2,
+                                                float inv_given) {
+  return inv_given != 0.f ? inv_given : float(1.0 / class_weight(cnt, cw0, cw1, cw2));
+}
+
 // Tensor-core training: gradient of the weighted mean softmax cross-entropy over a batch.  Each
 // block (one per SM: 206 KB of shared memory, all 512 tensor-memory columns) loops over tiles of
 // 128 samples.  Forward as in inference, keeping every layer's input A_l in shared memory both row
@@ -469,12 +436,12 @@ constexpr int TG_W1 = 0, TG_W2 = 8192, TG_W3 = 16384, TG_W4 = 24576, TG_W2T = 26
 __global__ void __launch_bounds__(TG_T) k_mlp_grad_tc(const float* __restrict__ P, int in,
                                                       const __nv_bfloat16* __restrict__ X,
                                                       const int8_t* __restrict__ y, int64_t B, float cw0,
-                                                      float cw1, float cw2, float* __restrict__ Gp,
-                                                      float* __restrict__ Lp, int* __restrict__ Cp,
+                                                      float cw1, float cw2, float inv_given,
+                                                      const unsigned long long* __restrict__ cnt,
+                                                      float* __restrict__ Gp, float* __restrict__ Lp,
                                                       int* __restrict__ status) {
   extern __shared__ unsigned char sm_raw[];
   unsigned char* sm = sm_raw + ((1024 - (tc::smem_addr(sm_raw) & 1023)) & 1023);
-  __shared__ int s_cnt[4];
   // thread t: row `row` of the tile (its warp's tensor-memory quarter), columns c0 .. c0 + 15
   const int t = threadIdx.x, warp = t >> 5, row = (warp & 3) * 32 + (t & 31), c0 = (warp >> 2) * 16;
   const Lay L = lay(in);
@@ -482,7 +449,7 @@ __global__ void __launch_bounds__(TG_T) k_mlp_grad_tc(const float* __restrict__ 
   auto put = [&](int off, uint32_t o, float v) {
     *reinterpret_cast<__nv_bfloat16*>(sm + off + o) = __float2bfloat16_rn(v);
   };
-  if (t < 4) s_cnt[t] = 0;
+  const float inv_wsum = inverse_weight(cnt, cw0, cw1, cw2, inv_given);
   // weights (BF16, zero padding) and their transposes for the backward products
   for (int idx = t; idx < H * 64; idx += TG_T) {
     const int o = idx >> 6, k = idx & 63;
@@ -563,7 +530,6 @@ __global__ void __launch_bounds__(TG_T) k_mlp_grad_tc(const float* __restrict__ 
     *reinterpret_cast<uint4*>(sm + rows + tc::canon_off(row, c0)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
     *reinterpret_cast<uint4*>(sm + rows + tc::canon_off(row, c0 + 8)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
   };
-  int cnt[4] = {0, 0, 0, 0};  // labels of each class, and labels outside -1..1
   auto sum_dzt_row = [&](int o) {  // fixed-order sum over the 128 samples of row o of DZT
     float acc = 0.f;
     for (int j = 0; j < TG_ROWS; j += 8) {
@@ -622,8 +588,7 @@ __global__ void __launch_bounds__(TG_T) k_mlp_grad_tc(const float* __restrict__ 
       tc::tmem_wait_ld();
       float dz[NOUT] = {0.f, 0.f, 0.f};
       const int cls = valid ? int(y[row0 + row]) + 1 : 0;
-      if (valid && (cls < 0 || cls >= NOUT)) ++cnt[3];
-      if (valid && cls >= 0 && cls < NOUT) {
+      if (valid && cls >= 0 && cls < NOUT) {  // any other label stops the update in the reduction
         float o[NOUT];
 #pragma unroll
         for (int c = 0; c < NOUT; ++c) o[c] = __uint_as_float(r[c]) + sb[3 * H + c];
@@ -632,13 +597,9 @@ __global__ void __launch_bounds__(TG_T) k_mlp_grad_tc(const float* __restrict__ 
         const float e0 = expf(o[0] - mx), e1 = expf(o[1] - mx), e2 = expf(o[2] - mx);
         const float sum = e0 + e1 + e2;
         const float pz[NOUT] = {e0 / sum, e1 / sum, e2 / sum};
-        // unnormalised: the batch's total weight divides the sums in the reduction
-        loss += -w * logf(cls == 0 ? pz[0] : (cls == 1 ? pz[1] : pz[2]));
+        loss += -w * inv_wsum * logf(cls == 0 ? pz[0] : (cls == 1 ? pz[1] : pz[2]));
 #pragma unroll
-        for (int c = 0; c < NOUT; ++c) {
-          dz[c] = w * (pz[c] - (c == cls ? 1.f : 0.f));
-          cnt[c] += c == cls;
-        }
+        for (int c = 0; c < NOUT; ++c) dz[c] = w * inv_wsum * (pz[c] - (c == cls ? 1.f : 0.f));
       }
       for (int c = 0; c < 16; ++c) put(TG_DZ, tc::canon_off(row, c), c < NOUT ? dz[c] : 0.f);
       for (int c = 0; c < NOUT; ++c) put(TG_DZT, tc::canon_off_w(c, row, 128), dz[c]);
@@ -709,20 +670,16 @@ __global__ void __launch_bounds__(TG_T) k_mlp_grad_tc(const float* __restrict__ 
     }
     if (t < NOUT) g[L.ob4 + t] = db[3];
   }
-  // loss: warp sums, then the four warps that hold it in order; label counts
+  // loss: warp sums, then the four warps that hold it in order
   float* red = reinterpret_cast<float*>(sm + TG_BIAS);
   __syncthreads();
   if (warp < 4) {
 #pragma unroll
     for (int w = 16; w > 0; w >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, w);
     if ((t & 31) == 0) red[warp] = loss;
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-      if (cnt[c]) atomicAdd(&s_cnt[c], cnt[c]);
   }
   __syncthreads();
   if (t == 0) Lp[blockIdx.x] = red[0] + red[1] + red[2] + red[3];
-  if (t < 4) Cp[blockIdx.x * 4 + t] = s_cnt[t];
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) {
@@ -731,46 +688,31 @@ __global__ void __launch_bounds__(TG_T) k_mlp_grad_tc(const float* __restrict__ 
   }
 }
 
-// Sums of the blocks' partial gradients and losses (a fixed order), divided by the batch's total class
-// weight (from the exact label counts, unless the caller gives its inverse), then either stored (G) or
-// applied by Adam (Kingma & Ba): m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
-// p -= lr mhat / (sqrt(vhat) + eps).  A wait that gave up in the gradient kernel, a label outside
-// -1..1 (status 2) or a total weight of zero (status 4) leaves everything unchanged.
+// Sums of the blocks' partial gradients and losses, in block order, stored (G) or applied by Adam
+// (Kingma & Ba): m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2, p -= lr mhat / (sqrt(vhat) + eps).  A wait
+// that gave up in the gradient kernel, a label outside -1..1 (status 2) or a total weight of zero (status
+// 4) leaves everything unchanged.
 struct AdamArgs {
   float *P, *m, *v;
   float lr, b1, b2, eps, c1, c2;
 };
 constexpr int RED_T = 64;
 __global__ void __launch_bounds__(RED_T) k_grad_reduce(const float* __restrict__ Gp, const float* __restrict__ Lp,
-                                                       const int* __restrict__ Cp, int nblk, int total, float cw0,
-                                                       float cw1, float cw2, float inv_given, float* __restrict__ G,
-                                                       float* __restrict__ loss, AdamArgs A, int* __restrict__ status) {
-  __shared__ int s_cnt[4];
+                                                       int nblk, int total, float cw0, float cw1, float cw2,
+                                                       float inv_given, const unsigned long long* __restrict__ cnt,
+                                                       float* __restrict__ G, float* __restrict__ loss, AdamArgs A,
+                                                       int* __restrict__ status) {
   const int t = threadIdx.x, p = blockIdx.x * RED_T + t;
-  if (t < 4) s_cnt[t] = 0;
-  __syncthreads();
-  for (int k = t; k < nblk * 4; k += RED_T) {
-    const int c = Cp[k];
-    if (c) atomicAdd(&s_cnt[k & 3], c);
-  }
-  __syncthreads();
-  const double ws = double(s_cnt[0]) * cw0 + double(s_cnt[1]) * cw1 + double(s_cnt[2]) * cw2;
-  const int bad = s_cnt[3] ? 2 : (inv_given == 0.f && ws == 0.0 ? 4 : 0);
+  const int bad = cnt[3] ? 2 : (inv_given == 0.f && class_weight(cnt, cw0, cw1, cw2) == 0.0 ? 4 : 0);
   if (bad) {
     if (blockIdx.x == 0 && t == 0) atomicOr(status, bad);
     return;
   }
   if (*status & 1) return;  // set before this kernel only
-  const float inv = inv_given != 0.f ? inv_given : float(1.0 / ws);
   if (p < total) {
-    float a[4] = {0.f, 0.f, 0.f, 0.f};
-    int c = 0;
-#pragma unroll 2
-    for (; c + 4 <= nblk; c += 4)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) a[j] += Gp[int64_t(c + j) * total + p];
-    for (; c < nblk; ++c) a[0] += Gp[int64_t(c) * total + p];
-    const float g = ((a[0] + a[1]) + (a[2] + a[3])) * inv;
+    float g = 0.f;
+#pragma unroll 8
+    for (int c = 0; c < nblk; ++c) g += Gp[int64_t(c) * total + p];
     if (G) {
       G[p] = g;
     } else {
@@ -781,12 +723,11 @@ __global__ void __launch_bounds__(RED_T) k_grad_reduce(const float* __restrict__
       A.P[p] -= A.lr * (mt / A.c1) / (sqrtf(vt / A.c2) + A.eps);
     }
   }
-  if (blockIdx.x == 0 && t < 32 && loss) {
+  if (p == 0 && loss) {
     float a = 0.f;
-    for (int c = t; c < nblk; c += 32) a += Lp[c];
-#pragma unroll
-    for (int w = 16; w > 0; w >>= 1) a += __shfl_xor_sync(0xffffffffu, a, w);
-    if (t == 0) *loss = a * inv;
+#pragma unroll 8
+    for (int c = 0; c < nblk; ++c) a += Lp[c];
+    *loss = a;
   }
 }
 
@@ -834,30 +775,22 @@ int mlp_in_dim(int dim) { return 2 * (dim == 2 ? 9 : 27) + 1; }
 int mlp_features(int dim, int p, const double* u, const uint64_t* keys, int64_t M, const KG& g,
                  int Dbase, double gamma, const DevOps& ops, void* d_X, cudaStream_t s, Err* err) {
   if (M <= 0) return 0;
-  (void)gamma;  // the features are relative: gamma - 1 cancels
   // Lagrange basis of the element's points evaluated at the 3-point Gauss-Legendre nodes
-  I3Fx I3{};
+  I3Mat I3{};
   const double g3[3] = {-std::sqrt(0.6), 0.0, std::sqrt(0.6)};
-  const int np = p + 1;
-  double c[3][NPMAX], sum = 0.0;
-  for (int t = 0; t < 3; ++t) {
-    double st = 0.0;
+  int np = p + 1;
+  for (int t = 0; t < 3; ++t)
     for (int j = 0; j < np; ++j) {
       double pr = 1.0;
       for (int k = 0; k < np; ++k)
         if (k != j) pr *= (g3[t] - ops.x[k]) / (ops.x[j] - ops.x[k]);
-      c[t][j] = pr;
-      st += std::fabs(pr);
+      const float h = float(pr);  // double-word constant: hi + lo
+      I3.m[t][j] = ff{h, float(pr - double(h))};
     }
-    sum = st > sum ? st : sum;
-  }
-  const int kI = fx_scale(sum);
-  for (int t = 0; t < 3; ++t)
-    for (int j = 0; j < np; ++j) I3.c[t][j] = fx_coef(c[t][j], kI);
   __nv_bfloat16* X = static_cast<__nv_bfloat16*>(d_X);
 #define FEAT(D_, N_)                                                                                        \
   k_features<D_, N_><<<unsigned((M + FeatBlk<D_, N_>::EPB - 1) / FeatBlk<D_, N_>::EPB), FT_T, 0, s>>>(u, keys, M, g, \
-                                                                                                       Dbase, I3, X)
+                                                                                                       Dbase, gamma, I3, X)
   if (dim == 2) {
     if (np == 2) FEAT(2, 2); else if (np == 3) FEAT(2, 3); else if (np == 4) FEAT(2, 4); else FEAT(2, 5);
   } else {
@@ -869,7 +802,7 @@ int mlp_features(int dim, int p, const double* u, const uint64_t* keys, int64_t 
 }
 
 // Gradient and loss of one batch on the tensor cores, stored into G or (G null) applied by Adam.  The
-// label counts that normalise the sums come from the gradient kernel; cw[3] != 0 gives 1 / sum_b w_{y_b}
+// labels are counted first for the factor that normalises them; cw[3] != 0 gives 1 / sum_b w_{y_b}
 // instead.  Synchronises: the status word is read at the end.
 static int grad_step(const float* d_params, int in, const void* d_X, const int8_t* d_y, int64_t B, const float* cw,
                      float* G, float* d_loss, const AdamArgs& adam, Alloc& A, cudaStream_t s, Err* err) {
@@ -883,18 +816,21 @@ static int grad_step(const float* d_params, int in, const void* d_X, const int8_
   const int grid = int(ntiles < sms ? ntiles : sms);  // one block per SM (shared memory, TMEM)
   // one block of scratch: status word, label counts, losses, partial gradients
   Scratch S(&A);
-  int* st = S.get<int>(64 + size_t(grid) * (5 + size_t(L.total)));
+  int* st = S.get<int>(64 + size_t(grid) * (1 + size_t(L.total)));
   if (!st) return set_error(err, FR_ENOMEM, "training scratch");
-  int* Cp = st + 64;
-  float* Lp = reinterpret_cast<float*>(Cp + size_t(grid) * 4);
+  unsigned long long* cnt = reinterpret_cast<unsigned long long*>(st + 2);
+  float* Lp = reinterpret_cast<float*>(st + 64);
   float* Gp = Lp + grid;
-  FR_CUDA(err, cudaMemsetAsync(st, 0, 4, s));
+  FR_CUDA(err, cudaMemsetAsync(st, 0, 64 * sizeof(int), s));
+  const int64_t nc = (B + 2047) / 2048;  // eight labels a thread
+  k_label_count<<<unsigned(nc < 4 * sms ? nc : 4 * sms), 256, 0, s>>>(d_y, B, cnt);
+  FR_LAUNCH_CHECK(err);
   FR_CUDA(err, cudaFuncSetAttribute(k_mlp_grad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_SMEM));
   k_mlp_grad_tc<<<unsigned(grid), TG_T, TG_SMEM, s>>>(d_params, in, static_cast<const __nv_bfloat16*>(d_X), d_y, B,
-                                                      cw[0], cw[1], cw[2], Gp, Lp, Cp, st);
+                                                      cw[0], cw[1], cw[2], cw[3], cnt, Gp, Lp, st);
   FR_LAUNCH_CHECK(err);
-  k_grad_reduce<<<unsigned((L.total + RED_T - 1) / RED_T), RED_T, 0, s>>>(Gp, Lp, Cp, grid, L.total, cw[0], cw[1], cw[2],
-                                                                          cw[3], G, d_loss, adam, st);
+  k_grad_reduce<<<unsigned((L.total + RED_T - 1) / RED_T), RED_T, 0, s>>>(Gp, Lp, grid, L.total, cw[0], cw[1], cw[2],
+                                                                          cw[3], cnt, G, d_loss, adam, st);
   FR_LAUNCH_CHECK(err);
   int h = 0;
   FR_CUDA(err, cudaMemcpyAsync(&h, st, 4, cudaMemcpyDeviceToHost, s));
