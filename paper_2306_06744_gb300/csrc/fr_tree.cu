@@ -216,7 +216,7 @@ __global__ void k_edit_write(const uint64_t* __restrict__ k, const int8_t* __res
 // Of the 3^dim-1 neighbour boxes only the 2^dim-1 that lie outside the leaf's parent in a set of axes,
 // each away from the parent's centre, are looked up: the others lie in the parent (whose cells are never
 // coarser than D) or share their depth-(D-1) cell with one of these, so that the leaf containing them
-// and the path to it are the same.  (600k points of a 3D torus, 829k leaves: see k_bal_gen_fast.)
+// and the path to it are the same.
 template <int DIM>
 struct Nofs {
   static constexpr int value = (1 << DIM) - 1;
@@ -466,6 +466,9 @@ __global__ void k_merge_write(const uint64_t* __restrict__ k, const int64_t* __r
 // (equal keys lie in the same leaf), and the sort kernel then reads the containing leaf instead of
 // searching for it.
 constexpr int PACK_BITS = 21;  // leaf indices below 2^21 (meshes of this path hold at most 2^20)
+// Balance of the 829k leaves of 600k points on a 3D torus, all passes' generation kernels: 26 boxes a leaf
+// and a warp for every leaf 3.27 ms (a first pass that was counted and generated again included), 7 boxes
+// and 8 lanes 0.69 ms, only the depth's own leaves 0.45 ms.
 template <int DIM>
 __global__ void k_bal_gen_fast(const uint64_t* __restrict__ k, int64_t* __restrict__ ctl, int64_t n_ub, KG g,
                                int D, uint64_t* __restrict__ out, int64_t cap, bool packed, int sn, int sg,
@@ -474,60 +477,79 @@ __global__ void k_bal_gen_fast(const uint64_t* __restrict__ k, int64_t* __restri
   __shared__ uint64_t s_tab[KEY_INDEX_MAX];
   constexpr int LPL = BalLanes<DIM>::value;
   constexpr int NC = 1 << DIM;
-  const int64_t gt = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t i = gt / LPL;
-  const int o = int(gt % LPL);
-  const int64_t n = ctl[CTL_OVER] == 0 ? ctl[sn] : 0;
-  // the key index is staged only by blocks that hold a depth-D leaf (the others search nothing)
-  const bool deep = i < n_ub && i < n && g.depth(k[i]) == D;
-  int m = 0;
-  if (__syncthreads_or(deep)) m = stage_key_index(X, n, s_tab);
-  uint32_t N[3];
-  int dA = 0;
-  int64_t jA = 0;
-  const bool gen = deep && bal_lane<DIM>(k, n, g, D, i, o, N, &dA, &jA, s_tab, m, X.sh) > 0;
-  // A lane emits the 2^dim children of its box's ancestor at each depth l-1, l = dA+1 .. D-1.
-  // Lanes of a warp whose boxes share that ancestor (neighbouring leaves looking into the same
-  // coarse leaf) would emit the same octants: per depth only the lowest such lane emits them, so
-  // the set of octants is unchanged and the sort and merge see fewer copies.
-  const int lane = int(threadIdx.x & 31);
-  const int l0 = int(__reduce_min_sync(0xffffffffu, unsigned(gen ? dA + 1 : D)));
-  const uint64_t rawN = gen ? interleave<DIM>(N) : 0ull;
-  uint32_t lead = 0;  // bit l - l0: this lane emits depth l's octants
-  int c = 0;
-  for (int l = l0; l <= D - 1; ++l) {
-    const bool act = gen && l > dA;
-    const uint64_t span = vol_raw<DIM>(g, l - 1);
-    // an ancestor key never equals the all-ones value of the lanes that emit nothing
-    const uint64_t anc = act ? g.make(rawN / span * span, l - 1) : ~0ull;
-    const unsigned same = __match_any_sync(0xffffffffu, anc);
-    if (act && lane == __ffs(same) - 1) {
-      lead |= 1u << (l - l0);
-      c += NC;
-    }
+  __shared__ int s_list[TB], s_n;
+  // The block's leaves, one per thread; those at depth D are listed in order and then taken by groups of
+  // lanes.  Most leaves of most passes are not at depth D: with a group of lanes for every leaf the grid
+  // was eight (four) times as large and idle but for them.
+  const int tid = int(threadIdx.x), lane = tid & 31;
+  const int64_t i0 = int64_t(blockIdx.x) * TB;
+  const int64_t n = ctl[CTL_OVER] == 0 ? min(ctl[sn], n_ub) : 0;
+  const bool mine = i0 + tid < n && g.depth(k[i0 + tid]) == D;
+  if (tid == 0) s_n = 0;
+  const int cnt = __syncthreads_count(mine);
+  if (cnt == 0) return;
+  const int m = stage_key_index(X, n, s_tab);  // ends with a barrier
+  {
+    // ascending places inside a warp keep neighbouring leaves together (their lanes share ancestors)
+    const unsigned b = __ballot_sync(0xffffffffu, mine);
+    int at = 0;
+    if (lane == 0 && b) at = atomicAdd(&s_n, __popc(b));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & ((1u << lane) - 1u));
+    if (mine) s_list[at] = tid;
   }
-  // every lane of the warp takes part: inclusive prefix of the counts, one atomic per warp
-  int incl = c;
-#pragma unroll
-  for (int w = 1; w < 32; w <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, w);
-    if (lane >= w) incl += y;
-  }
-  const int tot = __shfl_sync(0xffffffffu, incl, 31);
-  unsigned long long base = 0;
-  if (lane == 31 && tot > 0) base = atomicAdd(reinterpret_cast<unsigned long long*>(ctl + sg), (unsigned long long)tot);
-  base = __shfl_sync(0xffffffffu, base, 31);
-  if (c == 0) return;
-  int64_t q = int64_t(base) + (incl - c);
-  for (int l = l0; l <= D - 1; ++l) {
-    if (!((lead >> (l - l0)) & 1u)) continue;
-    const uint64_t span = vol_raw<DIM>(g, l - 1);
-    const uint64_t anc = g.make(rawN / span * span, l - 1);
-    for (int ch = 0; ch < NC; ++ch, ++q)
-      if (q < cap) {  // past the capacity: counted, not stored
-        const uint64_t ck = child_key<DIM>(g, anc, ch);
-        out[q] = packed ? (ck << PACK_BITS) | uint64_t(jA) : ck;
+  __syncthreads();
+  for (int j0 = 0; j0 < cnt; j0 += TB / LPL) {  // uniform over the block
+    const int j = j0 + tid / LPL, o = tid % LPL;
+    const int64_t i = i0 + (j < cnt ? s_list[j] : 0);
+    uint32_t N[3];
+    int dA = 0;
+    int64_t jA = 0;
+    const bool gen = j < cnt && bal_lane<DIM>(k, n, g, D, i, o, N, &dA, &jA, s_tab, m, X.sh) > 0;
+    // A lane emits the 2^dim children of its box's ancestor at each depth l-1, l = dA+1 .. D-1.
+    // Lanes of a warp whose boxes share that ancestor (neighbouring leaves looking into the same
+    // coarse leaf) would emit the same octants: per depth only the lowest such lane emits them, so
+    // the set of octants is unchanged and the sort and merge see fewer copies.
+    const int l0 = int(__reduce_min_sync(0xffffffffu, unsigned(gen ? dA + 1 : D)));
+    const uint64_t rawN = gen ? interleave<DIM>(N) : 0ull;
+    uint32_t lead = 0;  // bit l - l0: this lane emits depth l's octants
+    int c = 0;
+    for (int l = l0; l <= D - 1; ++l) {
+      const bool act = gen && l > dA;
+      const uint64_t span = vol_raw<DIM>(g, l - 1);
+      // an ancestor key never equals the all-ones value of the lanes that emit nothing
+      const uint64_t anc = act ? g.make(rawN / span * span, l - 1) : ~0ull;
+      const unsigned same = __match_any_sync(0xffffffffu, anc);
+      if (act && lane == __ffs(same) - 1) {
+        lead |= 1u << (l - l0);
+        c += NC;
       }
+    }
+    // every lane of the warp takes part: inclusive prefix of the counts, one atomic per warp
+    int incl = c;
+#pragma unroll
+    for (int w = 1; w < 32; w <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, w);
+      if (lane >= w) incl += y;
+    }
+    const int tot = __shfl_sync(0xffffffffu, incl, 31);
+    unsigned long long base = 0;
+    if (lane == 31 && tot > 0)
+      base = atomicAdd(reinterpret_cast<unsigned long long*>(ctl + sg), (unsigned long long)tot);
+    base = __shfl_sync(0xffffffffu, base, 31);
+    if (c > 0) {
+      int64_t q = int64_t(base) + (incl - c);
+      for (int l = l0; l <= D - 1; ++l) {
+        if (!((lead >> (l - l0)) & 1u)) continue;
+        const uint64_t span = vol_raw<DIM>(g, l - 1);
+        const uint64_t anc = g.make(rawN / span * span, l - 1);
+        for (int ch = 0; ch < NC; ++ch, ++q)
+          if (q < cap) {  // past the capacity: counted, not stored
+            const uint64_t ck = child_key<DIM>(g, anc, ch);
+            out[q] = packed ? (ck << PACK_BITS) | uint64_t(jA) : ck;
+          }
+      }
+    }
+    __syncwarp();
   }
 }
 
@@ -1408,7 +1430,7 @@ int tree_balance(int dim, const KG& g, int Dhigh, int Dlow, Buf<uint64_t>& keys,
       rc = set_error(err, FR_ENOMEM, "balance scratch");
       break;
     }
-    DIM_DISPATCH(dim, (launch_dependent(k_bal_gen_fast<D_>, nblk(n_ub * BalLanes<D_>::value), TB, s, keys.p, d_ctl,
+    DIM_DISPATCH(dim, (launch_dependent(k_bal_gen_fast<D_>, nblk(n_ub), TB, s, keys.p, d_ctl,
                                         n_ub, g, D, gen.p, capG, false, int(CTL_N), int(CTL_G), KeyIndex{})));
     ++launch_counter();
     if ((rc = cudaGetLastError() != cudaSuccess ? set_error(err, FR_ECUDA, "k_bal_gen_fast") : 0)) break;
@@ -1486,7 +1508,7 @@ int tree_balance_async(int dim, const KG& g, int Dlow, Buf<uint64_t>& keys, int6
       rc = set_error(err, FR_ENOMEM, "balance scratch");
       break;
     }
-    DIM_DISPATCH(dim, (launch_dependent(k_bal_gen_fast<D_>, nblk(nb * BalLanes<D_>::value), TB, s, keys.p, d_ctl, nb, g,
+    DIM_DISPATCH(dim, (launch_dependent(k_bal_gen_fast<D_>, nblk(nb), TB, s, keys.p, d_ctl, nb, g,
                                         D, gen.p, cap, packed, sn, sg, *X)));
     ++launch_counter();
     if (packed) {
