@@ -439,14 +439,15 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_transfer(KG g, const uint64
 // partials, so the sums are the same on every run.  The closed form does not depend on z, so its
 // density is formed once per column, and a vortex whose temperature term is below 2^-60 of the
 // background at a point is left out there (it cannot change the sum): what is left is the pressure, the
-// weighted sums and, near a vortex, one exponential and one power per column.  FP64-bound: four 3D
-// p = 3 tubes of 242k leaves, 11.5 ms with one thread per element and the closed form at every point.
+// weighted sums and, near a vortex, an exponential and a power per column.  FP64-bound.  One thread per
+// element with the whole closed form at every point took 11.5 ms for four 3D p = 3 tubes of 242k leaves and
+// 120 us for the 2D p = 3 run; so: 1.49 ms and 57 us.
 constexpr int NRM_T = 128, NRM_W = 8, NRM_GRID = 152 * 8;
 // the closed form's density, as far as norms need it
 struct NormVort {
   int n;
   double x[16], y[16], coef[16], iR2[16], r2max[16];  // centre at time t; dT = -coef exp(1 - r2)
-  double L, iL, Tinf, rho_inf, ex, gm1;
+  double L, iL, Tinf, iTinf, rho_inf, ex, gm1;
 };
 inline NormVort norm_vort(const DevProblem& P, double t) {
   NormVort V{};
@@ -455,6 +456,7 @@ inline NormVort norm_vort(const DevProblem& P, double t) {
   V.L = P.L;
   V.iL = 1.0 / P.L;
   V.Tinf = P.p_inf / P.rho_inf;
+  V.iTinf = P.rho_inf / P.p_inf;
   V.rho_inf = P.rho_inf;
   V.ex = 1.0 / (P.gamma - 1.0);
   V.gm1 = P.gamma - 1.0;
@@ -477,8 +479,8 @@ __device__ __forceinline__ double vortex_density(const NormVort& V, double x, do
     const double r2 = fma(dx, dx, dy * dy) * V.iR2[k];
     if (r2 < V.r2max[k]) dT = fma(-V.coef[k], exp(1.0 - r2), dT);
   }
-  const double T = V.Tinf + dT;
-  return T == V.Tinf ? V.rho_inf : V.rho_inf * pow(T / V.Tinf, V.ex);
+  // (1 + dT/Tinf)^ex through log1p: fewer operations than pow, and dT is not rounded into the sum
+  return V.Tinf + dT == V.Tinf ? V.rho_inf : V.rho_inf * exp(V.ex * log1p(dT * V.iTinf));
 }
 
 template <int DIM, int NP>
@@ -548,27 +550,26 @@ __global__ void __launch_bounds__(NRM_T) k_norms(const uint64_t* __restrict__ ke
   if (threadIdx.x < NRM_W) partial[int64_t(blockIdx.x) * NRM_W + threadIdx.x] = sm[threadIdx.x][0];
 }
 
+// thread t takes value t % 8 of the partials t / 8, t / 8 + 16, ...; then the 16 sums of a value in order
 __global__ void __launch_bounds__(NRM_T) k_norms_final(const double* __restrict__ partial,
                                                        int64_t nb, int nv, double* __restrict__ out) {
-  __shared__ double sm[NRM_W][NRM_T];
-  double acc[NRM_W];
-  for (int k = 0; k < NRM_W; ++k) acc[k] = (k == nv + 1 || k == nv + 2) ? 1e300 : 0.0;
-  for (int64_t b = threadIdx.x; b < nb; b += NRM_T)
-    for (int k = 0; k < NRM_W; ++k) {
-      double x = partial[b * NRM_W + k];
-      acc[k] = (k == nv + 1 || k == nv + 2) ? fmin(acc[k], x) : acc[k] + x;
-    }
-  for (int k = 0; k < NRM_W; ++k) sm[k][threadIdx.x] = acc[k];
-  __syncthreads();
-  for (int st = NRM_T / 2; st > 0; st >>= 1) {
-    if (int(threadIdx.x) < st)
-      for (int k = 0; k < NRM_W; ++k) {
-        double a = sm[k][threadIdx.x], b = sm[k][threadIdx.x + st];
-        sm[k][threadIdx.x] = (k == nv + 1 || k == nv + 2) ? fmin(a, b) : a + b;
-      }
-    __syncthreads();
+  __shared__ double sm[NRM_T];
+  const int k = threadIdx.x % NRM_W;
+  const bool least = k == nv + 1 || k == nv + 2;
+  double acc = least ? 1e300 : 0.0;
+  for (int64_t b = threadIdx.x / NRM_W; b < nb; b += NRM_T / NRM_W) {
+    const double x = partial[b * NRM_W + k];
+    acc = least ? fmin(acc, x) : acc + x;
   }
-  if (threadIdx.x < NRM_W) out[threadIdx.x] = sm[threadIdx.x][0];
+  sm[threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.x < NRM_W) {
+    for (int j = 1; j < NRM_T / NRM_W; ++j) {
+      const double x = sm[j * NRM_W + k];
+      acc = least ? fmin(acc, x) : acc + x;
+    }
+    out[k] = acc;
+  }
 }
 
 template <int DIM, int NP>
