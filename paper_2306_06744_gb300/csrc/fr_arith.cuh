@@ -198,15 +198,12 @@ __device__ __forceinline__ double sqrt_t(double a) {
   return fma(fma(-g, g, a), h, g);
 }
 __device__ __forceinline__ float sqrt_t(float a) { return sqrtf(a); }
-__device__ __forceinline__ double fabs_t(double a) { return fabs(a); }
 __device__ __forceinline__ float fabs_t(float a) { return fabsf(a); }
-__device__ __forceinline__ double fmax_t(double a, double b) { return fmax(a, b); }
 // the larger of two non-negative values: positive doubles order as their bit patterns, so the FP64
 // pipe is left out (a NaN wins)
 __device__ __forceinline__ double fmax_pos(double a, double b) {
   return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
 }
-__device__ __forceinline__ ff fmax_pos(ff a, ff b) { return fmax_t(a, b); }
 __device__ __forceinline__ float fmax_t(float a, float b) { return fmaxf(a, b); }
 
 // -x/2 without a multiplication where the exponent can be lowered (x normal, above 2^-1021)

@@ -178,7 +178,7 @@ __device__ __forceinline__ void rusanov2_ff(const ff* qL, const ff* qR, int axis
     }
   ff vL = mnL * rL, vR = mnR * rR;
   // |v| + c with c = sqrt(gamma) sqrt(p / rho)
-  const ff lam = fmax_pos(fma_t(sgam, sqrt_t(pL * rL), fabs_t(vL)), fma_t(sgam, sqrt_t(pR * rR), fabs_t(vR)));
+  const ff lam = fmax_t(fma_t(sgam, sqrt_t(pL * rL), fabs_t(vL)), fma_t(sgam, sqrt_t(pR * rR), fabs_t(vR)));
   // f(qL) + f(qR) - lambda (qR - qL), the sums as multiply-adds; the pressures enter the normal
   // momentum through the chain's start (a select) instead of an addition per component
   const ff pp = pL + pR;
@@ -321,10 +321,12 @@ constexpr int face_fpb(int per) {
   return best;
 }
 
-template <int DIM, int NP>
+// (FP32 at 3D p = 3, one face a block otherwise: 128 threads, two faces, take 107 instead of 119 us per
+// launch at 127k leaves; the other forms and degrees gain nothing or lose)
+template <int DIM, int NP, class A>
 struct FaceCfg {
   static constexpr int PER = (1 << (DIM - 1)) * (DIM == 2 ? NP : NP * NP);  // threads per hanging face
-  static constexpr int T0 = PER > 64 ? 128 : 64;
+  static constexpr int T0 = PER > 64 || (PER == 64 && std::is_same<A, float>::value) ? 128 : 64;
   static constexpr bool FULL = (T0 / PER) * PER * 10 >= T0 * 9;  // at most a tenth of T0 idle
   // otherwise (3D p = 2: one 36-point face per 64 threads) as many faces as fill whole warps
   static constexpr int FPB = FULL ? T0 / PER : face_fpb(PER);
@@ -332,11 +334,11 @@ struct FaceCfg {
 };
 
 template <int DIM, int NP, class T>
-__global__ void __launch_bounds__(FaceCfg<DIM, NP>::T) k_faces_t(FaceArgs A, const __grid_constant__ OpsT<T> ops) {
+__global__ void __launch_bounds__(FaceCfg<DIM, NP, T>::T) k_faces_t(FaceArgs A, const __grid_constant__ OpsT<T> ops) {
   using S = Sz<DIM, NP>;
   constexpr int NV = S::NV, NF = S::NF, NFC = S::NFC, NSUB = S::NSUB;
-  constexpr int PER = FaceCfg<DIM, NP>::PER, BT = FaceCfg<DIM, NP>::T;
-  constexpr int FPB = FaceCfg<DIM, NP>::FPB;
+  constexpr int PER = FaceCfg<DIM, NP, T>::PER, BT = FaceCfg<DIM, NP, T>::T;
+  constexpr int FPB = FaceCfg<DIM, NP, T>::FPB;
   __shared__ T sF[FPB][NSUB][NV][NF];
   // 3D: the sum-factorised mortar stages' partial sums (interpolation HA, back-projection HB)
   constexpr int HA = 2 * NV * NP * NP, HB = NSUB * NV * NP * NP;
@@ -706,7 +708,7 @@ int launch_faces_impl(int dim, int p, FaceArgs A, const DevOps& o, cudaStream_t 
   OpsT<T> ops = make_ops_t<T>(o);
   set_gas(&ops, A.gamma);
   FR_NP_DISPATCH(dim, p, ({
-                   using FC = FaceCfg<DD, NN>;
+                   using FC = FaceCfg<DD, NN, T>;
                    const int NF = DD == 2 ? NN : NN * NN;
                    A.nb_conf = (A.n_conf * NF + FC::T - 1) / FC::T;
                    A.nb_hang = (A.n_hang + FC::FPB - 1) / FC::FPB;
