@@ -58,6 +58,15 @@ def flops_per_point_stage(dim, p):
     return prim + flux + deriv + rk + traces
 
 
+def fp64_ops_per_point_stage(dim):
+    """Operations of the FP64 form's element kernel on the FP64 pipe, per point and averaged over the three
+    stages: reciprocal, velocities, pressure and pointwise fluxes, and the Runge-Kutta combination (1, 3 and
+    3 operations a value).  Its contractions run in fixed point on the integer pipes."""
+    nv = dim + 2
+    flux = 3 + 2 * dim + 3 + dim * (dim + 1) // 2 + dim
+    return flux + 7.0 * nv / 3.0
+
+
 def bytes_per_point_stage(dim, p):
     """Algorithmic DRAM bytes of the element kernel per solution point: read u_s, read u^n, write
     the result, read the common fluxes and write the traces (2*dim*nv/n values each)."""
@@ -324,12 +333,11 @@ def aggregate_ranks(units, seconds, device="cuda"):
 
 
 def _kernel_source_hash():
-    """Hash of the element-stage kernel's source text (the k_stage_t definition)."""
+    """Hash of the FP64 form's element kernel's source text (the k_stage_fx definition)."""
     import hashlib
-    src = open(os.path.join(ROOT, "paper_2306_06744_gb300", "csrc", "fr_kernels.cuh")).read()
-    a = src.index("k_stage_t(StageArgs")
-    b = src.index("// ---- per-precision launch bodies")
-    return hashlib.sha256(src[a:b].encode()).hexdigest()[:16]
+    src = open(os.path.join(ROOT, "paper_2306_06744_gb300", "csrc", "fr_stage_fx.cuh")).read()
+    a = src.index("k_stage_fx(StageArgs")
+    return hashlib.sha256(src[a:].encode()).hexdigest()[:16]
 
 
 def _traffic_from_profiles(kernel):
@@ -447,11 +455,11 @@ def main():
     norms = mesh.norms()  # state, time and leaf count at the end of the timed cycles
     M_final = mesh.M
 
-    # element-kernel roofline (FP64: bound by the FP64 pipe)
+    # element-kernel roofline: the operations that the kernel leaves to the FP64 pipe (two flop each)
     st_s = prof["stage_ms"] / 1e3
     stage_avg_ms = prof["stage_ms"] / max(1, prof["stage_launches"])
     n_stage = 3 * ae * args.steps  # element (and interface) kernel launches in the timed region
-    flops = prof["stage_points"] * flops_per_point_stage(dim, p)
+    flops = prof["stage_points"] * 2.0 * fp64_ops_per_point_stage(dim)
     nbytes = prof["stage_points"] * bytes_per_point_stage(dim, p)
     achieved_tflops = flops / st_s / 1e12
     achieved_gbs = nbytes / st_s / 1e9
@@ -461,7 +469,7 @@ def main():
     except Exception:
         pass
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
-    kname = "k_stage<%d,%d>" % (dim, p + 1)
+    kname = "k_stage_fx<%d,%d>" % (dim, p + 1)
     tr = _traffic_from_profiles(kname)
     # DRAM bytes per launch from the ncu capture of this kernel instance, scaled to this run's
     # mean launch size
@@ -469,6 +477,7 @@ def main():
                if tr else None)
     roofline = {"kernel": kname + " (element stage)", "bound": "alu",
                 "flop_per_point": flops_per_point_stage(dim, p),
+                "fp64_ops_per_point": fp64_ops_per_point_stage(dim),
                 "bytes_per_point": bytes_per_point_stage(dim, p),
                 "points_per_launch": prof["stage_points"] / max(1, prof["stage_launches"]),
                 "achieved": achieved_tflops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
