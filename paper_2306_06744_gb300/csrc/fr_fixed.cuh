@@ -97,27 +97,42 @@ __host__ __device__ __forceinline__ double fx_double(long long v, int e, bool ba
 
 // ---- sums of products of values (flux terms), each operand with its own exponent E ----
 // x = v 2^(E - 1082) with 60-bit v (one bit more than the operands of the operator contractions, whose
-// sums are longer).  All partial products are kept: the sums below are in units of
-// 2^(Ev + Ew - 2102 - FX_PK), below 2^62 and wrong by less than 5 units (one for each operand cut at its
-// last bit, and the rounding), that is 2^-55 of the product of the operands' powers of two.
-constexpr int FX_PK = 2;
+// sums are longer), limbs v = vh 2^31 + vl with 0 <= vl < 2^31.  All partial products are kept: the sums
+// below are in units of 2^(Ev + Ew - 2102 - pk), below 2^62 and wrong by less than 7 units (one for each
+// operand cut at its last bit, and the rounding).
+constexpr int FX_PK = 2, FX_PK3 = 1;  // pk of the sum of squares and of fx_dot3
 constexpr int FX_P_MIN = 600;  // smallest exponent of an operand: units of products stay normal
-__host__ __device__ __forceinline__ int2 fx_plimbs(double x, int E) { return fx_limbs(x, E - 1); }
+__host__ __device__ __forceinline__ long long fx_value(double x, int E) {
+  const uint64_t b = fx_bits(x);
+  const int e = int(b >> 52) & 0x7FF;
+  const uint64_t m = ((b << 10) & 0x3FFFFFFFFFFFFFFFull) | 0x4000000000000000ull;
+  int s = E - e + 3;
+  s = s < 63 ? s : 63;
+  const long long a = (long long)(m >> s), sg = (long long)b >> 63;
+  return (a ^ sg) - sg;
+}
+__host__ __device__ __forceinline__ int2 fx_split(long long v) {
+  return make_int2(int(v >> 31), int(uint32_t(v) & 0x7FFFFFFFu));
+}
+// a - b limb by limb: the low limbs' difference keeps its sign
+__host__ __device__ __forceinline__ int2 fx_diff(int2 a, int2 b) { return make_int2(a.x - b.x, a.y - b.y); }
 __host__ __device__ __forceinline__ int fx_pexp(uint32_t mag) {
   const int e = int(mag >> 20);
   return e < FX_P_MIN ? FX_P_MIN : e;
 }
-__host__ __device__ __forceinline__ int fx_punit(int Ev, int Ew) { return Ev + Ew - 1079 - FX_PK; }
+__host__ __device__ __forceinline__ int fx_punit(int Ev, int Ew, int pk) { return Ev + Ew - 1079 - pk; }
 // no finite result for certain: an operand that is not finite, or a unit too large for the sum's range
 __host__ __device__ __forceinline__ bool fx_pbad(int Ev, int Ew) {
-  return Ev >= FX_E_BAD || Ew >= FX_E_BAD || fx_punit(Ev, Ew) > 2046 - 62;
+  return Ev >= FX_E_BAD || Ew >= FX_E_BAD || fx_punit(Ev, Ew, FX_PK3) > 2046 - 62;
 }
-// a b + c d: |h| <= 2 2^58, |m| <= 4 2^60 + 2 2^31
-__host__ __device__ __forceinline__ long long fx_dot2(int2 a, int2 b, int2 c, int2 d) {
-  const long long h = (long long)a.x * b.x + (long long)c.x * d.x;
-  long long m = (long long)a.x * b.y + (long long)a.y * b.x + (long long)c.x * d.y + (long long)c.y * d.x;
-  m += (((long long)a.y * b.y) >> 31) + (((long long)c.y * d.y) >> 31);
-  return (h << FX_PK) + ((m + (1ll << (30 - FX_PK))) >> (31 - FX_PK));
+// a b + c d + e f, e a difference of two values (61 bits): |h| <= 2 2^58 + 2^59, |m| <= 4 2^60 + 2^61 +
+// 2^60 + 3 2^31 < 2^63
+__host__ __device__ __forceinline__ long long fx_dot3(int2 a, int2 b, int2 c, int2 d, int2 e, int2 f) {
+  const long long h = (long long)a.x * b.x + (long long)c.x * d.x + (long long)e.x * f.x;
+  long long m = (long long)a.x * b.y + (long long)a.y * b.x + (long long)c.x * d.y + (long long)c.y * d.x +
+                (long long)e.x * f.y + (long long)e.y * f.x;
+  m += (((long long)a.y * b.y) >> 31) + (((long long)c.y * d.y) >> 31) + (((long long)e.y * f.y) >> 31);
+  return (h << FX_PK3) + ((m + (1ll << (30 - FX_PK3))) >> (31 - FX_PK3));
 }
 // sum of n <= 3 squares: h <= 3 2^58, |m| <= 3 2^60 (half of the cross products)
 template <int n>

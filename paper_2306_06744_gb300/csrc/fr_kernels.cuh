@@ -193,8 +193,9 @@ __device__ __forceinline__ void rusanov2_ff(const ff* qL, const ff* qR, int axis
 
 // The same in FP64 with its products on the integer pipes (fr_fixed.cuh), which idle in this kernel
 // while the FP64 pipe (2 operations a clock and SM) bounds it: |m|^2 and, for every variable, the sum
-// F2 = qL (vL + lambda) + qR (vR - lambda) + pressure terms, whose products are kept to 2^-55 of
-// |q| lambda.  34 FP64 operations a point in 3D instead of 54.
+// F2 = qL vL + qR vR + lambda (qL - qR) + pressure terms, whose products are exact to 2^-55 of
+// |q| lambda and whose difference is exact.  32 FP64 operations a point in 3D instead of 54 in FP64: per
+// launch, 127k leaves of the 3D p = 3 tubes, 691 -> 447 us.
 template <int DIM>
 __device__ __forceinline__ void rusanov2_fx(const double* qL, const double* qR, int axis, double sgam, double gm1,
                                             double* F2) {
@@ -212,12 +213,12 @@ __device__ __forceinline__ void rusanov2_fx(const double* qL, const double* qR, 
   int2 lL[NV], lR[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    lL[v] = fx_plimbs(qL[v], E[fx_group(v, NV)]);
-    lR[v] = fx_plimbs(qR[v], E[fx_group(v, NV)]);
+    lL[v] = fx_split(fx_value(qL[v], E[fx_group(v, NV)]));
+    lR[v] = fx_split(fx_value(qR[v], E[fx_group(v, NV)]));
   }
   const bool badm = fx_pbad(E[1], E[1]);
-  const double m2L = fx_double(fx_sum_sq<DIM>(lL + 1), fx_punit(E[1], E[1]), badm);
-  const double m2R = fx_double(fx_sum_sq<DIM>(lR + 1), fx_punit(E[1], E[1]), badm);
+  const double m2L = fx_double(fx_sum_sq<DIM>(lL + 1), fx_punit(E[1], E[1], FX_PK), badm);
+  const double m2R = fx_double(fx_sum_sq<DIM>(lR + 1), fx_punit(E[1], E[1], FX_PK), badm);
   const double pL = gm1 * fma(m2L, neg_half(rL), qL[NV - 1]);
   const double pR = gm1 * fma(m2R, neg_half(rR), qR[NV - 1]);
   double mnL = qL[1], mnR = qR[1];
@@ -229,13 +230,12 @@ __device__ __forceinline__ void rusanov2_fx(const double* qL, const double* qR, 
     }
   const double vL = mnL * rL, vR = mnR * rR;
   const double lam = fmax_pos(fma(sgam, sqrt_t(pL * rL), fabs(vL)), fma(sgam, sqrt_t(pR * rR), fabs(vR)));
-  const double aL = vL + lam, aR = vR - lam;
-  const int Ea = fx_pexp(max(fx_mag(aL), fx_mag(aR)));
-  const int2 caL = fx_plimbs(aL, Ea), caR = fx_plimbs(aR, Ea);
+  const int Ea = fx_pexp(fx_mag(lam));  // |v| <= lambda
+  const int2 cL = fx_split(fx_value(vL, Ea)), cR = fx_split(fx_value(vR, Ea)), cl = fx_split(fx_value(lam, Ea));
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     const int Ev = E[fx_group(v, NV)];
-    F2[v] = fx_double(fx_dot2(lL[v], caL, lR[v], caR), fx_punit(Ev, Ea), fx_pbad(Ev, Ea));
+    F2[v] = fx_double(fx_dot3(lL[v], cL, lR[v], cR, fx_diff(lL[v], lR[v]), cl), fx_punit(Ev, Ea, FX_PK3), fx_pbad(Ev, Ea));
   }
   const double pp = pL + pR;
   double fn = F2[1];
@@ -333,8 +333,11 @@ struct FaceCfg {
   static constexpr int T = FULL ? T0 : (FPB * PER + 31) / 32 * 32;
 };
 
+// FP64 in 3D is compiled for 1024 threads an SM (64 registers): 149 -> 113 us per launch at p = 4 (15k
+// leaves, blocks of 512 threads), 69 -> 66 at p = 1; in 2D the compiler's own 72 registers are better.
 template <int DIM, int NP, class T>
-__global__ void __launch_bounds__(FaceCfg<DIM, NP, T>::T) k_faces_t(FaceArgs A, const __grid_constant__ OpsT<T> ops) {
+__global__ void __launch_bounds__(FaceCfg<DIM, NP, T>::T,
+                                  DIM == 3 && std::is_same<T, double>::value ? 1024 / FaceCfg<DIM, NP, T>::T : 0) k_faces_t(FaceArgs A, const __grid_constant__ OpsT<T> ops) {
   using S = Sz<DIM, NP>;
   constexpr int NV = S::NV, NF = S::NF, NFC = S::NFC, NSUB = S::NSUB;
   constexpr int PER = FaceCfg<DIM, NP, T>::PER, BT = FaceCfg<DIM, NP, T>::T;

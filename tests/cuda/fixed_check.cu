@@ -56,25 +56,28 @@ int main(int argc, char** argv) {
     }
     printf("n%d %.6f\n", n, worst);
   }
-  // sums of products and squares: 5 units (operands cut at their last bit, rounding), each
-  // 2^-58 2^(Ev - 1022) 2^(Ew - 1022) at FX_PK = 2, then one rounding to double
+  // sums of products (two, and the exact difference of the first factors with a third) and of squares:
+  // operands cut at their last bit and the rounding, each a unit of 2^-58 (2^-57) 2^(Ev - 1022)
+  // 2^(Ew - 1022) at most, two units for a square and for the difference; then one rounding to double
   double dot = 0.0, sq = 0.0;
   for (int t = 0; t < 200000; ++t) {
     const int ta = int(rnd() % 800) - 400, tb = int(rnd() % 800) - 400, spread = int(rnd() % 70);
-    double x[4], y[2];
+    double x[4], y[3];
     for (int k = 0; k < 4; ++k) x[k] = rnd() % 16 == 0 ? 0.0 : draw(ta - spread, ta);
-    for (int k = 0; k < 2; ++k) y[k] = draw(tb - spread, tb);
-    const int Ex = fx_pexp(std::max(fx_mag(x[0]), fx_mag(x[1]))), Ey = fx_pexp(std::max(fx_mag(y[0]), fx_mag(y[1])));
-    const double got = fx_double(fx_dot2(fx_plimbs(x[0], Ex), fx_plimbs(y[0], Ey), fx_plimbs(x[1], Ex), fx_plimbs(y[1], Ey)),
-                                 fx_punit(Ex, Ey), fx_pbad(Ex, Ey));
-    const long double want = (long double)x[0] * y[0] + (long double)x[1] * y[1];
-    const long double b = 5.0L * ldexpl(1.0L, Ex + Ey - 2102 - FX_PK) + 0x1p-53L * fabsl(want);
-    dot = std::max(dot, double(fabsl(got - want) / b));
+    for (int k = 0; k < 3; ++k) y[k] = draw(tb - spread, tb);
+    const int Ex = fx_pexp(std::max(fx_mag(x[0]), fx_mag(x[1])));
+    const int Ey = fx_pexp(std::max(fx_mag(y[0]), std::max(fx_mag(y[1]), fx_mag(y[2]))));
+    const long long a = fx_value(x[0], Ex), b = fx_value(x[1], Ex);
+    const double got = fx_double(fx_dot3(fx_split(a), fx_split(fx_value(y[0], Ey)), fx_split(b), fx_split(fx_value(y[1], Ey)),
+                                         fx_diff(fx_split(a), fx_split(b)), fx_split(fx_value(y[2], Ey))),
+                                 fx_punit(Ex, Ey, FX_PK3), fx_pbad(Ex, Ey));
+    const long double want = (long double)x[0] * y[0] + (long double)x[1] * y[1] + ((long double)x[0] - x[1]) * y[2];
+    const long double bd = 9.0L * ldexpl(1.0L, Ex + Ey - 2102 - FX_PK3) + 0x1p-53L * fabsl(want);
+    dot = std::max(dot, double(fabsl(got - want) / bd));
     const int Es = fx_pexp(std::max(fx_mag(x[1]), std::max(fx_mag(x[2]), fx_mag(x[3]))));
-    const int2 l[3] = {fx_plimbs(x[1], Es), fx_plimbs(x[2], Es), fx_plimbs(x[3], Es)};
-    const double gs = fx_double(fx_sum_sq<3>(l), fx_punit(Es, Es), fx_pbad(Es, Es));
+    const int2 l[3] = {fx_split(fx_value(x[1], Es)), fx_split(fx_value(x[2], Es)), fx_split(fx_value(x[3], Es))};
+    const double gs = fx_double(fx_sum_sq<3>(l), fx_punit(Es, Es, FX_PK), fx_pbad(Es, Es));
     const long double ws = (long double)x[1] * x[1] + (long double)x[2] * x[2] + (long double)x[3] * x[3];
-    // every square of a cut operand is wrong by at most two units
     const long double bs = 7.0L * ldexpl(1.0L, 2 * Es - 2102 - FX_PK) + 0x1p-53L * ws;
     sq = std::max(sq, double(fabsl(gs - ws) / bs));
   }
