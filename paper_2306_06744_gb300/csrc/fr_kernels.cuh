@@ -475,12 +475,13 @@ __global__ void __launch_bounds__(FaceCfg<DIM, NP, T>::T,
   }
 }
 
-// Resident blocks the element kernel is compiled for: the FP32 form is bound by memory latency
-// and wants every block shared memory allows (the register budget is set to fit them); the others
-// keep the compiler's choice.
+// Resident blocks the element kernel is compiled for: the FP32 form wants every block shared memory allows
+// (the register budget is set to fit them); the double-word form leaves the choice to the compiler (0).  A
+// minimum of one block is no such choice: it spends registers on it (2D p = 3 62 instead of 40, 3D p = 2
+// 72 instead of 56), 525 against 466 us per launch at 3D p = 2 with 184k leaves, 803 against 779 at p = 3.
 template <class T>
 struct StageMinBlocks {
-  static constexpr int value = std::is_same<T, float>::value ? 12 : 1;
+  static constexpr int value = std::is_same<T, float>::value ? 12 : 0;
 };
 
 // element stage: R = -sum_a (2/h) [ sum_j Dt_ij f_j + gL_i F(-1) + gR_i F(+1) ] along each axis
