@@ -80,7 +80,9 @@ typedef struct {
                               element's flux-derivative contraction on the tensor cores in TF32
                               (FP32 accumulation); 3 the same in split BF16 (bf16x3: hi*hi +
                               hi*lo + lo*hi, FP32 accumulation); 4 double-word (two-float, ~48-bit
-                              significand) on the FP32 pipes.  2 and 3 are built for dim 3, p 3
+                              significand) on the FP32 pipes, the Runge-Kutta combination in FP64.
+                              0 forms its linear operators and flux products in fixed point of at
+                              least 58 bits on the integer pipes.  2 and 3 are built for dim 3, p 3
                               (64-point hexahedra, Sec. 2.1's operator as 16 x 16 Kronecker blocks);
                               other dim/p return FR_EINVAL.  A tensor-core completion wait that
                               gives up is reported as FR_ETIMEOUT by the next fr_adapt/fr_run

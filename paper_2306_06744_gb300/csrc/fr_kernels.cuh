@@ -1,7 +1,8 @@
 // fr_kernels.cuh -- the time-step kernels of flux reconstruction (arXiv 2306.06744, Sec. 2.1 and
 // 4.3), templated on the dimension, the number of points per direction n = p+1 and the
-// arithmetic type T (double, float or double-word ff; see fr_arith.cuh).  The state u is FP64 in
-// memory for every T; face traces and common fluxes are stored in T.  Each precision is
+// arithmetic type T (double, float or double-word ff; see fr_arith.cuh): the interface kernel for all
+// three, the element and trace kernels for float and ff (FP64's are in fr_stage_fx.cuh).  The state u is
+// FP64 in memory for every T; face traces and common fluxes are stored in T.  Each precision is
 // instantiated in its own translation unit (fr_prec_*.cu).
 #pragma once
 
