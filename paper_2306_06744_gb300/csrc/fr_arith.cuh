@@ -18,6 +18,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fr_fixed.cuh"
+
 namespace frg {
 
 struct __align__(8) ff {  // one 8-byte access
@@ -173,11 +175,15 @@ __device__ __forceinline__ double fma_t(double a, double b, double c) { return f
 // reciprocals: FP64 from the hardware approximation r (relative error e ~2^-23) by one third-order
 // step, r (1 + e + e^2), which leaves e^3 (three FP64 operations; two Newton steps take four); FP32 by
 // the fast divide; double-word by the corrected quotient above.
-__device__ __forceinline__ double rcp_t(double x) {
+__host__ __device__ __forceinline__ double rcp_t(double x) {
+#ifdef __CUDA_ARCH__
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   const double e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
+#else
+  return 1.0 / x;
+#endif
 }
 __device__ __forceinline__ float rcp_t(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ ff rcp_t(ff x) { return ff{1.f, 0.f} / x; }
@@ -187,7 +193,8 @@ __device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(
 // (Markstein 1990), which leaves half an ulp and 2^-66: five FP64 operations, the halving is done on
 // the exponent.  Zero, values below 2^-959 (whose residual could fall below the normal range),
 // infinities, NaN and negative values take the library's.
-__device__ __forceinline__ double sqrt_t(double a) {
+__host__ __device__ __forceinline__ double sqrt_t(double a) {
+#ifdef __CUDA_ARCH__
   const uint32_t ex = uint32_t(__double2hiint(a)) >> 20;  // sign and exponent
   if (ex - 64u > 1982u) return sqrt(a);
   double y;
@@ -196,19 +203,25 @@ __device__ __forceinline__ double sqrt_t(double a) {
   double g = a * y;
   g = fma(g, fma(-g, h, 0.5), g);
   return fma(fma(-g, g, a), h, g);
+#else
+  return sqrt(a);
+#endif
 }
 __device__ __forceinline__ float sqrt_t(float a) { return sqrtf(a); }
 __device__ __forceinline__ float fabs_t(float a) { return fabsf(a); }
-// the larger of two non-negative values: positive doubles order as their bit patterns, so the FP64
-// pipe is left out (a NaN wins)
-__device__ __forceinline__ double fmax_pos(double a, double b) {
-  return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+// fmax of two values that are non-negative or NaN, on their bit patterns (the FP64 pipe is left out):
+// without the sign they order as the values do, and less the pattern above infinity, modulo 2^64, every
+// NaN, whatever its sign, comes below every number.  So a wave speed that is not a number (one side's
+// pressure is negative) loses to the other side's, as in the FP32 form.
+__host__ __device__ __forceinline__ double fmax_num(double a, double b) {
+  constexpr uint64_t MAG = 0x7FFFFFFFFFFFFFFFull, NAN0 = 0x7FF0000000000001ull;
+  return (fx_bits(a) & MAG) - NAN0 > (fx_bits(b) & MAG) - NAN0 ? a : b;
 }
 __device__ __forceinline__ float fmax_t(float a, float b) { return fmaxf(a, b); }
 
 // -x/2 without a multiplication where the exponent can be lowered (x normal, above 2^-1021)
-__device__ __forceinline__ double neg_half(double x) {
-  return __hiloint2double((__double2hiint(x) - (1 << 20)) ^ int(0x80000000u), __double2loint(x));
+__host__ __device__ __forceinline__ double neg_half(double x) {
+  return fx_from_bits((fx_bits(x) - (1ull << 52)) ^ (1ull << 63));
 }
 __device__ __forceinline__ ff neg_half(ff x) { return {-0.5f * x.h, -0.5f * x.l}; }
 

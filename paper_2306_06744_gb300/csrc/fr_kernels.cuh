@@ -195,10 +195,10 @@ __device__ __forceinline__ void rusanov2_ff(const ff* qL, const ff* qR, int axis
 // The same in FP64 with its products on the integer pipes (fr_fixed.cuh), which idle in this kernel
 // while the FP64 pipe (2 operations a clock and SM) bounds it: |m|^2 and, for every variable, the sum
 // F2 = qL vL + qR vR + lambda (qL - qR) + pressure terms, whose products are exact to 2^-55 of
-// |q| lambda and whose difference is exact.  32 FP64 operations a point in 3D instead of 54 in FP64: per
+// |q| max(lambda, |v|) and whose difference is exact.  32 FP64 operations a point in 3D instead of 54 in FP64: per
 // launch, 127k leaves of the 3D p = 3 tubes, 691 -> 447 us.
 template <int DIM>
-__device__ __forceinline__ void rusanov2_fx(const double* qL, const double* qR, int axis, double sgam, double gm1,
+__host__ __device__ __forceinline__ void rusanov2_fx(const double* qL, const double* qR, int axis, double sgam, double gm1,
                                             double* F2) {
   constexpr int NV = DIM + 2;
   const double rLR = rcp_t(qL[0] * qR[0]);
@@ -230,8 +230,9 @@ __device__ __forceinline__ void rusanov2_fx(const double* qL, const double* qR, 
       mnR = qR[1 + b];
     }
   const double vL = mnL * rL, vR = mnR * rR;
-  const double lam = fmax_pos(fma(sgam, sqrt_t(pL * rL), fabs(vL)), fma(sgam, sqrt_t(pR * rR), fabs(vR)));
-  const int Ea = fx_pexp(fx_mag(lam));  // |v| <= lambda
+  const double lam = fmax_num(fma(sgam, sqrt_t(pL * rL), fabs(vL)), fma(sgam, sqrt_t(pR * rR), fabs(vR)));
+  // |v| <= lambda except where a side's own wave speed is not a number; a NaN velocity makes all sums NaN
+  const int Ea = fx_pexp(max(fx_mag(lam), max(fx_mag(vL), fx_mag(vR))));
   const int2 cL = fx_split(fx_value(vL, Ea)), cR = fx_split(fx_value(vR, Ea)), cl = fx_split(fx_value(lam, Ea));
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
