@@ -221,10 +221,6 @@ __host__ __device__ __forceinline__ double fmax_num(double a, double b) {
 }
 __device__ __forceinline__ float fmax_t(float a, float b) { return fmaxf(a, b); }
 
-// -x/2 without a multiplication where the exponent can be lowered (x normal, above 2^-1021)
-__host__ __device__ __forceinline__ double neg_half(double x) {
-  return fx_from_bits((fx_bits(x) - (1ull << 52)) ^ (1ull << 63));
-}
 __device__ __forceinline__ ff neg_half(ff x) { return {-0.5f * x.h, -0.5f * x.l}; }
 
 // zero / constant helpers

@@ -198,30 +198,52 @@ __device__ __forceinline__ void rusanov2_ff(const ff* qL, const ff* qR, int axis
 // |q| max(lambda, |v|) and whose difference is exact.  32 FP64 operations a point in 3D instead of 54 in FP64: per
 // launch, 127k leaves of the 3D p = 3 tubes, 691 -> 447 us.
 template <int DIM>
-__host__ __device__ __forceinline__ void rusanov2_fx(const double* qL, const double* qR, int axis, double sgam, double gm1,
-                                            double* F2) {
+__host__ __device__ __forceinline__ void rusanov2_fx(const double* qL, const double* qR, int axis, double sgam,
+                                                     double gm1, double* F2) {
   constexpr int NV = DIM + 2;
   const double rLR = rcp_t(qL[0] * qR[0]);
   const double rL = qR[0] * rLR, rR = qL[0] * rLR;
-  int E[FX_GROUPS];
+  // exponents of density, momenta and energy of both sides, and of either side's momenta: the thin side of a
+  // density jump would lose its |m|^2 beside the other side's (its pressure and wave speed with it, by 2^-58
+  // times the square of the jump)
+  int EL, ER;
   {
-    uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
+    uint32_t wL = 0u, wR = 0u;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) w[fx_group(v, NV)] = max(w[fx_group(v, NV)], max(fx_mag(qL[v]), fx_mag(qR[v])));
-#pragma unroll
-    for (int g = 0; g < FX_GROUPS; ++g) E[g] = fx_pexp(w[g]);
+    for (int b = 0; b < DIM; ++b) {
+      wL = max(wL, fx_mag(qL[1 + b]));
+      wR = max(wR, fx_mag(qR[1 + b]));
+    }
+    EL = fx_pexp(wL);
+    ER = fx_pexp(wR);
   }
+  const int E[FX_GROUPS] = {fx_pexp(max(fx_mag(qL[0]), fx_mag(qR[0]))), max(EL, ER),
+                            fx_pexp(max(fx_mag(qL[NV - 1]), fx_mag(qR[NV - 1])))};
   int2 lL[NV], lR[NV];
+  double kL, kR;  // |m|^2 / 2, halved in its unit
+  {
+    long long a[DIM], c[DIM];
+    int2 s[DIM];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
+    for (int b = 0; b < DIM; ++b) s[b] = fx_split(a[b] = fx_value(qL[1 + b], EL));
+    kL = fx_double(fx_sum_sq<DIM>(s), fx_punit(EL, EL, FX_PK) - 1, fx_pbad(EL, EL));
+#pragma unroll
+    for (int b = 0; b < DIM; ++b) s[b] = fx_split(c[b] = fx_value(qR[1 + b], ER));
+    kR = fx_double(fx_sum_sq<DIM>(s), fx_punit(ER, ER, FX_PK) - 1, fx_pbad(ER, ER));
+    const int sL = min(E[1] - EL, 63), sR = min(E[1] - ER, 63);
+#pragma unroll
+    for (int b = 0; b < DIM; ++b) {
+      lL[1 + b] = fx_split(a[b] >> sL);
+      lR[1 + b] = fx_split(c[b] >> sR);
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < NV; v += NV - 1) {
     lL[v] = fx_split(fx_value(qL[v], E[fx_group(v, NV)]));
     lR[v] = fx_split(fx_value(qR[v], E[fx_group(v, NV)]));
   }
-  const bool badm = fx_pbad(E[1], E[1]);
-  const double m2L = fx_double(fx_sum_sq<DIM>(lL + 1), fx_punit(E[1], E[1], FX_PK), badm);
-  const double m2R = fx_double(fx_sum_sq<DIM>(lR + 1), fx_punit(E[1], E[1], FX_PK), badm);
-  const double pL = gm1 * fma(m2L, neg_half(rL), qL[NV - 1]);
-  const double pR = gm1 * fma(m2R, neg_half(rR), qR[NV - 1]);
+  const double pL = gm1 * fma(-kL, rL, qL[NV - 1]);
+  const double pR = gm1 * fma(-kR, rR, qR[NV - 1]);
   double mnL = qL[1], mnR = qR[1];
 #pragma unroll
   for (int b = 1; b < DIM; ++b)

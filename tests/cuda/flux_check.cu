@@ -118,6 +118,15 @@ static void kinds() {
     worst = fmax(worst, ratio<DIM>(qL, qR, t % DIM));
   }
   line("plain");
+  // one side 10 to 1e8 times as dense as the other at the same speeds and temperatures
+  worst = 0;
+  for (int t = 0; t < 20000; ++t) {
+    const double f = std::pow(10.0, 1.0 + 7.0 * rnd());
+    state<DIM>(t & 1 ? f : 1.0, 0.1 + rnd(), qL);
+    state<DIM>(t & 1 ? 1.0 : f, 0.1 + rnd(), qR);
+    worst = fmax(worst, ratio<DIM>(qL, qR, t % DIM));
+  }
+  line("jump");
   // one side's pressure negative: its wave speed is not a number, the other side's counts; its own
   // speed is up to 100 times that
   worst = 0;

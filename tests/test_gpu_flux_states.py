@@ -97,6 +97,17 @@ def test_negative_pressure_on_one_side(dim, p):
     assert (np.abs(got - want) <= TOL * scale[:, :, None]).all()
 
 
+@pytest.mark.parametrize("jump", [1e2, 1e4, 1e6, 1e8])
+@pytest.mark.parametrize("dim,p", [(2, 1), (2, 3), (3, 2)])
+def test_density_jump_across_faces(dim, p, jump):
+    # one element in eight lighter by the factor, speeds and temperatures alike
+    g, keys, cells = _mesh(dim, p, 2)
+    q = _states(len(keys), dim, 6)
+    q[(cells % 2 == 0).all(1)] /= jump
+    want, scale = _rhs(q, cells, p, 2)
+    assert (np.abs(_run(g, keys, q) - want) <= TOL * scale[:, :, None]).all()
+
+
 @pytest.mark.parametrize("value", [np.nan, -np.nan, np.inf, -np.inf])
 @pytest.mark.parametrize("dim,p", [(2, 2), (3, 1)])
 def test_special_values_reach_the_neighbours(dim, p, value):
