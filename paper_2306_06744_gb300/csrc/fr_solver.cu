@@ -521,10 +521,12 @@ __global__ void __launch_bounds__(NRM_T) k_norms(const uint64_t* __restrict__ ke
       double m2 = q[1] * q[1];
 #pragma unroll
       for (int b = 1; b < DIM; ++b) m2 = fma(q[1 + b], q[1 + b], m2);
-      // |m|^2 / rho from the reciprocal and one residual correction
+      // |m|^2 / rho from the reciprocal and one residual correction; where that gives no number, or rho is
+      // zero or near the ends of the range, the division (an infinite quotient has to reach the minimum)
       const double r = rcp_t(q[0]);
       double k2 = m2 * r;
       k2 = fma(fma(-k2, q[0], m2), r, k2);
+      if ((fx_mag(q[0]) >> 20) - 64u > 1918u || fx_mag(k2) >= 0x7FF00000u) k2 = m2 / q[0];
       acc[NV + 1] = fmin(acc[NV + 1], q[0]);
       acc[NV + 2] = fmin(acc[NV + 2], V.gm1 * fma(-0.5, k2, q[NV - 1]));
     }
