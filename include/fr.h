@@ -189,9 +189,10 @@ const char* fr_last_error(const fr_mesh* m);
    pressure give 100*(rho_i - mean rho)/mean rho and 100*(p_i - mean p)/mean p, then
    (D - Dbase)/max(1, Dmax - Dbase).
    Labels are classes -1/0/+1 (coarsen/keep/refine), int8.  class_w = {w_coarsen, w_keep, w_refine,
-   1/sum_batch w_label}: the loss is sum_b w_b CE_b * class_w[3] (weighted mean cross-entropy); with
-   class_w[3] = 0 the library forms that factor from the batch's labels (FR_EINVAL if it is infinite).
-   Labels outside -1..1 give FR_EINVAL and leave the parameters as they are.
+   1/sum_batch w_label}: the loss is sum_b w_b CE_b * class_w[3] (weighted mean cross-entropy).
+   fr_mlp_grad and fr_mlp_train_step take class_w[3] as it is; in the _alloc forms class_w[3] = 0 lets the
+   library form that factor from the batch's labels (FR_EINVAL if it is infinite).  Labels outside -1..1
+   give FR_EINVAL.  With either error nothing is written to the parameters, moments, gradient or loss.
    fr_mlp_train_step performs one Adam step (beta 0.9/0.999, eps 1e-8; d_m, d_v the moment arrays,
    step counts from 0) in place on d_params; d_loss (device, may be NULL) receives the batch loss.
    fr_mlp_grad returns the gradient of that loss instead.  Device pointers throughout; 1 <= IN <= 64
@@ -219,10 +220,13 @@ int fr_mlp_grad(int in_dim, const float* d_params, const void* d_X_bf16, const i
 int fr_mlp_train_step(int in_dim, float* d_params, float* d_m, float* d_v, int64_t step,
                       const void* d_X_bf16, const int8_t* d_y, int64_t B, const float* class_w,
                       float lr, float* d_loss, void* stream);
-/* The same with the call's scratch memory from the caller's allocator (NULL: the stream-ordered pool,
+/* The same (but for class_w[3] = 0, see above) with the call's scratch memory from the caller's allocator (NULL: the stream-ordered pool,
    which gives its memory back at every synchronisation, so that the next call pays for it again). */
 int fr_mlp_forward_alloc(int in_dim, const float* d_params, const void* d_X_bf16, int64_t n,
                          float* d_logits, int8_t* d_flags, void* stream, const fr_allocator* alloc);
+int fr_mlp_grad_alloc(int in_dim, const float* d_params, const void* d_X_bf16, const int8_t* d_y,
+                      int64_t B, const float* class_w, float* d_grad, float* d_loss, void* stream,
+                      const fr_allocator* alloc);
 int fr_mlp_train_step_alloc(int in_dim, float* d_params, float* d_m, float* d_v, int64_t step,
                             const void* d_X_bf16, const int8_t* d_y, int64_t B, const float* class_w,
                             float lr, float* d_loss, void* stream, const fr_allocator* alloc);

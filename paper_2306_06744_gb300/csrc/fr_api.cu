@@ -1100,31 +1100,45 @@ int fr_mlp_forward(int in_dim, const float* d_params, const void* d_X, int64_t n
 
 void fr_tc_set_wait_limit(long long cycles) { mlp_set_wait_cycles(cycles); }
 
-int fr_mlp_grad(int in_dim, const float* d_params, const void* d_X, const int8_t* d_y, int64_t B,
-                const float* class_w, float* d_grad, float* d_loss, void* stream) {
+static int mlp_grad_call(int in_dim, const float* d_params, const void* d_X, const int8_t* d_y, int64_t B,
+                         const float* class_w, bool norm, float* d_grad, float* d_loss, void* stream,
+                         const fr_allocator* alloc) {
   if (in_dim < 1 || in_dim > 64 || B <= 0 || !class_w)
     return set_error(global_err(), FR_EINVAL, "bad arguments");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  Alloc A{nullptr, s, global_err()};
-  FR_TRY(mlp_grad(d_params, in_dim, d_X, d_y, B, class_w, d_grad, d_loss, A, s, global_err()));
-  FR_CUDA(global_err(), cudaStreamSynchronize(s));
-  return 0;
+  CallAlloc CA(alloc, s, global_err());
+  return mlp_grad(d_params, in_dim, d_X, d_y, B, class_w, norm, d_grad, d_loss, CA.A, s, global_err());
+}
+int fr_mlp_grad(int in_dim, const float* d_params, const void* d_X, const int8_t* d_y, int64_t B,
+                const float* class_w, float* d_grad, float* d_loss, void* stream) {
+  return mlp_grad_call(in_dim, d_params, d_X, d_y, B, class_w, false, d_grad, d_loss, stream, nullptr);
+}
+int fr_mlp_grad_alloc(int in_dim, const float* d_params, const void* d_X, const int8_t* d_y, int64_t B,
+                      const float* class_w, float* d_grad, float* d_loss, void* stream, const fr_allocator* alloc) {
+  return mlp_grad_call(in_dim, d_params, d_X, d_y, B, class_w, class_w && class_w[3] == 0.f, d_grad, d_loss, stream,
+                       alloc);
 }
 
-int fr_mlp_train_step_alloc(int in_dim, float* d_params, float* d_m, float* d_v, int64_t step, const void* d_X,
-                            const int8_t* d_y, int64_t B, const float* class_w, float lr, float* d_loss,
-                            void* stream, const fr_allocator* alloc) {
+static int mlp_train_call(int in_dim, float* d_params, float* d_m, float* d_v, int64_t step, const void* d_X,
+                          const int8_t* d_y, int64_t B, const float* class_w, bool norm, float lr, float* d_loss,
+                          void* stream, const fr_allocator* alloc) {
   if (in_dim < 1 || in_dim > 64 || B <= 0 || !class_w || step < 0)
     return set_error(global_err(), FR_EINVAL, "bad arguments");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CallAlloc CA(alloc, s, global_err());
-  return mlp_train_step(d_params, d_m, d_v, step, in_dim, d_X, d_y, B, class_w, lr, d_loss, CA.A, s, global_err());
+  return mlp_train_step(d_params, d_m, d_v, step, in_dim, d_X, d_y, B, class_w, norm, lr, d_loss, CA.A, s,
+                        global_err());
 }
-
 int fr_mlp_train_step(int in_dim, float* d_params, float* d_m, float* d_v, int64_t step,
                       const void* d_X, const int8_t* d_y, int64_t B, const float* class_w, float lr,
                       float* d_loss, void* stream) {
-  return fr_mlp_train_step_alloc(in_dim, d_params, d_m, d_v, step, d_X, d_y, B, class_w, lr, d_loss, stream, nullptr);
+  return mlp_train_call(in_dim, d_params, d_m, d_v, step, d_X, d_y, B, class_w, false, lr, d_loss, stream, nullptr);
+}
+int fr_mlp_train_step_alloc(int in_dim, float* d_params, float* d_m, float* d_v, int64_t step, const void* d_X,
+                            const int8_t* d_y, int64_t B, const float* class_w, float lr, float* d_loss,
+                            void* stream, const fr_allocator* alloc) {
+  return mlp_train_call(in_dim, d_params, d_m, d_v, step, d_X, d_y, B, class_w, class_w && class_w[3] == 0.f, lr,
+                        d_loss, stream, alloc);
 }
 
 // ---- tree primitives on caller-owned device arrays ----

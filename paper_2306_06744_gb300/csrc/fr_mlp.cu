@@ -402,13 +402,10 @@ __global__ void __launch_bounds__(256) k_label_count(const int8_t* __restrict__ 
     if (n && (threadIdx.x & 31) == 0) atomicAdd(&cnt[k], (unsigned long long)n);
   }
 }
-// total class weight of the batch, and its inverse (or the caller's)
-__device__ __forceinline__ double class_weight(const unsigned long long* cnt, float cw0, float cw1, float cw2) {
-  return double(cnt[0]) * cw0 + double(cnt[1]) * cw1 + double(cnt[2]) * cw2;
-}
-__device__ __forceinline__ float inverse_weight(const unsigned long long* cnt, float cw0, float cw1, float cw2,
-                                                float inv_given) {
-  return inv_given != 0.f ? inv_given : float(1.0 / class_weight(cnt, cw0, cw1, cw2));
+// factor of the weighted mean: the inverse of the batch's total class weight (norm), or the caller's
+__device__ __forceinline__ float loss_factor(const unsigned long long* cnt, float cw0, float cw1, float cw2,
+                                             float given, bool norm) {
+  return norm ? float(1.0 / (double(cnt[0]) * cw0 + double(cnt[1]) * cw1 + double(cnt[2]) * cw2)) : given;
 }
 
 // Tensor-core training: gradient of the weighted mean softmax cross-entropy over a batch.  Each
@@ -436,7 +433,7 @@ constexpr int TG_W1 = 0, TG_W2 = 8192, TG_W3 = 16384, TG_W4 = 24576, TG_W2T = 26
 __global__ void __launch_bounds__(TG_T) k_mlp_grad_tc(const float* __restrict__ P, int in,
                                                       const __nv_bfloat16* __restrict__ X,
                                                       const int8_t* __restrict__ y, int64_t B, float cw0,
-                                                      float cw1, float cw2, float inv_given,
+                                                      float cw1, float cw2, float given, bool norm,
                                                       const unsigned long long* __restrict__ cnt,
                                                       float* __restrict__ Gp, float* __restrict__ Lp,
                                                       int* __restrict__ status) {
@@ -449,7 +446,7 @@ __global__ void __launch_bounds__(TG_T) k_mlp_grad_tc(const float* __restrict__ 
   auto put = [&](int off, uint32_t o, float v) {
     *reinterpret_cast<__nv_bfloat16*>(sm + off + o) = __float2bfloat16_rn(v);
   };
-  const float inv_wsum = inverse_weight(cnt, cw0, cw1, cw2, inv_given);
+  const float inv_wsum = loss_factor(cnt, cw0, cw1, cw2, given, norm);
   // weights (BF16, zero padding) and their transposes for the backward products
   for (int idx = t; idx < H * 64; idx += TG_T) {
     const int o = idx >> 6, k = idx & 63;
@@ -690,8 +687,8 @@ __global__ void __launch_bounds__(TG_T) k_mlp_grad_tc(const float* __restrict__ 
 
 // Sums of the blocks' partial gradients and losses, in block order, stored (G) or applied by Adam
 // (Kingma & Ba): m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2, p -= lr mhat / (sqrt(vhat) + eps).  A wait
-// that gave up in the gradient kernel, a label outside -1..1 (status 2) or a total weight of zero (status
-// 4) leaves everything unchanged.
+// that gave up in the gradient kernel, a label outside -1..1 (status 2) or a batch whose factor is infinite
+// (status 4: its weights sum to zero, or nearly) leaves everything unchanged.
 struct AdamArgs {
   float *P, *m, *v;
   float lr, b1, b2, eps, c1, c2;
@@ -699,11 +696,12 @@ struct AdamArgs {
 constexpr int RED_T = 64;
 __global__ void __launch_bounds__(RED_T) k_grad_reduce(const float* __restrict__ Gp, const float* __restrict__ Lp,
                                                        int nblk, int total, float cw0, float cw1, float cw2,
-                                                       float inv_given, const unsigned long long* __restrict__ cnt,
+                                                       float given, bool norm,
+                                                       const unsigned long long* __restrict__ cnt,
                                                        float* __restrict__ G, float* __restrict__ loss, AdamArgs A,
                                                        int* __restrict__ status) {
   const int t = threadIdx.x, p = blockIdx.x * RED_T + t;
-  const int bad = cnt[3] ? 2 : (inv_given == 0.f && class_weight(cnt, cw0, cw1, cw2) == 0.0 ? 4 : 0);
+  const int bad = cnt[3] ? 2 : (norm && isinf(loss_factor(cnt, cw0, cw1, cw2, given, norm)) ? 4 : 0);
   if (bad) {
     if (blockIdx.x == 0 && t == 0) atomicOr(status, bad);
     return;
@@ -802,10 +800,10 @@ int mlp_features(int dim, int p, const double* u, const uint64_t* keys, int64_t 
 }
 
 // Gradient and loss of one batch on the tensor cores, stored into G or (G null) applied by Adam.  The
-// labels are counted first for the factor that normalises them; cw[3] != 0 gives 1 / sum_b w_{y_b}
-// instead.  Synchronises: the status word is read at the end.
+// labels are counted first, for their range and, with norm, for the factor 1 / sum_b w_{y_b}; otherwise the
+// factor is cw[3].  Synchronises: the status word is read at the end.
 static int grad_step(const float* d_params, int in, const void* d_X, const int8_t* d_y, int64_t B, const float* cw,
-                     float* G, float* d_loss, const AdamArgs& adam, Alloc& A, cudaStream_t s, Err* err) {
+                     bool norm, float* G, float* d_loss, const AdamArgs& adam, Alloc& A, cudaStream_t s, Err* err) {
   if (B <= 0) return set_error(err, FR_EINVAL, "empty batch");
   if (in < 1 || in > 64) return set_error(err, FR_EINVAL, "the MLP takes 1..64 inputs");
   const Lay L = lay(in);
@@ -827,31 +825,31 @@ static int grad_step(const float* d_params, int in, const void* d_X, const int8_
   FR_LAUNCH_CHECK(err);
   FR_CUDA(err, cudaFuncSetAttribute(k_mlp_grad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_SMEM));
   k_mlp_grad_tc<<<unsigned(grid), TG_T, TG_SMEM, s>>>(d_params, in, static_cast<const __nv_bfloat16*>(d_X), d_y, B,
-                                                      cw[0], cw[1], cw[2], cw[3], cnt, Gp, Lp, st);
+                                                      cw[0], cw[1], cw[2], cw[3], norm, cnt, Gp, Lp, st);
   FR_LAUNCH_CHECK(err);
   k_grad_reduce<<<unsigned((L.total + RED_T - 1) / RED_T), RED_T, 0, s>>>(Gp, Lp, grid, L.total, cw[0], cw[1], cw[2],
-                                                                          cw[3], cnt, G, d_loss, adam, st);
+                                                                          cw[3], norm, cnt, G, d_loss, adam, st);
   FR_LAUNCH_CHECK(err);
   int h = 0;
   FR_CUDA(err, cudaMemcpyAsync(&h, st, 4, cudaMemcpyDeviceToHost, s));
   FR_CUDA(err, cudaStreamSynchronize(s));
   if (h & 1) return set_error(err, FR_ETIMEOUT, "a tensor-core completion wait gave up (training)");
   if (h & 2) return set_error(err, FR_EINVAL, "labels must be -1, 0 or 1");
-  return h ? set_error(err, FR_EINVAL, "the batch's class weights sum to zero") : 0;
+  return h ? set_error(err, FR_EINVAL, "the inverse of the batch's total class weight is infinite") : 0;
 }
 
 int mlp_train_step(float* d_params, float* d_m, float* d_v, int64_t step, int in, const void* d_X,
-                   const int8_t* d_y, int64_t B, const float* cw, float lr, float* d_loss,
+                   const int8_t* d_y, int64_t B, const float* cw, bool norm, float lr, float* d_loss,
                    Alloc& A, cudaStream_t s, Err* err) {
   const float b1 = 0.9f, b2 = 0.999f;
   const AdamArgs adam{d_params, d_m, d_v, lr, b1, b2, 1e-8f, 1.f - std::pow(b1, float(step + 1)),
                       1.f - std::pow(b2, float(step + 1))};
-  return grad_step(d_params, in, d_X, d_y, B, cw, nullptr, d_loss, adam, A, s, err);
+  return grad_step(d_params, in, d_X, d_y, B, cw, norm, nullptr, d_loss, adam, A, s, err);
 }
 
 int mlp_grad(const float* d_params, int in, const void* d_X, const int8_t* d_y, int64_t B,
-             const float* cw, float* d_grad, float* d_loss, Alloc& A, cudaStream_t s, Err* err) {
-  return grad_step(d_params, in, d_X, d_y, B, cw, d_grad, d_loss, AdamArgs{}, A, s, err);
+             const float* cw, bool norm, float* d_grad, float* d_loss, Alloc& A, cudaStream_t s, Err* err) {
+  return grad_step(d_params, in, d_X, d_y, B, cw, norm, d_grad, d_loss, AdamArgs{}, A, s, err);
 }
 
 }  // namespace frg

@@ -18,11 +18,12 @@ int mlp_features(int dim, int p, const double* u, const uint64_t* keys, int64_t 
 void mlp_set_wait_cycles(long long cycles);
 int mlp_forward(const float* d_params, int in, const void* d_X, int64_t n, float* d_logits,
                 int8_t* d_flags, int* d_status, cudaStream_t s, Err* err);
-// cw[0..2] class weights (coarsen, keep, refine), cw[3] = 1 / (sum over the batch of w_label)
+// cw[0..2] class weights (coarsen, keep, refine); the loss's factor is cw[3] or, with norm, 1 / (sum over
+// the batch of w_label)
 int mlp_grad(const float* d_params, int in, const void* d_X, const int8_t* d_y, int64_t B,
-             const float* cw, float* d_grad, float* d_loss, Alloc& A, cudaStream_t s, Err* err);
+             const float* cw, bool norm, float* d_grad, float* d_loss, Alloc& A, cudaStream_t s, Err* err);
 int mlp_train_step(float* d_params, float* d_m, float* d_v, int64_t step, int in, const void* d_X,
-                   const int8_t* d_y, int64_t B, const float* cw, float lr, float* d_loss,
+                   const int8_t* d_y, int64_t B, const float* cw, bool norm, float lr, float* d_loss,
                    Alloc& A, cudaStream_t s, Err* err);
 
 }  // namespace frg

@@ -77,7 +77,7 @@ EXPORTS = ["fr_mesh_init", "fr_mesh_free", "fr_step", "fr_run", "fr_adapt", "fr_
            "fr_tree_conn", "fr_profile_enable", "fr_profile_read", "fr_kernel_launches",
            "fr_keys_sort_noalloc", "fr_tree_complete", "fr_mlp_param_count", "fr_features",
            "fr_set_learned_indicator", "fr_mlp_forward", "fr_mlp_grad", "fr_mlp_train_step",
-           "fr_mlp_forward_alloc", "fr_mlp_train_step_alloc", "fr_tree_complete_alloc", "fr_tree_balance_alloc",
+           "fr_mlp_forward_alloc", "fr_mlp_grad_alloc", "fr_mlp_train_step_alloc", "fr_tree_complete_alloc", "fr_tree_balance_alloc",
            "fr_tc_set_wait_limit"]
 NOALLOC_SORT_MAX_KEYS = 1 << 18
 
@@ -133,7 +133,7 @@ def load(build_if_missing: bool = True):
     lib.fr_mlp_grad.argtypes = [C.c_int, vp, vp, vp, i64, vp, vp, vp, vp]
     lib.fr_mlp_train_step.argtypes = [C.c_int, vp, vp, vp, i64, vp, vp, i64, vp, C.c_float, vp, vp]
     al = C.POINTER(FRAllocator)
-    for name in ("fr_mlp_forward", "fr_mlp_train_step", "fr_tree_complete", "fr_tree_balance"):
+    for name in ("fr_mlp_forward", "fr_mlp_grad", "fr_mlp_train_step", "fr_tree_complete", "fr_tree_balance"):
         getattr(lib, name + "_alloc").argtypes = getattr(lib, name).argtypes + [al]
     lib.fr_profile_enable.argtypes = [vp, C.c_int]
     lib.fr_profile_read.argtypes = [vp, C.POINTER(FRProfile)]
@@ -405,7 +405,8 @@ def mlp_param_count(in_dim: int) -> int:
 
 
 def _class_w(cw):
-    """The C ABI's class_w: three weights, and 0 for the library to normalise by the batch's labels."""
+    """The class_w of the C ABI's _alloc forms: three weights, and 0 for the library to normalise by the
+    batch's labels."""
     cw = np.asarray(cw, dtype=np.float64)
     return np.array([cw[0], cw[1], cw[2], 0.0], dtype=np.float32)
 
@@ -417,8 +418,8 @@ def mlp_forward(params, X, stream=None):
     logits = torch.empty((n, 3), dtype=torch.float32, device="cuda")
     flags = torch.empty(n, dtype=torch.int8, device="cuda")
     _check(load().fr_mlp_forward_alloc(n_in, C.c_void_p(params.data_ptr()), C.c_void_p(X.data_ptr()), n,
-                                 C.c_void_p(logits.data_ptr()), C.c_void_p(flags.data_ptr()),
-                                 _stream_handle(stream), _call_alloc()))
+                                       C.c_void_p(logits.data_ptr()), C.c_void_p(flags.data_ptr()),
+                                       _stream_handle(stream), _call_alloc()))
     return logits, flags
 
 
@@ -433,9 +434,9 @@ def mlp_grad(params, X, y, class_w, stream=None):
     g = torch.empty_like(params)
     loss = torch.empty(1, dtype=torch.float32, device="cuda")
     cw = _class_w(class_w)
-    _check(load().fr_mlp_grad(n_in, C.c_void_p(params.data_ptr()), C.c_void_p(X.data_ptr()),
-                              C.c_void_p(y.data_ptr()), n, _np_ptr(cw), C.c_void_p(g.data_ptr()),
-                              C.c_void_p(loss.data_ptr()), _stream_handle(stream)))
+    _check(load().fr_mlp_grad_alloc(n_in, C.c_void_p(params.data_ptr()), C.c_void_p(X.data_ptr()),
+                                    C.c_void_p(y.data_ptr()), n, _np_ptr(cw), C.c_void_p(g.data_ptr()),
+                                    C.c_void_p(loss.data_ptr()), _stream_handle(stream), _call_alloc()))
     return float(loss.item()), g
 
 
