@@ -477,24 +477,24 @@ __global__ void k_bal_gen_fast(const uint64_t* __restrict__ k, int64_t* __restri
   __shared__ uint64_t s_tab[KEY_INDEX_MAX];
   constexpr int LPL = BalLanes<DIM>::value;
   constexpr int NC = 1 << DIM;
-  __shared__ int s_list[TB], s_n;
+  __shared__ int s_list[TB], s_cnt[TB / 32];
   // The block's leaves, one per thread; those at depth D are listed in order and then taken by groups of
   // lanes.  Most leaves of most passes are not at depth D: with a group of lanes for every leaf the grid
-  // was eight (four) times as large and idle but for them.
+  // was eight (four) times as large and idle but for them.  The order decides which leaves share a warp,
+  // with it how many equal octants are left out and whether a pass fits its room: it is the leaves' own,
+  // so a tree takes the same path on every run.
   const int tid = int(threadIdx.x), lane = tid & 31;
   const int64_t i0 = int64_t(blockIdx.x) * TB;
   const int64_t n = ctl[CTL_OVER] == 0 ? min(ctl[sn], n_ub) : 0;
   const bool mine = i0 + tid < n && g.depth(k[i0 + tid]) == D;
-  if (tid == 0) s_n = 0;
+  const unsigned b = __ballot_sync(0xffffffffu, mine);
+  if (lane == 0) s_cnt[tid >> 5] = __popc(b);
   const int cnt = __syncthreads_count(mine);
   if (cnt == 0) return;
   const int m = stage_key_index(X, n, s_tab);  // ends with a barrier
   {
-    // ascending places inside a warp keep neighbouring leaves together (their lanes share ancestors)
-    const unsigned b = __ballot_sync(0xffffffffu, mine);
-    int at = 0;
-    if (lane == 0 && b) at = atomicAdd(&s_n, __popc(b));
-    at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & ((1u << lane) - 1u));
+    int at = __popc(b & ((1u << lane) - 1u));
+    for (int w = 0; w < tid >> 5; ++w) at += s_cnt[w];
     if (mine) s_list[at] = tid;
   }
   __syncthreads();
