@@ -761,11 +761,12 @@ KG geo_or_err(int dim, int Dmax, int* rc) {
 
 // Device memory of one call of a primitive: blocks released inside the call serve its later requests
 // (a depth pass of the balance asks for the sizes of the one before), and all of them go back to the
-// caller's allocator, or to the stream-ordered pool, when the call ends.
+// caller's allocator, or to the stream-ordered pool, when the call ends or an allocation fails (which is then
+// tried again, so that a call needs no more memory than without the cache).
 struct CallAlloc {
   BlockCache cache;
   Alloc A;
-  CallAlloc(const fr_allocator* user, cudaStream_t s, Err* err) : A{user, s, err, &cache} {}
+  CallAlloc(const fr_allocator* user, cudaStream_t s, Err* err) : A{user, s, err, &cache} { cache.give_back = true; }
   ~CallAlloc() {
     auto live = cache.live;  // none but after an error
     for (auto& b : live) A.put(b.first);

@@ -328,6 +328,7 @@ __device__ __forceinline__ void map_leaf(const uint64_t* __restrict__ old, int64
 struct BlockCache {
   std::vector<std::pair<void*, size_t>> free_blocks;
   std::vector<std::pair<void*, size_t>> live;  // block -> size of blocks handed out
+  bool give_back = false;  // return the free blocks, and try again, when an allocation fails
 };
 
 struct Alloc {

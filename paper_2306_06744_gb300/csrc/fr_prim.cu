@@ -72,6 +72,11 @@ void* Alloc::get(size_t bytes) {
     }
   }
   void* p = raw_get(user, stream, bytes);
+  if (!p && cache && cache->give_back && !cache->free_blocks.empty()) {
+    // short of memory: what the call has released goes back first
+    release_cache();
+    p = raw_get(user, stream, bytes);
+  }
   if (p && cache) cache->live.push_back({p, bytes});
   return p;
 }

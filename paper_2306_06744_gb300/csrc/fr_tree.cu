@@ -1421,12 +1421,14 @@ int tree_balance(int dim, const KG& g, int Dhigh, int Dlow, Buf<uint64_t>& keys,
     }
     Scratch S(&A);
     // one search pass: the octants are placed by an atomic counter (sorted next, so their order
-    // does not matter) into room for max(2^16, 2n) of them, up to 8n while that stays below 2^24 (128
-    // MB: the first pass of a tree completed from points asks for about 3n); a pass that generates
-    // more is counted, scanned and generated again at exact positions, which costs two more searches
-    int64_t capG = 2 * n_ub > (int64_t(1) << 16) ? 2 * n_ub : (int64_t(1) << 16);
-    if (capG < (int64_t(1) << 24)) capG = 8 * n_ub < (int64_t(1) << 24) ? std::max(capG, 8 * n_ub) : (int64_t(1) << 24);
-    if (gen.ensure(A, size_t(capG)) || cudaMemsetAsync(d_ctl + CTL_G, 0, 8, s) != cudaSuccess) {
+    // does not matter) into room for max(2^16, 2n) of them or, where that is more and can be had, min(8n,
+    // 2^24) (at most 128 MB).  The first pass of a tree completed from points asks for about 3n, which
+    // fits up to 5.6M leaves.  A pass that generates more is counted, scanned and generated again at
+    // exact positions, which costs two more searches
+    const int64_t least = std::max(2 * n_ub, int64_t(1) << 16);
+    int64_t capG = std::max(least, std::min(8 * n_ub, int64_t(1) << 24));
+    if ((gen.ensure(A, size_t(capG)) && (capG == least || gen.ensure(A, size_t(capG = least)))) ||
+        cudaMemsetAsync(d_ctl + CTL_G, 0, 8, s) != cudaSuccess) {
       rc = set_error(err, FR_ENOMEM, "balance scratch");
       break;
     }
