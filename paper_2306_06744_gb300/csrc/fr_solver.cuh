@@ -33,10 +33,14 @@ struct StageArgs {
 };
 
 // The element kernel of the FP32 and double-word forms fetches its common fluxes asynchronously.  Its
-// volume part needs none and overlaps the interface kernel's drain, which matters while the grid is about
-// one wave (up to 4 waves here); in a grid of many waves the blocks instead wait for the interface kernel
-// at their start and let the fetch run behind the volume part.
-constexpr int64_t STAGE_EARLY_BLOCKS = 152 * 8 * 4;
+// volume part needs none and overlaps the interface kernel's drain, which is worth more up to a few tens of
+// waves; in larger grids, whose fluxes come from DRAM, the blocks instead wait for the interface kernel at
+// their start and let the fetch run behind the volume part.  Step times, early against late fetch, uniform
+// meshes: 2k blocks 3D p = 1 FP32 61.2 / 57.4 us, 8k 2D p = 1 double-word 330 / 319, 3D p = 2 380 / 370, 16k
+// 3D p = 1 931 / 908, 3D p = 3 FP32 297.2 / 299.6, 33k 2D p = 3 832 / 827, 3D p = 4 FP32 615 / 619; 66k 3D
+// p = 2 FP32 1245 / 1286, double-word 2787 / 2807, 131k 3D p = 3 2146 / 2215 and 5825 / 5877, 2D p = 3 1751 /
+// 1763 and 3243 / 3252.
+constexpr int64_t STAGE_EARLY_BLOCKS = 152 * 8 * 40;
 enum { FETCH_EARLY = 1, FETCH_WIDE = 2 };  // wide: the common fluxes start on a 16-byte boundary
 inline int fetch_mode(int64_t blocks, const void* fcomm) {
   return (blocks >= STAGE_EARLY_BLOCKS ? FETCH_EARLY : 0) |
