@@ -101,7 +101,7 @@ __host__ __device__ __forceinline__ double fx_double(long long v, int e, bool ba
 // below are in units of 2^(Ev + Ew - 2102 - pk), below 2^62 and wrong by less than 7 units (one for each
 // operand cut at its last bit, and the rounding).
 constexpr int FX_PK = 2, FX_PK3 = 1;  // pk of the sum of squares and of fx_dot3
-constexpr int FX_P_MIN = 600;  // smallest exponent of an operand: units of products stay normal
+constexpr int FX_P_MIN = 542;  // smallest exponent of an operand (2^-481): the unit of half a square (fx_half_sq) is normal
 __host__ __device__ __forceinline__ long long fx_value(double x, int E) {
   const uint64_t b = fx_bits(x);
   const int e = int(b >> 52) & 0x7FF;
@@ -147,6 +147,11 @@ __host__ __device__ __forceinline__ long long fx_sum_sq(const int2* v) {
   }
   m += (long long)(l >> 32);
   return (h << FX_PK) + ((m + (1ll << (29 - FX_PK))) >> (30 - FX_PK));
+}
+// half of it as a double, from limbs of exponent E: halved in its unit
+template <int n>
+__host__ __device__ __forceinline__ double fx_half_sq(const int2* v, int E) {
+  return fx_double(fx_sum_sq<n>(v), fx_punit(E, E, FX_PK) - 1, fx_pbad(E, E));
 }
 
 // biased exponent of one unit of a result: values of group exponent E, entries scaled by 2^k

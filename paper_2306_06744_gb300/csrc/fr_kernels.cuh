@@ -220,16 +220,16 @@ __host__ __device__ __forceinline__ void rusanov2_fx(const double* qL, const dou
   const int E[FX_GROUPS] = {fx_pexp(max(fx_mag(qL[0]), fx_mag(qR[0]))), max(EL, ER),
                             fx_pexp(max(fx_mag(qL[NV - 1]), fx_mag(qR[NV - 1])))};
   int2 lL[NV], lR[NV];
-  double kL, kR;  // |m|^2 / 2, halved in its unit
+  double kL, kR;  // |m|^2 / 2
   {
     long long a[DIM], c[DIM];
     int2 s[DIM];
 #pragma unroll
     for (int b = 0; b < DIM; ++b) s[b] = fx_split(a[b] = fx_value(qL[1 + b], EL));
-    kL = fx_double(fx_sum_sq<DIM>(s), fx_punit(EL, EL, FX_PK) - 1, fx_pbad(EL, EL));
+    kL = fx_half_sq<DIM>(s, EL);
 #pragma unroll
     for (int b = 0; b < DIM; ++b) s[b] = fx_split(c[b] = fx_value(qR[1 + b], ER));
-    kR = fx_double(fx_sum_sq<DIM>(s), fx_punit(ER, ER, FX_PK) - 1, fx_pbad(ER, ER));
+    kR = fx_half_sq<DIM>(s, ER);
     const int sL = min(E[1] - EL, 63), sR = min(E[1] - ER, 63);
 #pragma unroll
     for (int b = 0; b < DIM; ++b) {

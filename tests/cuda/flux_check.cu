@@ -118,6 +118,16 @@ static void kinds() {
     worst = fmax(worst, ratio<DIM>(qL, qR, t % DIM));
   }
   line("plain");
+  // units in which all values are tiny or huge
+  for (int e : {-470, -440, 440}) {
+    worst = 0;
+    for (int t = 0; t < 5000; ++t) {
+      state<DIM>(std::ldexp(1.0, e), 0.1 + rnd(), qL);
+      state<DIM>(std::ldexp(1.0, e), 0.1 + rnd(), qR);
+      worst = fmax(worst, ratio<DIM>(qL, qR, t % DIM));
+    }
+    line(e == -470 ? "smallest" : (e < 0 ? "tiny" : "huge"));
+  }
   // one side 10 to 1e8 times as dense as the other at the same speeds and temperatures
   worst = 0;
   for (int t = 0; t < 20000; ++t) {

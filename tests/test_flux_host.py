@@ -1,7 +1,8 @@
 """The FP64 form's interface flux (rusanov2_fx) on the host against the same flux in long double, with the
-states that its integer products could get wrong: one side up to 1e8 times as dense, one side's pressure negative (its wave speed is not a
-number, and its speed may exceed the other side's wave speed), NaN of either sign and infinities
-(tests/cuda/flux_check.cu, which derives the bounds)."""
+states that its integer products could get wrong: units in which all values are tiny (from 2^-470) or huge, one
+side up to 1e8 times as dense, one side's pressure negative (its wave speed is not a number, and its speed may
+exceed the other side's wave speed), NaN of either sign and infinities (tests/cuda/flux_check.cu, which
+derives the bounds)."""
 import os
 import subprocess
 import tempfile
@@ -24,7 +25,7 @@ def results():
 
 
 @pytest.mark.parametrize("dim", [2, 3])
-@pytest.mark.parametrize("kind", ["plain", "jump", "negative_pressure"])
+@pytest.mark.parametrize("kind", ["plain", "smallest", "tiny", "huge", "jump", "negative_pressure"])
 def test_flux_within_its_bound(results, kind, dim):
     assert 0.0 < float(results["%s%d" % (kind, dim)]) <= 1.0, results
 

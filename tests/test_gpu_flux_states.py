@@ -97,6 +97,15 @@ def test_negative_pressure_on_one_side(dim, p):
     assert (np.abs(got - want) <= TOL * scale[:, :, None]).all()
 
 
+@pytest.mark.parametrize("e", [-470, -300, 440])
+@pytest.mark.parametrize("dim,p", [(2, 2), (3, 3)])
+def test_units_far_from_one(dim, p, e):
+    g, keys, cells = _mesh(dim, p, 2)
+    q = np.ldexp(_states(len(keys), dim, 8), e)
+    want, scale = _rhs(q, cells, p, 2)
+    assert (np.abs(_run(g, keys, q) - want) <= TOL * scale[:, :, None]).all()
+
+
 @pytest.mark.parametrize("jump", [1e2, 1e4, 1e6, 1e8])
 @pytest.mark.parametrize("dim,p", [(2, 1), (2, 3), (3, 2)])
 def test_density_jump_across_faces(dim, p, jump):
