@@ -333,10 +333,10 @@ def aggregate_ranks(units, seconds, device="cuda"):
 
 
 def _kernel_source_hash():
-    """Hash of the FP64 form's element kernel's source text (the k_stage_fx definition)."""
+    """Hash of the FP64 form's element kernel's source text (k_stage_fx and its bodies)."""
     import hashlib
     src = open(os.path.join(ROOT, "paper_2306_06744_gb300", "csrc", "fr_stage_fx.cuh")).read()
-    a = src.index("k_stage_fx(StageArgs")
+    a = src.index("struct StageMem")
     return hashlib.sha256(src[a:].encode()).hexdigest()[:16]
 
 

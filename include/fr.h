@@ -81,8 +81,18 @@ typedef struct {
                               (FP32 accumulation); 3 the same in split BF16 (bf16x3: hi*hi +
                               hi*lo + lo*hi, FP32 accumulation); 4 double-word (two-float, ~48-bit
                               significand) on the FP32 pipes, the Runge-Kutta combination in FP64.
-                              0 forms its linear operators and flux products in fixed point of at
-                              least 58 bits on the integer pipes.  2 and 3 are built for dim 3, p 3
+                              0 forms its linear operators and flux products in fixed point on the
+                              integer pipes: operands are cut at 2^-59 of the largest magnitude of
+                              their group (density, momenta, energy) in the element (flux products:
+                              of the two sides of the face point), sums rounded at 2^-58 of their
+                              range; elements whose density or energy spans more than 5 binary
+                              exponents are formed in FP64.  The residual has plain FP64's error
+                              (measured with jumps of 1e8 inside and between elements, and with one
+                              momentum 2^-40 of the others; that one's own traces and face fluxes
+                              hold 58 - k bits, k binary places below the largest momentum).  An
+                              infinity, a NaN or a magnitude above 2^1017 (momenta above 2^509 on a
+                              face) makes its group's results of the whole element (face point) NaN;
+                              momenta and speeds below 2^-481 lose bits on faces.  2 and 3 are built for dim 3, p 3
                               (64-point hexahedra, Sec. 2.1's operator as 16 x 16 Kronecker blocks);
                               other dim/p return FR_EINVAL.  A tensor-core completion wait that
                               gives up is reported as FR_ETIMEOUT by the next fr_adapt/fr_run

@@ -3,9 +3,13 @@
 // GB300 issues 2 FP64 multiply-adds per clock and SM against 128 32-bit operations, so the FP64
 // pipe bounds the element kernel while the integer pipes idle.  The linear parts of the method (the
 // folded derivative, the correction terms, the traces) are contractions with a fixed small matrix;
-// they are computed here on integers, exactly up to one rounding of the operands at 2^-59 of the
-// element's largest value in the variable group and one of the sum at 2^-58 of the largest
-// possible sum, against 2^-53 per operation of a chain of FP64 multiply-adds.
+// they are computed here on integers, exactly up to the operands, cut at 2^-59 of the element's
+// largest value in the variable group, and one rounding of the sum at 2^-58 of the largest possible
+// sum, against 2^-53 of its terms per operation of a chain of FP64 multiply-adds.  So terms k > 5 binary
+// places below the group's largest value have fewer bits than in FP64: elements that span so much in density
+// or energy are left to FP64 (fx_low).  A single small momentum is not: its residual holds the pressure, which
+// rounds at the larger unit in FP64 as well (one momentum 2^-20 of the others, relative error of its residual
+// at 3D p = 3: 6.9e-15 in FP64, 6.1e-15 so).
 //
 // A value x of an element is the 60-bit integer v = trunc(x 2^(1081 - E)), E the biased exponent of
 // the largest magnitude of its group (density, momenta, energy) in the element, so |v| < 2^59.
@@ -29,6 +33,7 @@ constexpr int FX_GROUPS = 3;      // density, momenta, energy: one exponent each
 constexpr int FX_E_MIN = 64;      // smallest group exponent: results never fall below the normal range
 constexpr int FX_E_BAD = 2040;    // groups with infinities, NaN or values above 2^1017: results are NaN
 constexpr int FX_SUM_BITS = 61;   // log2 of the bound on the sum of |C|
+constexpr int FX_SPREAD = 5;      // exponents that a group may span with no fewer bits than FP64
 
 struct FxAcc {
   long long h, m;
@@ -172,57 +177,72 @@ inline int fx_scale(double sum) {
   return k < 67 ? k : 67;
 }
 
-// Largest magnitude (high words) per group over the N threads of one element, thread i of it, into
-// s[3] of the element (biased exponents; zeroed before a barrier by the caller, read after one).
-// All threads of the block call it; those without a point bring zeros and act = false.  With N a power
-// of two up to 16 an element lies in one warp and the values are stored, not accumulated.
-template <int N>
-__device__ __forceinline__ void fx_group_max(uint32_t w0, uint32_t w1, uint32_t w2, int i, bool act, uint32_t* s) {
+// Largest of each of K exponents over the N threads of one element, thread i of it, into s[K] of the
+// element (zeroed before a barrier by the caller, read after one).  All threads of the block call it;
+// those without a point bring zeros and act = false.  With N a power of two up to 16 an element lies in one
+// warp and the values are stored, not accumulated.
+template <int N, int K>
+__device__ __forceinline__ void fx_group_max(const uint32_t (&w)[K], int i, bool act, uint32_t* s) {
   const int lane = threadIdx.x & 31;
   if constexpr (N % 32 == 0) {
     // whole warps belong to one element
-    w0 = __reduce_max_sync(~0u, w0);
-    w1 = __reduce_max_sync(~0u, w1);
-    w2 = __reduce_max_sync(~0u, w2);
-    if (act && lane == 0) {
-      atomicMax(&s[0], w0 >> 20);
-      atomicMax(&s[1], w1 >> 20);
-      atomicMax(&s[2], w2 >> 20);
-    }
-  } else if constexpr (32 % N == 0) {
-    // whole elements in a warp: one value per element, no atomics
-    uint32_t p = (w0 >> 20) | ((w1 >> 20) << 16), q = w2 >> 20;
 #pragma unroll
-    for (int o = 1; o < N; o <<= 1) {
-      p = __vmaxu2(p, __shfl_xor_sync(~0u, p, o));
-      q = max(q, __shfl_xor_sync(~0u, q, o));
-    }
-    if (act && i == 0) {
-      s[0] = p & 0xFFFFu;
-      s[1] = p >> 16;
-      s[2] = q;
+    for (int k = 0; k < K; ++k) {
+      const uint32_t m = __reduce_max_sync(~0u, w[k]);
+      if (act && lane == 0) atomicMax(&s[k], m);
     }
   } else {
-    // segments of N lanes that may cross warps: each segment's first lane in a warp collects it;
-    // two groups to a register, exponents only
-    uint32_t p = (w0 >> 20) | ((w1 >> 20) << 16), q = w2 >> 20;
+    constexpr int P = (K + 1) / 2;  // two to a register
+    uint32_t p[P];
 #pragma unroll
-    for (int o = 1; o < 32 && o < N; o <<= 1) {
-      const uint32_t po = __shfl_down_sync(~0u, p, o), qo = __shfl_down_sync(~0u, q, o);
-      if (i + o < N && lane + o < 32) {
-        p = __vmaxu2(p, po);
-        q = q > qo ? q : qo;
+    for (int k = 0; k < P; ++k) p[k] = 2 * k + 1 < K ? w[2 * k] | (w[2 * k + 1] << 16) : w[2 * k];
+    if constexpr (32 % N == 0) {
+      // whole elements in a warp: one value per element, no atomics
+#pragma unroll
+      for (int o = 1; o < N; o <<= 1)
+#pragma unroll
+        for (int k = 0; k < P; ++k) p[k] = __vmaxu2(p[k], __shfl_xor_sync(~0u, p[k], o));
+      if (act && i == 0) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) s[k] = k & 1 ? p[k / 2] >> 16 : p[k / 2] & 0xFFFFu;
       }
-    }
-    if (act && (i == 0 || lane == 0)) {
-      atomicMax(&s[0], p & 0xFFFFu);
-      atomicMax(&s[1], p >> 16);
-      atomicMax(&s[2], q);
+    } else {
+      // segments of N lanes that may cross warps: each segment's first lane in a warp collects it
+#pragma unroll
+      for (int o = 1; o < 32 && o < N; o <<= 1) {
+        const bool in = i + o < N && lane + o < 32;
+#pragma unroll
+        for (int k = 0; k < P; ++k) {
+          const uint32_t q = __shfl_down_sync(~0u, p[k], o);
+          if (in) p[k] = __vmaxu2(p[k], q);
+        }
+      }
+      if (act && (i == 0 || lane == 0)) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) atomicMax(&s[k], k & 1 ? p[k / 2] >> 16 : p[k / 2] & 0xFFFFu);
+      }
     }
   }
 }
 // the group of variable v of nv: 0 density, 1 momenta, 2 energy
 __host__ __device__ constexpr int fx_group(int v, int nv) { return v == 0 ? 0 : (v == nv - 1 ? 2 : 1); }
+// exponents of a point of state q: the largest of each group
+template <int NV>
+__device__ __forceinline__ void fx_state_exps(const double* q, uint32_t (&w)[FX_GROUPS]) {
+  uint32_t m = fx_mag(q[1]);
+#pragma unroll
+  for (int v = 2; v < NV - 1; ++v) m = max(m, fx_mag(q[v]));
+  w[0] = fx_mag(q[0]) >> 20;
+  w[1] = m >> 20;
+  w[2] = fx_mag(q[NV - 1]) >> 20;
+}
+// a point with exponent e too low for its element's largest, emax, to leave it FP64's bits
+__device__ __forceinline__ bool fx_low(uint32_t e, uint32_t emax) { return e + FX_SPREAD < emax; }
+// the same for a state with exponents w whose element has the largest ones s: by density and energy (a
+// single small momentum, or the stagnation of all three, is no reason)
+__device__ __forceinline__ bool fx_low_state(const uint32_t (&w)[FX_GROUPS], const uint32_t* s) {
+  return fx_low(w[0], s[0]) || fx_low(w[2], s[2]);
+}
 __device__ __forceinline__ int fx_exp(uint32_t e) { return int(e) < FX_E_MIN ? FX_E_MIN : int(e); }
 
 }  // namespace frg

@@ -382,29 +382,33 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_transfer(KG g, const uint64
     // FP64 form: the traces of this block's refined and fused elements in fixed point, bitwise those
     // of the element and trace kernels (the last round ended with a barrier, sb is free)
     __shared__ uint32_t se[EPB * FX_GROUPS];
+    __shared__ int8_t s_wide[EPB];
+    __shared__ int s_low;
     __shared__ int2 slm[NP], slp[NP];
     for (int k = threadIdx.x; k < EPB * FX_GROUPS; k += blockDim.x) se[k] = 0u;
+    if (threadIdx.x < EPB) s_wide[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_low = 0;
     if (threadIdx.x < NP) {
       slm[threadIdx.x] = tfx.lm[threadIdx.x];
       slp[threadIdx.x] = tfx.lp[threadIdx.x];
     }
     __syncthreads();
     uint32_t w[FX_GROUPS] = {0u, 0u, 0u};
-    if (work) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) w[fx_group(v, NV)] = max(w[fx_group(v, NV)], fx_mag(acc[v]));
-    }
-    fx_group_max<N>(w[0], w[1], w[2], i, act, se + (act ? le : 0) * FX_GROUPS);
+    if (work) fx_state_exps<NV>(acc, w);
+    fx_group_max<N>(w, i, act, se + (act ? le : 0) * FX_GROUPS);
     __syncthreads();
     int2* sv = reinterpret_cast<int2*>(&sb[0][0]);
     if (work) {
+      if (fx_low_state(w, se + le * FX_GROUPS)) s_wide[le] = s_low = 1;
 #pragma unroll
       for (int v = 0; v < NV; ++v)
         sv[le * EU + v * N + fx_place<DIM, NP>(i)] = fx_limbs(acc[v], fx_exp(se[le * FX_GROUPS + fx_group(v, NV)]));
     }
     __syncthreads();
     const int ne = int((Mn - j0) < EPB ? (Mn - j0) : EPB);
-    fx_traces<DIM, NP>(sv, se, slm, slp, tfx.kt, ne, s_tag, static_cast<double*>(tc.dst) + j0 * S::EF);
+    double* to = static_cast<double*>(tc.dst) + j0 * S::EF;
+    fx_traces<DIM, NP>(sv, se, slm, slp, tfx.kt, ne, s_tag, to);
+    if (s_low) wide_traces<DIM, NP>(un + j0 * EU, tfx, ne, s_wide, s_tag, to);
   } else if (tc.dst && rounds > 0) {
     // the same in the other forms' trace types: FP64 sums in the trace kernel's order, from the new
     // state staged in shared memory, one thread per (element, face, face point), all variables
