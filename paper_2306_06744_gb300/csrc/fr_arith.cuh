@@ -135,16 +135,10 @@ __device__ __forceinline__ double ff_to_double(ff a) {
   return f_to_double_bits(a.h) + f_to_double_bits(a.l);  // one FP64 add
 }
 
-// ---- uniform interface over the three types ----
+// ---- conversions to and from the arithmetic types of the FP32 and double-word forms ----
 template <class T>
 struct Ar;
 
-template <>
-struct Ar<double> {
-  static __device__ __forceinline__ double from_d(double x) { return x; }
-  static __device__ __forceinline__ double to_d(double x) { return x; }
-  static __device__ __forceinline__ double c(double x) { return x; }
-};
 // double -> float by integer manipulation of the bit pattern (no FP64-rate conversion): the
 // significand is cut to 24 bits and rounded half away from zero (a carry moves into the exponent);
 // magnitudes below 2^-126 become a signed zero, above the float range infinity, NaN stays NaN.

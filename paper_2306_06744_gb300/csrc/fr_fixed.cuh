@@ -106,7 +106,7 @@ __host__ __device__ __forceinline__ double fx_double(long long v, int e, bool ba
 // below are in units of 2^(Ev + Ew - 2102 - pk), below 2^62 and wrong by less than 7 units (one for each
 // operand cut at its last bit, and the rounding).
 constexpr int FX_PK = 2, FX_PK3 = 1;  // pk of the sum of squares and of fx_dot3
-constexpr int FX_P_MIN = 542;  // smallest exponent of an operand (2^-481): the unit of half a square (fx_half_sq) is normal
+constexpr int FX_P_MIN = 542;  // smallest exponent of an operand (2^-481): fx_half_sq's unit is normal
 __host__ __device__ __forceinline__ long long fx_value(double x, int E) {
   const uint64_t b = fx_bits(x);
   const int e = int(b >> 52) & 0x7FF;

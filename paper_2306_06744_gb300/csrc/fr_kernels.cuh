@@ -259,7 +259,8 @@ __host__ __device__ __forceinline__ void rusanov2_fx(const double* qL, const dou
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     const int Ev = E[fx_group(v, NV)];
-    F2[v] = fx_double(fx_dot3(lL[v], cL, lR[v], cR, fx_diff(lL[v], lR[v]), cl), fx_punit(Ev, Ea, FX_PK3), fx_pbad(Ev, Ea));
+    F2[v] = fx_double(fx_dot3(lL[v], cL, lR[v], cR, fx_diff(lL[v], lR[v]), cl), fx_punit(Ev, Ea, FX_PK3),
+                      fx_pbad(Ev, Ea));
   }
   const double pp = pL + pR;
   double fn = F2[1];
@@ -361,7 +362,8 @@ struct FaceCfg {
 // leaves, blocks of 512 threads), 69 -> 66 at p = 1; in 2D the compiler's own 72 registers are better.
 template <int DIM, int NP, class T>
 __global__ void __launch_bounds__(FaceCfg<DIM, NP, T>::T,
-                                  DIM == 3 && std::is_same<T, double>::value ? 1024 / FaceCfg<DIM, NP, T>::T : 0) k_faces_t(FaceArgs A, const __grid_constant__ OpsT<T> ops) {
+                                  DIM == 3 && std::is_same<T, double>::value ? 1024 / FaceCfg<DIM, NP, T>::T : 0)
+    k_faces_t(FaceArgs A, const __grid_constant__ OpsT<T> ops) {
   using S = Sz<DIM, NP>;
   constexpr int NV = S::NV, NF = S::NF, NFC = S::NFC, NSUB = S::NSUB;
   constexpr int PER = FaceCfg<DIM, NP, T>::PER, BT = FaceCfg<DIM, NP, T>::T;
@@ -519,7 +521,8 @@ struct StageMinBlocks {
 // FP64 and the asynchronous fetch give, per launch at 3D p = 3 with 127k leaves, FP32 374 -> 274 us and
 // double-word 959 -> 806 us (2D p = 3, 11k leaves: 12.6 -> 11.9 and 20.5 -> 18.6 us).
 template <int DIM, int NP, class T>
-__global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value) k_stage_t(StageArgs A, const __grid_constant__ OpsT<T> ops) {
+__global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value)
+    k_stage_t(StageArgs A, const __grid_constant__ OpsT<T> ops) {
   using S = Sz<DIM, NP>;
   constexpr int N = S::N, NV = S::NV, NF = S::NF, EU = S::EU, EF = S::EF;
   constexpr int EPB = S::EPB;
@@ -709,12 +712,6 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageMinBlocks<T>::value) k_s
       return set_error(err, FR_EINVAL, "dim out of range");        \
     }                                                                \
   } while (0)
-
-inline int ipow_k(int b, int e) {
-  int r = 1;
-  while (e-- > 0) r *= b;
-  return r;
-}
 
 template <class T>
 int launch_traces_impl(int dim, int p, const double* u, int64_t M, const DevOps& o, void* tr,

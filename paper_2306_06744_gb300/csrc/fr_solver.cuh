@@ -85,8 +85,8 @@ int launch_indicator(int dim, int p, int mode, double th_r, double th_c, double 
                      cudaStream_t s, Err* err);
 // Traces carried over by the transfer (all null: none): an unchanged element's `bytes` of traces
 // are copied from src (old elements) to dst (new elements); a refined or fused element's traces
-// are computed from its new state (FP64 sums in the trace kernel's order) and stored in the
-// arithmetic type `kind` of the traces (0 FP64, 1 FP32, 2 double-word).
+// are computed from its new state and stored in the arithmetic type `kind` of the traces: 0 FP64 (by the
+// element kernel's own function), 1 FP32, 2 double-word (FP64 sums in the trace kernel's order).
 struct TraceCopy {
   const void* src;
   void* dst;
