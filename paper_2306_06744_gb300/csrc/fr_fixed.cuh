@@ -168,6 +168,10 @@ inline int2 fx_coef(double c, int k) {
   const long long h = (C + (1ll << 30)) >> 31;
   return make_int2(int(h), int(C - (h << 31)));
 }
+// ... and back, rounded to FP64 (k <= 67)
+__device__ __forceinline__ double fx_coef_value(int2 c, int k) {
+  return fma(double(c.x), 2147483648.0, double(c.y)) * __hiloint2double((1023 - k) << 20, 0);
+}
 // largest k with sum 2^k <= 2^FX_SUM_BITS; at most 67, so that the smallest group exponent leaves a
 // unit (fx_unit) in the normal range
 inline int fx_scale(double sum) {

@@ -19,8 +19,8 @@
 
 #include "fr_arith.cuh"
 #include "fr_internal.cuh"
-#include "fr_mlp.cuh"
 #include "fr_kernels.cuh"
+#include "fr_mlp.cuh"
 #include "fr_tc.cuh"
 
 namespace frg {

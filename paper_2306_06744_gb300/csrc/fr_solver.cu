@@ -384,6 +384,7 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_transfer(KG g, const uint64
     __shared__ uint32_t se[EPB * FX_GROUPS];
     __shared__ int8_t s_wide[EPB];
     __shared__ int s_low;
+    __shared__ double sl[2 * NP];
     __shared__ int2 slm[NP], slp[NP];
     for (int k = threadIdx.x; k < EPB * FX_GROUPS; k += blockDim.x) se[k] = 0u;
     if (threadIdx.x < EPB) s_wide[threadIdx.x] = 0;
@@ -408,7 +409,7 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_transfer(KG g, const uint64
     const int ne = int((Mn - j0) < EPB ? (Mn - j0) : EPB);
     double* to = static_cast<double*>(tc.dst) + j0 * S::EF;
     fx_traces<DIM, NP>(sv, se, slm, slp, tfx.kt, ne, s_tag, to);
-    if (s_low) wide_traces<DIM, NP>(un + j0 * EU, tfx, ne, s_wide, s_tag, to);
+    if (s_low) wide_traces<DIM, NP>(un + j0 * EU, slm, slp, tfx.kt, sl, ne, s_wide, s_tag, to);
   } else if (tc.dst && rounds > 0) {
     // the same in the other forms' trace types: FP64 sums in the trace kernel's order, from the new
     // state staged in shared memory, one thread per (element, face, face point), all variables

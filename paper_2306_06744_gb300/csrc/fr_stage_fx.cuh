@@ -11,15 +11,13 @@ namespace frg {
 // memory by the kernels because threads of a warp read different rows)
 struct TraceFx {
   int2 lm[NPMAX], lp[NPMAX];
-  int kt;                       // scale of the entries
-  double l[2][NPMAX];           // the same in FP64: l(-1), l(+1)
+  int kt;  // scale of the entries
 };
 struct OpsFx {
   int2 Dt[NPMAX][NPMAX], gLh[NPMAX], gRh[NPMAX];
   int kd;                    // scale of the derivative and its correction
   TraceFx tr;
   double D[NPMAX][NPMAX];    // plain derivative (density-gradient indicator, FP64)
-  double fDt[NPMAX][NPMAX], fgLh[NPMAX], fgRh[NPMAX];  // Dt, gLh, gRh in FP64 (elements of wide range)
   double gm1, ngmh;          // gamma - 1, -(gamma - 1)/2
 };
 inline TraceFx make_trace_fx(int p, const DevOps& o) {
@@ -33,8 +31,6 @@ inline TraceFx make_trace_fx(int p, const DevOps& o) {
   for (int i = 0; i <= p; ++i) {
     r.lm[i] = fx_coef(o.lm[i], r.kt);
     r.lp[i] = fx_coef(o.lp[i], r.kt);
-    r.l[0][i] = o.lm[i];
-    r.l[1][i] = o.lp[i];
   }
   return r;
 }
@@ -56,10 +52,7 @@ inline OpsFx make_ops_fx(int dim, int p, const DevOps& o, double gamma) {
     for (int j = 0; j < n; ++j) {
       r.Dt[i][j] = fx_coef(o.Dt[i][j], r.kd);
       r.D[i][j] = o.D[i][j];
-      r.fDt[i][j] = o.Dt[i][j];
     }
-    r.fgLh[i] = 0.5 * o.gL[i];
-    r.fgRh[i] = 0.5 * o.gR[i];
   }
   r.gm1 = gamma - 1.0;
   r.ngmh = -0.5 * (gamma - 1.0);
@@ -109,19 +102,23 @@ __device__ __forceinline__ void fx_traces(const int2* sv, const uint32_t* se, co
 // chains from the state u in memory, each by the thread that wrote the first one.  With one exponent per
 // group and element the thin side of a jump r inside an element has traces off by 2^-59 r of themselves; the
 // wave speeds formed from them carried that into the whole residual (1e-13 of it at r = 1e5, 1e-10 at 1e8,
-// now 5e-16).  Rare, so not inlined.
+// now 5e-16).  Rare, so not inlined, and with the operator's entries from the fixed-point ones, into sl[2 NP]
+// (tables of their own among the kernel's parameters cost every launch 0.3 us).  All threads of the block.
 template <int DIM, int NP>
-__device__ __noinline__ void wide_traces(const double* u, const TraceFx& ops, int ne, const int8_t* wide,
-                                         const int8_t* need, double* to) {
+__device__ __noinline__ void wide_traces(const double* u, const int2* slm, const int2* slp, int kt, double* sl,
+                                         int ne, const int8_t* wide, const int8_t* need, double* to) {
   using S = Sz<DIM, NP>;
   constexpr int N = S::N, NV = S::NV, NF = S::NF, EU = S::EU, EF = S::EF, FQ = S::NFC * NF;
+  if (threadIdx.x < 2 * NP) sl[threadIdx.x] = fx_coef_value(threadIdx.x < NP ? slm[threadIdx.x] : slp[threadIdx.x - NP], kt);
+  __syncthreads();
   for (int k = threadIdx.x; k < ne * FQ; k += blockDim.x) {
     const int le = k / FQ, r = k % FQ, f = r / NF, q = r % NF;
     if (!wide[le] || (need && !need[le])) continue;
+    const double* l = sl + (f & 1) * NP;
     for (int v = 0; v < NV; ++v) {
       double t = 0.0;
 #pragma unroll
-      for (int j = 0; j < NP; ++j) t = fma(ops.l[f & 1][j], u[le * EU + v * N + line_pt<DIM, NP>(f >> 1, q, j)], t);
+      for (int j = 0; j < NP; ++j) t = fma(l[j], u[le * EU + v * N + line_pt<DIM, NP>(f >> 1, q, j)], t);
       to[int64_t(le) * EF + (f * NV + v) * NF + q] = t;
     }
   }
@@ -143,6 +140,7 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_traces_fx(const double* __r
   __shared__ uint32_t se[EPB * FX_GROUPS];
   __shared__ int8_t need[EPB], wide[EPB];
   __shared__ int low;
+  __shared__ double sl[2 * NP];
   const int tid = threadIdx.x;
   if (d_M && *d_M < M) M = *d_M;  // the element count on the device (M is then a bound of it)
   const int64_t e0 = int64_t(blockIdx.x) * EPB;
@@ -176,7 +174,7 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT) k_traces_fx(const double* __r
   }
   __syncthreads();
   fx_traces<DIM, NP>(sv, se, slm, slp, ops.kt, ne, need, tr + e0 * S::EF);
-  if (low) wide_traces<DIM, NP>(u + e0 * EU, ops, ne, wide, need, tr + e0 * S::EF);
+  if (low) wide_traces<DIM, NP>(u + e0 * EU, slm, slp, ops.kt, sl, ne, wide, need, tr + e0 * S::EF);
 }
 
 // planes of the element's fluxes: the axes' mass fluxes, the distinct entries of the symmetric
@@ -224,8 +222,8 @@ struct StageOcc {
 // Elements of wide range (fx_low) take FP64 chains.  A point that is too low sets a flag of its block before a
 // barrier that the block has anyway, and the block leaves for a body of its own that is not inlined.  Per
 // launch at 3D p = 3 with 242k leaves: 1595 us without the test, 1703 with branches inside or with a vote by
-// the barrier (__syncthreads_or), 1611 so (3D p = 2, 184k: 603, 620 and 610 us).  Blocks that do leave take about
-// three times as long, 17 to 31% longer than when the whole form was FP64.
+// the barrier (__syncthreads_or), 1596 so (3D p = 2, 184k: 603, 620 and 612 us).  Blocks that do leave take about
+// three times as long, 20 to 32% longer than when the whole form was FP64.
 template <int DIM, int NP>
 struct StageMem {
   using S = Sz<DIM, NP>;
@@ -237,6 +235,7 @@ struct StageMem {
   uint32_t rho0[EPB];           // exponent of the first point's density
   int low[2];                   // a point too low for its element's exponents: old state, new state
   int8_t wide[EPB];             // elements of wide range (mixed body)
+  double f64[NP * NP + 2 * NP];  // their operators' entries: D, gL, gR; then l(-1), l(+1)
   double h2[EPB];               // per element: c * (-2/h)
   unsigned long long g2[EPB];   // per element: the indicator's max |D rho|^2 (as bits)
 };
@@ -261,7 +260,8 @@ __device__ __noinline__ void stage_traces_wide(const StageArgs& A, const OpsFx& 
     if (fx_low_state(w, m.eo + le * FX_GROUPS)) m.wide[le] = 1;
   }
   __syncthreads();
-  wide_traces<DIM, NP>(u, ops.tr, ne, m.wide, nullptr, static_cast<double*>(A.trace_out) + e0 * S::EF);
+  wide_traces<DIM, NP>(u, m.lm, m.lp, ops.tr.kt, m.f64, ne, m.wide, nullptr,
+                       static_cast<double*>(A.trace_out) + e0 * S::EF);
 }
 
 // The element stage from the derivative on (fluxes staged, exponents known)
@@ -296,8 +296,9 @@ __device__ __forceinline__ void stage_rest(const StageArgs& A, const OpsFx& ops,
 #pragma unroll
       for (int j = 0; j < NP; ++j) {
         const double* f = reinterpret_cast<const double*>(m.fl) + le * NPL * N + line_pt<DIM, NP>(a, qf, j);
+        const double d = m.f64[ia * NP + j];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) vol[v] = fma(ops.fDt[ia][j], f[FP::of(a, v) * N], vol[v]);
+        for (int v = 0; v < NV; ++v) vol[v] = fma(d, f[FP::of(a, v) * N], vol[v]);
       }
     }
   } else {
@@ -390,10 +391,10 @@ __device__ __forceinline__ void stage_rest(const StageArgs& A, const OpsFx& ops,
         fx_mac(acc[v], Fm[(NV + v) * NF], cr);
       }
       if (MIXED && wide) {
+        const double dl = m.f64[NP * NP + ia], dr = m.f64[NP * NP + NP + ia];
 #pragma unroll
         for (int v = 0; v < NV; ++v)
-          vol[v] = fma(ops.fgLh[ia], F[(2 * a * NV + v) * NF + qf],
-                       fma(ops.fgRh[ia], F[((2 * a + 1) * NV + v) * NF + qf], vol[v]));
+          vol[v] = fma(dl, F[(2 * a * NV + v) * NF + qf], fma(dr, F[((2 * a + 1) * NV + v) * NF + qf], vol[v]));
       }
     }
     const double cs = m.h2[le < ne ? le : 0];
@@ -502,6 +503,9 @@ __device__ __noinline__ void stage_rest_mixed(const StageArgs& A, const OpsFx& o
   const int64_t e0 = int64_t(blockIdx.x) * EPB;
   const int ne = int((A.M - e0) < EPB ? (A.M - e0) : EPB);
   if (tid < EPB) m.wide[tid] = 0;
+  if (tid < NP * NP + 2 * NP)
+    m.f64[tid] = fx_coef_value(
+        tid < NP * NP ? m.D[tid] : (tid < NP * NP + NP ? m.gL[tid - NP * NP] : m.gR[tid - NP * NP - NP]), ops.kd);
   __syncthreads();
   double fl[NPL];
   if (le < ne) {
@@ -565,8 +569,6 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageOcc<DIM, NP>::value)
     m.lm[tid] = ops.tr.lm[tid];
     m.lp[tid] = ops.tr.lp[tid];
   }
-  const uint32_t e_rho = fx_mag(q[0]) >> 20;
-  if (own && i == 0) m.rho0[le] = e_rho;
   __syncthreads();
   int E[FX_GROUPS];
   {
@@ -577,6 +579,8 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageOcc<DIM, NP>::value)
     flux_exps<DIM>(fl, w);
     if (!own) w[0] = w[1] = w[2] = 0u;
     fx_group_max<N>(w, i, own, m.ef + le * FX_GROUPS);
+    const uint32_t e_rho = fx_mag(q[0]) >> 20;
+    if (own && i == 0) m.rho0[le] = e_rho;
     __syncthreads();
     const uint32_t* se = m.ef + le * FX_GROUPS;
     const uint32_t e[FX_GROUPS] = {se[0], se[1], se[2]}, rho0 = m.rho0[le];
