@@ -3,8 +3,8 @@
 // projection at 2:1 hanging faces, owner-computes back-projection without atomics), the element
 // stage (corrected-flux divergence folded with the DG correction, SSP-RK3 combination, traces of
 // the new state), the adaptation indicator, solution transfer and deterministic norms.
-// All arithmetic is FP64, the transfer's traces in the fixed point of fr_fixed.cuh.  Kernels are instantiated per (dim, p+1) so every small contraction is
-// fully unrolled.
+// All arithmetic is FP64, the transfer's traces in the fixed point of fr_fixed.cuh.  Kernels are instantiated
+// per (dim, p+1) so every small contraction is fully unrolled.
 #include <cmath>
 
 #include "fr_internal.cuh"

@@ -109,7 +109,8 @@ __device__ __noinline__ void wide_traces(const double* u, const int2* slm, const
                                          int ne, const int8_t* wide, const int8_t* need, double* to) {
   using S = Sz<DIM, NP>;
   constexpr int N = S::N, NV = S::NV, NF = S::NF, EU = S::EU, EF = S::EF, FQ = S::NFC * NF;
-  if (threadIdx.x < 2 * NP) sl[threadIdx.x] = fx_coef_value(threadIdx.x < NP ? slm[threadIdx.x] : slp[threadIdx.x - NP], kt);
+  if (threadIdx.x < 2 * NP)
+    sl[threadIdx.x] = fx_coef_value(threadIdx.x < NP ? slm[threadIdx.x] : slp[threadIdx.x - NP], kt);
   __syncthreads();
   for (int k = threadIdx.x; k < ne * FQ; k += blockDim.x) {
     const int le = k / FQ, r = k % FQ, f = r / NF, q = r % NF;

@@ -253,9 +253,10 @@ __device__ __forceinline__ int64_t bal_nS(const int64_t* ctl, int64_t cap) {
   return (ctl[CTL_OVER] != 0 || G > cap) ? 0 : G;
 }
 
-// A group of lanes per leaf (4 in 2D, 8 in 3D), one lane per neighbour box looked up: the lanes search in parallel and combine by warp shuffles, so the scan that
-// places the generated octants runs over leaves, not over (leaf, neighbour) pairs.  Lanes past
-// the leaf count (an upper bound of it sizes the grid) contribute zeros.
+// A group of lanes per leaf (4 in 2D, 8 in 3D), one lane per neighbour box looked up: the lanes search in
+// parallel and combine by warp shuffles, so the scan that places the generated octants runs over leaves, not
+// over (leaf, neighbour) pairs.  Lanes past the leaf count (an upper bound of it sizes the grid) contribute
+// zeros.
 template <int DIM>
 struct BalLanes {
   static constexpr int value = 1 << DIM;
