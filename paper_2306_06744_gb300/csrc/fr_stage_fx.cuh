@@ -222,9 +222,9 @@ struct StageOcc {
 //
 // Elements of wide range (fx_low) take FP64 chains.  A point that is too low sets a flag of its block before a
 // barrier that the block has anyway, and the block leaves for a body of its own that is not inlined.  Per
-// launch at 3D p = 3 with 242k leaves: 1595 us without the test, 1703 with branches inside or with a vote by
-// the barrier (__syncthreads_or), 1596 so (3D p = 2, 184k: 603, 620 and 612 us).  Blocks that do leave take about
-// three times as long, 20 to 32% longer than when the whole form was FP64.
+// launch at 3D p = 3 with 242k leaves: 1597 us without the test, 1703 with branches inside or with a vote by
+// the barrier (__syncthreads_or), 1597 so (3D p = 2, 184k: 603, 620 and 603 us; 2D p = 3, 11k: 21.9 and 22.6 us).
+// Blocks that do leave take about three times as long, 20 to 32% longer than when the whole form was FP64.
 template <int DIM, int NP>
 struct StageMem {
   using S = Sz<DIM, NP>;
@@ -581,23 +581,28 @@ __global__ void __launch_bounds__(Sz<DIM, NP>::BT, StageOcc<DIM, NP>::value)
     if (!own) w[0] = w[1] = w[2] = 0u;
     fx_group_max<N>(w, i, own, m.ef + le * FX_GROUPS);
     const uint32_t e_rho = fx_mag(q[0]) >> 20;
+    // the element's first density: by a shuffle where elements lie in a warp (the mixed body reads it, too)
+    uint32_t rho0 = 32 % N == 0 ? __shfl_sync(~0u, e_rho, (tid & 31) / N * N) : 0u;
     if (own && i == 0) m.rho0[le] = e_rho;
     __syncthreads();
+    if (32 % N != 0) rho0 = m.rho0[le];
     const uint32_t* se = m.ef + le * FX_GROUPS;
-    const uint32_t e[FX_GROUPS] = {se[0], se[1], se[2]}, rho0 = m.rho0[le];
+    const uint32_t e[FX_GROUPS] = {se[0], se[1], se[2]};
+    const bool low = own && stage_low(w[1], e_rho, e, rho0);
 #pragma unroll
     for (int g = 0; g < FX_GROUPS; ++g) E[g] = fx_exp(e[g]);
     if (own) {
 #pragma unroll
       for (int k = 0; k < NPL; ++k) m.fl[(le * NPL + k) * N + i] = fx_limbs(fl[k], E[FP::group(k)]);
     }
-    if (own && stage_low(w[1], e_rho, e, rho0)) m.low[0] = 1;
+    if (low) m.low[0] = 1;
   }
   __syncthreads();
-  if (m.low[0])
-    stage_rest_mixed<DIM, NP>(A, ops, m);
-  else
+  if (!m.low[0]) {
     stage_rest<DIM, NP, false>(A, ops, m, E);
+    return;
+  }
+  stage_rest_mixed<DIM, NP>(A, ops, m);
 }
 
 }  // namespace frg
